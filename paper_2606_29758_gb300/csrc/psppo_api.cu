@@ -41,6 +41,8 @@ static int begin_call(void* ws, size_t ws_bytes, size_t need, cudaStream_t s) {
 }
 
 static uint32_t* status_word(void* ws) { return static_cast<uint32_t*>(ws); }
+// A second word of the header, zeroed with the status at the call's start: a count of finished blocks.
+static uint32_t* ticket_word(void* ws) { return static_cast<uint32_t*>(ws) + 1; }
 
 constexpr uint64_t kCutoffKeyTag = 0x5053505030303031ull;  // "PSPP0001"
 
@@ -363,47 +365,128 @@ __device__ __forceinline__ float2 merge_parts(const float2* __restrict__ part, i
   return make_float2(m, S);
 }
 
-// Fixed-order block sum of the rows' loss terms: warp shuffles, then warp 0 over the warp sums.
-__device__ __forceinline__ void block_loss_sum(double rl, double* __restrict__ block_loss) {
-  __shared__ double ws_sum[kFinThreads / 32];
+// A block of the forward's finalize (and of the shard statistics' merge) takes kMergeRows rows, one
+// per lane, and kMergeSlices warps that each merge every kMergeSlices-th of the rows' vocabulary
+// parts. A row of the 152k vocabulary has 1188 parts (9.5 KB), so the kernels are bound by reading
+// them: a warp's 32 rows of one part are 256 contiguous bytes, and 8 parts are in flight per thread.
+// One thread per row instead (two passes over the parts) left a few hundred rows on a handful of
+// SMs with a serial chain of 1188 loads: 254 us for 185 rows and 291 us for 7.8k rows at V = 152064
+// with the loss reduction then launched after it, against 16 and 25 us now; 208 us, 4.9 TB/s, at 106k
+// rows (before: 501 us). The order of the merge depends
+// on the number of parts alone, so a row's result does not depend on the batch around it.
+constexpr int kMergeRows = 32;
+constexpr int kMergeSlices = 16;
+constexpr int kMergeBatch = 8;
+
+// S 2^(x - m) for parts whose maximum x is at most m; a part without columns (x = -inf, S = 0) adds 0
+// even where no part has any yet (m = -inf).
+__device__ __forceinline__ float scaled_sum(float x, float S, float m) { return x == m ? S : S * exp2f(x - m); }
+
+// The merged (max, sum) of row `part` (its `count` parts, `stride` apart): valid in warp 0. Every warp
+// of the block calls it; rows past the end (live false) read nothing.
+__device__ __forceinline__ float2 merge_parts_block(const float2* __restrict__ part, int count, int64_t stride,
+                                                    bool live) {
+  __shared__ float2 slice_s[kMergeSlices][kMergeRows];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float m = -INFINITY, S = 0.f;
+  if (live) {
+    const float2* p = part + static_cast<int64_t>(warp) * stride;
+    const int64_t step = static_cast<int64_t>(kMergeSlices) * stride;
+    int c = warp;
+    for (; c + (kMergeBatch - 1) * kMergeSlices < count; c += kMergeBatch * kMergeSlices, p += kMergeBatch * step) {
+      float2 v[kMergeBatch];
 #pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) rl += __shfl_down_sync(0xffffffffu, rl, o);
-  if ((threadIdx.x & 31) == 0) ws_sum[threadIdx.x >> 5] = rl;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < kFinThreads / 32 ? ws_sum[threadIdx.x] : 0.0;
+      for (int j = 0; j < kMergeBatch; ++j) v[j] = p[j * step];
+      float mn = m;
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (threadIdx.x == 0) block_loss[blockIdx.x] = v;
+      for (int j = 0; j < kMergeBatch; ++j) mn = fmaxf(mn, v[j].x);
+      S = scaled_sum(m, S, mn);
+      m = mn;
+#pragma unroll
+      for (int j = 0; j < kMergeBatch; ++j) S += scaled_sum(v[j].x, v[j].y, m);
+    }
+    for (; c < count; c += kMergeSlices, p += step) {
+      const float2 v = *p;
+      const float mn = fmaxf(m, v.x);
+      S = scaled_sum(m, S, mn) + scaled_sum(v.x, v.y, mn);
+      m = mn;
+    }
   }
+  slice_s[warp][lane] = make_float2(m, S);
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int k = 0; k < kMergeSlices; ++k) m = fmaxf(m, slice_s[k][lane].x);
+    S = 0.f;
+#pragma unroll
+    for (int k = 0; k < kMergeSlices; ++k) S += scaled_sum(slice_s[k][lane].x, slice_s[k][lane].y, m);
+  }
+  return make_float2(m, S);
 }
 
-__global__ void __launch_bounds__(kFinThreads)
-    fwd_finalize_kernel(int64_t N, int V, int splits, const float2* __restrict__ part, const float* __restrict__ ztok,
+static unsigned merge_blocks(int64_t N) { return static_cast<unsigned>((N + kMergeRows - 1) / kMergeRows); }
+
+// Sum of v over the block in a fixed order (warp shuffles, then warp 0 over the warps' sums), in thread 0.
+__device__ __forceinline__ double block_sum(double v) {
+  __shared__ double ws_sum[32];
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) ws_sum[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    v = threadIdx.x < (blockDim.x >> 5) ? ws_sum[threadIdx.x] : 0.0;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  }
+  return v;
+}
+
+// The block's sum of row losses goes where its rows' first parts were (nobody else reads them), and
+// the last block to finish (`ticket`, zeroed at the call's start, counts them) adds the sums up: one
+// launch less than a separate reduction, and the same order of addition whichever block is last.
+__global__ void __launch_bounds__(kMergeRows* kMergeSlices)
+    fwd_finalize_kernel(int64_t N, int V, int splits, float2* __restrict__ part, const float* __restrict__ ztok,
                         const int32_t* __restrict__ tok, const float* __restrict__ oldlogp,
                         const float* __restrict__ adv, const float* __restrict__ w, double eps, double loss_scale,
-                        float* __restrict__ lse, float* __restrict__ logp, float* __restrict__ ratio,
-                        float* __restrict__ coef, float* __restrict__ row_loss, double* __restrict__ block_loss,
-                        uint32_t* status) {
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * kFinThreads + threadIdx.x;
-  double rl = 0.0;
-  if (i < N) {
-    const float2 ms = merge_parts(part + i, splits, N);
-    rl = finalize_row(i, ms.x, ms.y, ztok[i], tok[i], V, oldlogp, adv, w, eps, loss_scale, lse, logp, ratio, coef,
-                      row_loss, status);
+                        double* __restrict__ loss, float* __restrict__ lse, float* __restrict__ logp,
+                        float* __restrict__ ratio, float* __restrict__ coef, float* __restrict__ row_loss,
+                        uint32_t* ticket, uint32_t* status) {
+  __shared__ bool last;
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * kMergeRows + (threadIdx.x & 31);
+  const float2 ms = merge_parts_block(part + i, splits, N, i < N);
+  if (threadIdx.x < 32) {
+    double rl = 0.0;
+    if (i < N)
+      rl = finalize_row(i, ms.x, ms.y, ztok[i], tok[i], V, oldlogp, adv, w, eps, loss_scale, lse, logp, ratio, coef,
+                        row_loss, status);
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) rl += __shfl_down_sync(0xffffffffu, rl, o);
+    if (threadIdx.x == 0) {
+      *reinterpret_cast<double*>(part + i) = rl;
+      __threadfence();
+      last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
   }
-  block_loss_sum(rl, block_loss);
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double v = 0.0;
+  for (int64_t b = threadIdx.x; b < gridDim.x; b += blockDim.x)
+    v += __ldcg(reinterpret_cast<const double*>(part + b * kMergeRows));
+  v = block_sum(v);
+  if (threadIdx.x == 0) *loss = v;
 }
 
 // A vocabulary shard's statistics: its vocabulary tiles' (max, sum) pairs merged per row, and the
 // chosen logit where the row's token lies in the shard ([tok_base, tok_base + Vs)), -inf elsewhere.
-__global__ void __launch_bounds__(kFinThreads)
+__global__ void __launch_bounds__(kMergeRows* kMergeSlices)
     stats_merge_kernel(int64_t N, int splits, const float2* __restrict__ part, const float* __restrict__ ztok_ws,
                        const int32_t* __restrict__ tok, int64_t tok_base, int Vs, float2* __restrict__ stats,
                        float* __restrict__ ztok) {
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * kFinThreads + threadIdx.x;
-  if (i >= N) return;
-  stats[i] = merge_parts(part + i, splits, N);
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * kMergeRows + (threadIdx.x & 31);
+  const float2 ms = merge_parts_block(part + i, splits, N, i < N);
+  if (threadIdx.x >= 32 || i >= N) return;
+  stats[i] = ms;
   const int64_t t = static_cast<int64_t>(tok[i]) - tok_base;
   ztok[i] = (t >= 0 && t < Vs) ? ztok_ws[i] : -INFINITY;
 }
@@ -428,27 +511,20 @@ __global__ void __launch_bounds__(kFinThreads)
     rl = finalize_row(i, ms.x, ms.y, zt, tok[i], V, oldlogp, adv, w, eps, loss_scale, lse, logp, ratio, coef,
                       row_loss, status);
   }
-  block_loss_sum(rl, block_loss);
+  rl = block_sum(rl);
+  if (threadIdx.x == 0) block_loss[blockIdx.x] = rl;
 }
 
 __global__ void __launch_bounds__(1024) loss_reduce_kernel(int64_t nblocks, const double* __restrict__ part,
                                                            double* __restrict__ loss) {
   double v = 0.0;
   for (int64_t b = threadIdx.x; b < nblocks; b += 1024) v += part[b];
-  __shared__ double s[32];
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double u = s[threadIdx.x];
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) u += __shfl_down_sync(0xffffffffu, u, o);
-    if (threadIdx.x == 0) *loss = u;
-  }
+  v = block_sum(v);
+  if (threadIdx.x == 0) *loss = v;
 }
 
-// Forward workspace: header | ztok [N] f32 | block_loss [nb] f64 | part [S][N] float2. The
+// Forward workspace: header | ztok [N] f32 | 8 ceil(N / 256) bytes, unused (they keep the layout, and so
+// what a given workspace holds) | part [S][N] float2. The
 // (max, sum of exp) partials come last: S is as many as the workspace holds, up to two per
 // 256-column vocabulary tile (bf16: one per column group of the forward's epilogue, so the
 // vocabulary ranges per row are S / 2; at one range per tile every unit of the forward GEMM is one
@@ -456,7 +532,6 @@ __global__ void __launch_bounds__(1024) loss_reduce_kernel(int64_t nblocks, cons
 struct FwdWs {
   float2* part;
   float* ztok;
-  double* block_loss;
   int splits;       // S that fits (0 if not even one)
   size_t bytes;     // bytes used with that S
 };
@@ -478,7 +553,6 @@ static FwdWs fwd_ws(void* ws, int64_t N, int V, int dtype, size_t ws_bytes) {
   FwdWs f;
   uint8_t* base = static_cast<uint8_t*>(ws);
   f.ztok = reinterpret_cast<float*>(base + kWsHeader);
-  f.block_loss = reinterpret_cast<double*>(base + kWsHeader + align_up(sizeof(float) * N, 256));
   f.part = reinterpret_cast<float2*>(base + fixed);
   const int g = fwd_group(dtype);
   int S = full;
@@ -660,12 +734,9 @@ static int lmhead_fwd_impl(int64_t N, int d, int V, int dtype, const void* Hpk, 
                       status_word(ws), s);
   }
   if (rc != PS_OK) return rc;
-  const int64_t nb = (N + kFinThreads - 1) / kFinThreads;
-  fwd_finalize_kernel<<<static_cast<unsigned>(nb), kFinThreads, 0, s>>>(N, V, splits, f.part, f.ztok, tok, oldlogp,
-                                                                       adv, w, eps, loss_scale, lse, logp, ratio,
-                                                                       coef, row_loss, f.block_loss, status_word(ws));
-  if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
-  loss_reduce_kernel<<<1, 1024, 0, s>>>(nb, f.block_loss, loss);
+  fwd_finalize_kernel<<<merge_blocks(N), kMergeRows * kMergeSlices, 0, s>>>(
+      N, V, splits, f.part, f.ztok, tok, oldlogp, adv, w, eps, loss_scale, loss, lse, logp, ratio, coef, row_loss,
+      ticket_word(ws), status_word(ws));
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }
 
@@ -795,9 +866,8 @@ static int logit_stats_impl(int64_t N, int d, int Vs, int64_t v0, int dtype, con
                       f.ztok, status_word(ws), s, static_cast<int>(v0));
   }
   if (rc != PS_OK) return rc;
-  const int64_t nb = (N + kFinThreads - 1) / kFinThreads;
-  stats_merge_kernel<<<static_cast<unsigned>(nb), kFinThreads, 0, s>>>(N, splits, f.part, f.ztok, tok, v0, Vs,
-                                                                        reinterpret_cast<float2*>(stats), ztok);
+  stats_merge_kernel<<<merge_blocks(N), kMergeRows * kMergeSlices, 0, s>>>(N, splits, f.part, f.ztok, tok, v0, Vs,
+                                                                           reinterpret_cast<float2*>(stats), ztok);
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }
 
