@@ -69,11 +69,11 @@ struct GemmCfg {
   static constexpr int kAccBufs = HALVES == 1 ? 2 : 1;        // accumulator buffers in TMEM
 };
 
-// Epilogues that store through TMA (Epi::kTmaStore) stage each 32-row x 32-column 2-byte slice of a
-// warp in shared memory, 64-byte swizzled (a 64-byte row per TMEM lane, its 16-byte units permuted
-// by row bits 1-2, so a warp's stores hit every bank group): two buffers per warp with 4 epilogue
-// warps, one with 8 (two fit beside the wide-tile ring, 230.5 KB, but measured no faster).
-constexpr int kStageBytes = 32 * 64;
+// Epilogues that store through TMA (Epi::kTmaStore) stage each 32-row x 32-column slice of a warp in
+// shared memory (Epi::kStageBytes of it): 2-byte elements 64-byte swizzled (a 64-byte row per TMEM
+// lane, its 16-byte units permuted by row bits 1-2), 4-byte elements 128-byte swizzled (units permuted
+// by row bits 0-2), so a warp's stores hit every bank group either way. One buffer per warp: two for
+// 2-byte slices fit beside the wide-tile ring (230.5 KB) but measured no faster.
 
 // Epilogue warps per CTA: Epi::kEpiWarps, 4 or 8. With 8, each accumulator row is read by two
 // warps (columns 0..127 and 128..255 of every tile), which halves the time an epilogue holds a
@@ -84,15 +84,13 @@ struct EpiWarps {
   static_assert(Epi::kEpiWarps == 4 || Epi::kEpiWarps == 8, "4 or 8 epilogue warps");
   static constexpr int value = Epi::kEpiWarps;
 };
-template <int EW>
-struct StageBufs { static constexpr int value = EW == 8 ? 1 : 2; };
 
-template <int HALVES, int EW = 4>
+template <int HALVES, int EW, int SBYTES>
 struct GemmSmemT {
   // 1024-byte aligned tile ring first (128-byte swizzle atoms repeat every 1 KB)
   uint8_t a[GemmCfg<HALVES>::kStagesH][GemmCfg<HALVES>::kABytes];
   uint8_t b[GemmCfg<HALVES>::kStagesH][kTileBBytes];
-  uint8_t stage[EW][StageBufs<EW>::value][kStageBytes];   // store staging of the epilogue warps
+  uint8_t stage[EW][SBYTES > 0 ? SBYTES : 16];   // store staging of the epilogue warps
   uint64_t full[GemmCfg<HALVES>::kStagesH];
   uint64_t empty[GemmCfg<HALVES>::kStagesH];
   uint64_t tfull[2];
@@ -101,8 +99,10 @@ struct GemmSmemT {
   uint32_t tmem_base;
   int abort;
 };
-template <int HALVES, int EW = 4>
-constexpr size_t gemm_smem_bytes() { return sizeof(GemmSmemT<HALVES, EW>) + 1024; }  // + alignment slack
+template <int HALVES, class Epi>
+constexpr size_t gemm_smem_bytes() {   // + alignment slack
+  return sizeof(GemmSmemT<HALVES, EpiWarps<Epi>::value, Epi::kStageBytes>) + 1024;
+}
 
 // tmC: the output map of epilogues that store through TMA (unused by the others). An epilogue's
 // begin_unit / end_unit see the unit's split index times the column groups (1 with 4 epilogue
@@ -118,10 +118,9 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
   constexpr int EW = EpiWarps<Epi>::value;
   constexpr int G = EW / 4;                 // column groups per TMEM lane quarter
   constexpr int CPG = (kBN / 32) / G;       // 32-column chunks per group
-  constexpr int SB = StageBufs<EW>::value;
+  using Smem = GemmSmemT<HALVES, EW, Epi::kStageBytes>;
   extern __shared__ uint8_t smem_raw[];
-  GemmSmemT<HALVES, EW>& sm =
-      *reinterpret_cast<GemmSmemT<HALVES, EW>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
 
@@ -283,7 +282,6 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
     const int row_in_tile = quad * 32 + lane;
     typename Epi::State st[HALVES];             // a thread owns row r of each half
     uint32_t tile = 0;
-    uint32_t nstore = 0;                        // TMA-stored slices of this warp
     bool ok = true;
     for (int u = blockIdx.x; ok && u < sched.num_units; u += gridDim.x) {
       int m_blk, split, n0, n1;
@@ -319,17 +317,16 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
             if constexpr (Epi::kTmaStore) {
               // the slice goes to a staging buffer, then one lane stores the warp's 32 x 32 box
               if (col0 < Epi::cols(ep)) {
-                uint8_t* buf = sm.stage[ew][nstore % SB];
-                if (lane == 0) bulk_wait_group_read<SB - 1>();   // the store that last used it has read it
+                uint8_t* buf = sm.stage[ew];
+                if (lane == 0) bulk_wait_group_read<0>();   // the store that last used it has read it
                 __syncwarp();
                 Epi::chunk_to_smem(ep, st[h], row, col0, r, buf, lane);
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                  tma_store_2d(&tmC, buf, col0, m_blk * Cfg::kRows + h * kBM + quad * 32);
+                  Epi::store(ep, &tmC, buf, col0, m_blk * Cfg::kRows + h * kBM + quad * 32);
                   bulk_commit_group();
                 }
-                ++nstore;
               }
             } else {
               Epi::chunk(ep, st[h], row, col0, r);
