@@ -6,6 +6,7 @@
 // TMEM. Backward: the same product is recomputed per chunk of rows and turned into
 // dZ = coef (onehot - softmax) in bf16; dH = dZ W and dW = dZ^T Hpk are two more
 // tensor-core products over that chunk.
+#include <atomic>
 #include <mutex>
 
 #include <cuda_bf16.h>
@@ -645,6 +646,88 @@ static int launch_gemm_pair(const CUtensorMap& ta, const CUtensorMap& tb, int64_
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }
 
+// Clusters of `ranks` CTAs of the split-K kernel that run at once (one CTA per SM; a cluster stays inside
+// a GPC, so 152 SMs hold 76 pairs but 36 clusters of four and 16 of eight). Asked once per device.
+static int splitk_clusters_at_once(int ranks) {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[kDevices][4];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return num_sms_current() / (ranks + 1);
+  std::atomic<int>& slot = known[dev][ranks == 2 ? 1 : ranks == 4 ? 2 : 3];
+  int n = slot.load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  auto kern = umma_gemm_splitk_kernel<false, true, 2>;
+  constexpr size_t smem = sizeof(GemmSplitSmem<2>) + 1024;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(ranks);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(static_cast<unsigned>(num_sms_current() / ranks * ranks), 1, 1);
+  cfg.blockDim = dim3(kSplitThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(kern), &cfg) != cudaSuccess || n <= 0) {
+    cudaGetLastError();
+    n = num_sms_current() / (ranks + 1);
+  }
+  slot.store(n, std::memory_order_relaxed);
+  return n;
+}
+
+// Ranks per output tile (1: the persistent kernel) of a product with `tiles` output tiles and num_kb
+// k-blocks: the fewest rounds of (k-blocks per rank + the exchange). dH of a few rows has few tiles and
+// the vocabulary as its K loop. Measured, one CTA per tile against 2 / 4 / 8 ranks (us):
+//   d = 3584, V = 152064: 185 rows (14 tiles) 1353 / 688 / 363 / 217; 400 (28) 1332 / 676 / 357 / 412;
+//     1000 (56) 1326 / 660 / 710 / 832; 2048 (112) 1297 / 1342 / 1408 / 1668; 3000 (168) 2639 / 2010 /
+//     1770 / 2503; 4000 (224) 2631 / 1999 / 2482 / 3169.
+//   d = 392, V = 2000: 185 rows (2) 22.9 / 18.5 / 14.7 / 12.3; 4000 (32) 27.0 / 23.3 / 20.2 / 41.9.
+// Over 54 such sizes the rule picked the fastest of the four or one within 3% of it, but for one (600 rows,
+// d = 3584, V = 32000: 172 us with 8 ranks, 158 with 2). From two
+// tiles per SM on the persistent kernel's last round costs less than a third, and the split is off, so
+// that whole batches and their shards (hundreds of tiles each) add dH up in the same order.
+constexpr int kSplitOverheadKb = 12;   // the exchange and the launch, in k-blocks of a wide tile (0.55 us each)
+static int choose_splitk(int64_t tiles, int num_kb) {
+  if (tiles >= 2 * num_sms_current()) return 1;
+  auto cost = [&](int S) {
+    const int64_t at_once = S == 1 ? num_sms_current() : splitk_clusters_at_once(S);
+    return (tiles + at_once - 1) / at_once * ((num_kb + S - 1) / S + (S > 1 ? kSplitOverheadKb : 0));
+  };
+  int best = 1;
+  for (int S = 2; S <= 8 && S <= num_kb; S *= 2)
+    if (cost(S) * 100 < cost(best) * 97) best = S;
+  return best;
+}
+template <bool A_MN, bool B_MN, int HALVES>
+static int launch_gemm_splitk(const CUtensorMap& ta, const CUtensorMap& tb, int64_t M, int64_t N, int64_t K, int ranks,
+                              const SplitOut& o, uint32_t* status, cudaStream_t s) {
+  const int64_t m_blocks = (M + kBM * HALVES - 1) / (kBM * HALVES);
+  const int n_blocks = static_cast<int>((N + kBN - 1) / kBN);
+  auto kern = umma_gemm_splitk_kernel<A_MN, B_MN, HALVES>;
+  constexpr size_t smem = sizeof(GemmSplitSmem<HALVES>) + 1024;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    return PS_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(ranks);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(static_cast<unsigned>(m_blocks * n_blocks * ranks), 1, 1);
+  cfg.blockDim = dim3(kSplitThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, ta, tb, n_blocks, static_cast<int>((K + kBK - 1) / kBK), o, status,
+                            kDefaultTimeoutNs) == cudaSuccess
+             ? PS_OK
+             : PS_ERR_CUDA;
+}
+
 int fwd_tile_splits_bf16(int V) { return (V + kBN - 1) / kBN; }
 int fwd_partials_per_split_bf16() {
   static_assert(FwdLseEpi::kEpiWarps == FwdLseStoreEpi::kEpiWarps, "the two forwards write the same partials");
@@ -810,7 +893,18 @@ int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, flo
     if (!map_kmajor(&ta, dz, rc, V, ldz, 2 * kBM) || !map_mnmajor(&tb, W, V, d, d) || !map_out_f32(&tc, dH, rc, d, d))
       return PS_ERR_INVALID_ARG;
     StoreF32Epi::Params ep{d, dh_accumulate};
-    rcode = launch_gemm_single<false, true, StoreF32Epi, 2>(ta, tb, tc, rc, d, V, 0, kBandGrad, ep, status, s);
+    const int64_t tiles = ((rc + 2 * kBM - 1) / (2 * kBM)) * ((d + kBN - 1) / kBN);
+    const int ranks = choose_splitk(tiles, (V + kBK - 1) / kBK);
+    if (ranks > 1) {
+      const SplitOut o{dH, d, static_cast<int>(rc), d, dh_accumulate};
+      if (rc > kBM) {
+        rcode = launch_gemm_splitk<false, true, 2>(ta, tb, rc, d, V, ranks, o, status, s);
+      } else {   // one 128-row half holds every row
+        if (!map_kmajor(&ta, dz, rc, V, ldz, kBM)) return PS_ERR_INVALID_ARG;
+        rcode = launch_gemm_splitk<false, true, 1>(ta, tb, rc, d, V, ranks, o, status, s);
+      }
+    } else
+      rcode = launch_gemm_single<false, true, StoreF32Epi, 2>(ta, tb, tc, rc, d, V, 0, kBandGrad, ep, status, s);
     if (rcode != PS_OK) return rcode;
   }
   if (dW) {

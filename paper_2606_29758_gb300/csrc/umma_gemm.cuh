@@ -567,4 +567,206 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   }
 }
 
+// =============================================================================================
+// Split-K variant: a cluster of S = 2, 4 or 8 CTAs computes one 128 x 256 (HALVES = 1) or 256 x 256
+// output tile, rank r accumulating its share of the k-blocks in its own TMEM. The partial tiles meet
+// through distributed shared memory, 128 rows at a time: every CTA puts its partial into its own (idle)
+// operand ring, and each rank reads the S partials of its share of the columns (8 / S slices of 32), adds
+// them in rank order and writes the output, so the result does not depend on timing and no workspace is
+// needed. The owner pulls whole 128-byte lines: partials pushed from the accumulator's registers into the
+// owner (16 bytes per row and store) took 28 instead of 15 us for 400 rows at d = 392, V = 2000, and 448
+// instead of 412 us at d = 3584, V = 152064 (8 ranks). For outputs with fewer tiles than the chip has
+// SMs and a long K loop. Every CTA passes every cluster barrier, also after an expired wait (its partial is then
+// wrong and PS_DEV_TIMEOUT is set), so no peer is left waiting.
+// =============================================================================================
+constexpr int kSplitThreads = 320;
+
+template <int HALVES>
+struct GemmSplitSmem {
+  uint8_t a[GemmCfg<HALVES>::kStagesH][GemmCfg<HALVES>::kABytes];
+  uint8_t b[GemmCfg<HALVES>::kStagesH][kTileBBytes];
+  uint64_t full[GemmCfg<HALVES>::kStagesH];
+  uint64_t empty[GemmCfg<HALVES>::kStagesH];
+  uint64_t tfull;
+  uint32_t tmem_base;
+  int abort;
+};
+// the 8 slices of 128 rows x 32 f32 columns of a half's partial lie over the ring
+static_assert(GemmCfg<1>::kStagesH * (GemmCfg<1>::kABytes + kTileBBytes) >= 8 * 128 * 128, "ring too small");
+static_assert(GemmCfg<2>::kStagesH * (GemmCfg<2>::kABytes + kTileBBytes) >= 8 * 128 * 128, "ring too small");
+
+struct SplitOut {
+  float* out;   // [M][ld] f32, 16-byte aligned rows
+  int64_t ld;
+  int M, N;     // N % 4 == 0
+  int accumulate;
+};
+
+template <bool A_MN, bool B_MN, int HALVES>
+__global__ void __launch_bounds__(kSplitThreads, 1)
+    umma_gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                            int n_blocks, int num_kb, const SplitOut o, uint32_t* status, uint64_t timeout_ns) {
+  using Cfg = GemmCfg<HALVES>;
+  constexpr int S = Cfg::kStagesH;
+  extern __shared__ uint8_t smem_raw[];
+  GemmSplitSmem<HALVES>& sm = *reinterpret_cast<GemmSplitSmem<HALVES>*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const int nranks = static_cast<int>(cluster_nctarank());
+  const int rank = static_cast<int>(cluster_ctarank());
+  const int tile = blockIdx.x / nranks;
+  const int m_blk = tile / n_blocks, n_blk = tile - m_blk * n_blocks;
+  const int kb0 = static_cast<int>(static_cast<long long>(num_kb) * rank / nranks);
+  const int kb1 = static_cast<int>(static_cast<long long>(num_kb) * (rank + 1) / nranks);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(&sm.full[s], 1);
+      mbar_init(&sm.empty[s], 1);
+    }
+    mbar_init(&sm.tfull, 1);
+    sm.abort = 0;
+    fence_mbar_init();
+  }
+  if (warp == 0 && lane == 0) {
+    tma_prefetch_desc(&tmA);
+    tma_prefetch_desc(&tmB);
+  }
+  if (warp == 1) {
+    tmem_alloc(&sm.tmem_base, kTmemCols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = sm.tmem_base;
+  volatile int* abort = &sm.abort;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      uint32_t kc = 0;
+      bool ok = true;
+      const int m0 = m_blk * Cfg::kRows, nn0 = n_blk * kBN;
+      for (int kb = kb0; kb < kb1; ++kb, ++kc) {
+        const int s = kc % S;
+        if (!mbar_wait(&sm.empty[s], ((kc / S) & 1u) ^ 1u, timeout_ns, abort)) { ok = false; break; }
+        mbar_arrive_expect_tx(&sm.full[s], Cfg::kABytes + kTileBBytes);
+        const int k0 = kb * kBK;
+        if (A_MN) {
+          for (int i = 0; i < Cfg::kRows / 64; ++i)
+            tma_load_2d(sm.a[s] + i * (kBK * 128), &tmA, &sm.full[s], m0 + i * 64, k0);
+        } else {
+          tma_load_2d(sm.a[s], &tmA, &sm.full[s], k0, m0);
+        }
+        if (B_MN) {
+          for (int i = 0; i < kBN / 64; ++i)
+            tma_load_2d(sm.b[s] + i * (kBK * 128), &tmB, &sm.full[s], nn0 + i * 64, k0);
+        } else {
+          tma_load_2d(sm.b[s], &tmB, &sm.full[s], k0, nn0);
+        }
+      }
+      if (!ok) {
+        *abort = 1;
+        raise_status(status, PS_DEV_TIMEOUT);
+      }
+      // the ring is reused below: every load has landed (without an expired wait the MMAs saw to that)
+      const uint32_t first = kc > static_cast<uint32_t>(S) ? kc - S : 0;
+      for (uint32_t j = first; j < kc; ++j) mbar_wait(&sm.full[j % S], (j / S) & 1u, timeout_ns, nullptr);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      constexpr uint32_t idesc = idesc_bf16_f32(kBM, kBN, A_MN, B_MN);
+      constexpr uint32_t a_lbo = A_MN ? kBK * 128 : 16, a_step = A_MN ? 2048 : 32;
+      constexpr uint32_t b_lbo = B_MN ? kBK * 128 : 16, b_step = B_MN ? 2048 : 32;
+      uint32_t kc = 0;
+      for (int kb = kb0; kb < kb1; ++kb, ++kc) {
+        const int s = kc % S;
+        if (!mbar_wait(&sm.full[s], (kc / S) & 1u, timeout_ns, abort)) {
+          *abort = 1;
+          raise_status(status, PS_DEV_TIMEOUT);
+          break;
+        }
+        tc_fence_after();
+        const uint32_t a_base = smem_addr(sm.a[s]);
+        const uint32_t b_base = smem_addr(sm.b[s]);
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h)
+#pragma unroll
+          for (int k = 0; k < kBK / 16; ++k)
+            umma_bf16(tmem_base + h * kBN, smem_desc_sw128(a_base + h * kTileABytes + k * a_step, a_lbo, 1024),
+                      smem_desc_sw128(b_base + k * b_step, b_lbo, 1024), idesc, (kc | k) != 0 ? 1u : 0u);
+        umma_commit(&sm.empty[s]);
+      }
+      umma_commit(&sm.tfull);   // also after an expired wait: the MMAs issued so far still finish
+    }
+  }
+  __syncwarp();
+  {
+    // the accumulator is complete (bounded; a failure has set the status already or sets it here)
+    int got = 0;
+    if (lane == 0) got = mbar_wait(&sm.tfull, 0, timeout_ns, nullptr) ? 1 : 0;
+    got = __shfl_sync(0xffffffffu, got, 0);
+    if (!got && lane == 0) raise_status(status, PS_DEV_TIMEOUT);
+  }
+  tc_fence_after();
+  cluster_sync_all();   // every ring of the cluster is idle
+
+  const int per_owner = (kBN / 32) / nranks;   // 32-column slices a rank adds up and writes
+  const uint32_t base = smem_addr(sm.a);
+#pragma unroll 1
+  for (int h = 0; h < HALVES; ++h) {
+    if (warp >= 2) {
+      // this rank's partial of the half: slice c is 128 rows of 128 bytes, units permuted by row
+      const int quad = warp & 3, grp = (warp - 2) >> 2;
+      const int r = quad * 32 + lane;
+      const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + h * kBN;
+#pragma unroll 1
+      for (int c = grp * 4; c < grp * 4 + 4; ++c) {
+        uint32_t v[32];
+        tmem_ld32(t_row + c * 32, v);
+        tmem_ld_wait();
+        uint4* dst = reinterpret_cast<uint4*>(&sm.a[0][0]) + (c * 128 + r) * 8;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          dst[q ^ (r & 7)] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      }
+    }
+    cluster_sync_all();   // every rank's partial of this half is in its shared memory
+    for (int i = threadIdx.x; i < per_owner * 128 * 8; i += kSplitThreads) {
+      const int q = i & 7, r = (i >> 3) & 127, c = rank * per_owner + (i >> 10);
+      const int row = m_blk * Cfg::kRows + h * kBM + r;
+      const int col = n_blk * kBN + c * 32 + q * 4;
+      if (row >= o.M || col >= o.N) continue;
+      // the ranks' partials, two loads in flight per pair, added in rank order
+      const uint32_t at = base + ((c * 128 + r) * 8 + (q ^ (r & 7))) * 16;
+      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int k = 0; k < nranks; k += 2) {
+        const float4 x = ld_cluster_v4(mapa_shared(at, k)), y = ld_cluster_v4(mapa_shared(at, k + 1));
+        s.x = k ? (s.x + x.x) + y.x : x.x + y.x;
+        s.y = k ? (s.y + x.y) + y.y : x.y + y.y;
+        s.z = k ? (s.z + x.z) + y.z : x.z + y.z;
+        s.w = k ? (s.w + x.w) + y.w : x.w + y.w;
+      }
+      float4* d = reinterpret_cast<float4*>(o.out + static_cast<int64_t>(row) * o.ld + col);
+      if (o.accumulate) {
+        const float4 t = *d;
+        s.x += t.x;
+        s.y += t.y;
+        s.z += t.z;
+        s.w += t.w;
+      }
+      *d = s;
+    }
+    cluster_sync_all();   // nobody reads this rank's partial any more: it may be replaced, or the CTA may exit
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, kTmemCols);
+  }
+}
+
 }  // namespace psk
