@@ -865,7 +865,7 @@ int proxy_topk_gemm_bf16(int64_t N, int d, int V, const void* Hrows, const void*
 
 int bwd_chunk_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, const int32_t* tok,
                    const float* lse, const float* coef, float* dH, float* dW, int dw_accumulate, void* dz,
-                   int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate) {
+                   int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call) {
   int rcode;
   {
     CUtensorMap ta, tb;
@@ -879,21 +879,21 @@ int bwd_chunk_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, con
                                                                     kBandRecompute / kRecHalves, ep, status, s);
     if (rcode != PS_OK) return rcode;
   }
-  return bwd_grads_bf16(rc, d, V, Hpk, W, dH, dW, dw_accumulate, dz, ldz, status, s, dh_accumulate);
+  return bwd_grads_bf16(rc, d, V, Hpk, W, dH, dW, dw_accumulate, dz, ldz, status, s, dh_accumulate, n_call);
 }
 
 // dH = dZ W and dW (+)= dZ^T H over rc rows of dZ [rc][ldz] bf16. Both have long K loops (V and rc):
 // one CTA computes a 256 x 256 tile as two M = 128 halves that share each B stage (a third fewer
-// operand bytes per FLOP).
+// operand bytes per FLOP); a call of few rows splits dH's K loop over clusters (choose_splitk).
 int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, float* dH, float* dW, int dw_accumulate,
-                   const void* dz, int64_t ldz, uint32_t* status, cudaStream_t s, int dh_accumulate) {
+                   const void* dz, int64_t ldz, uint32_t* status, cudaStream_t s, int dh_accumulate, int64_t n_call) {
   int rcode;
   if (dH) {
     CUtensorMap ta, tb, tc;
     if (!map_kmajor(&ta, dz, rc, V, ldz, 2 * kBM) || !map_mnmajor(&tb, W, V, d, d) || !map_out_f32(&tc, dH, rc, d, d))
       return PS_ERR_INVALID_ARG;
     StoreF32Epi::Params ep{d, dh_accumulate};
-    const int64_t tiles = ((rc + 2 * kBM - 1) / (2 * kBM)) * ((d + kBN - 1) / kBN);
+    const int64_t tiles = ((n_call + 2 * kBM - 1) / (2 * kBM)) * ((d + kBN - 1) / kBN);
     const int ranks = choose_splitk(tiles, (V + kBK - 1) / kBK);
     if (ranks > 1) {
       const SplitOut o{dH, d, static_cast<int>(rc), d, dh_accumulate};

@@ -771,7 +771,7 @@ static int bwd_from_store_impl(int64_t N, int d, int V, int64_t tok_base, int dt
   rc = dz_from_store_bf16(N, V, store, L.ldz, scale, N, tok, lse, logp, coef, s, static_cast<int>(tok_base));
   if (rc != PS_OK) return rc;
   return bwd_grads_bf16(N, d, V, Hpk, W, dH, dW, (flags & PS_DW_ACCUMULATE) ? 1 : 0, store, L.ldz, status_word(ws),
-                        s, (flags & PS_DH_ACCUMULATE) ? 1 : 0);
+                        s, (flags & PS_DH_ACCUMULATE) ? 1 : 0, N);
 }
 
 extern "C" {
@@ -967,12 +967,12 @@ static int lmhead_bwd_impl(int64_t N, int d, int V, int64_t tok_base, int dtype,
     if (dtype == PS_DTYPE_BF16) {
       const uint16_t* h = static_cast<const uint16_t*>(Hpk) + r0 * d;
       rc = bwd_chunk_bf16(rcn, d, V, h, W, tok + r0, lse + r0, coef + r0, dH ? dH + r0 * d : nullptr, dW, acc, dz,
-                          ldz, status_word(ws), s, static_cast<int>(tok_base), hacc);
+                          ldz, status_word(ws), s, static_cast<int>(tok_base), hacc, N);
     } else {
       const float* h = static_cast<const float*>(Hpk) + r0 * d;
       rc = bwd_chunk_f32(rcn, d, V, h, static_cast<const float*>(W), tok + r0, lse + r0, coef + r0,
                          dH ? dH + r0 * d : nullptr, dW, acc, static_cast<float*>(dz), ldz, status_word(ws), s,
-                         static_cast<int>(tok_base), hacc);
+                         static_cast<int>(tok_base), hacc, N);
     }
     if (rc != PS_OK) return rc;
   }
