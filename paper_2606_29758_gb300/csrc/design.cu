@@ -208,24 +208,33 @@ __global__ void group_offsets_kernel(int B, const int32_t* __restrict__ L, int64
 }
 
 // ================================================================== design
-// Lanes of the warp that tries saturated prefixes side by side in the capped design.
-constexpr int kCapLanes = 32;
+constexpr int kDesignThreads = 256;
+constexpr int kDesignWarps = kDesignThreads / 32;
 
+// Arrays of 2 T_max entries that the capped design takes from each of bW, bs and bn per prompt (the workspace
+// has room for 16 of each).
+constexpr int kDesignArrays = 16;
 struct DesignWs {
   double* w;       // [P][T_max] weights
   double* xi;      // [P][T_max]
-  double* bW;      // [P][T_max][kCapLanes] PAV block weights, one stack per lane (interleaved)
-  double* bs;      // [P][T_max][kCapLanes] PAV block scores sqrt(W / n)
-  int32_t* bn;     // [P][T_max][kCapLanes] PAV block lengths
-  int64_t* off;    // [P][K] row offsets of the group's completions
+  double* bW;      // [P][kDesignArrays][2 T_max]
+  double* bs;      // [P][kDesignArrays][2 T_max]
+  int32_t* bn;     // [P][kDesignArrays][2 T_max]
 };
 
 // True when the block (Wc, nc) violates the order against the block (Wp, np) below it, i.e. when
 // sqrt(Wp / np) < sqrt(Wc / nc) with both quotients and roots rounded to double, exactly as the
 // sequential definition decides it. The cross products Wp nc and Wc np settle every case whose
-// quotients differ by more than 2^-40 relative (then the rounded roots are ordered the same way);
-// only near-ties pay for the two divisions and square roots, which are slow in double precision.
+// quotients differ by more than 2^-40 relative (then the rounded roots are ordered the same way), and
+// in float (each within 2^-22) those that differ by more than 2^-19: an SM of GB300 does two FP64 operations a clock,
+// so double operations, let alone the near-ties' divisions and square roots, are slow (the design
+// of 8 prompts of 15350 steps: 1.71 ms, without the float test 1.86).
 __device__ __forceinline__ bool pav_violates(double Wp, int np, double Wc, int nc) {
+  const float fa = static_cast<float>(Wp) * static_cast<float>(nc), fb = static_cast<float>(Wc) * static_cast<float>(np);
+  if (fa > 1e-30f && fb > 1e-30f && fa < 1e30f && fb < 1e30f) {
+    if (fb > fa * (1.0f + 0x1p-19f)) return true;
+    if (fb < fa * (1.0f - 0x1p-19f)) return false;
+  }
   const double a = __dmul_rn(Wp, static_cast<double>(nc));
   const double b = __dmul_rn(Wc, static_cast<double>(np));
   if (a > 0x1p-900 && b > 0x1p-900 && a < 0x1p900 && b < 0x1p900) {
@@ -235,206 +244,475 @@ __device__ __forceinline__ bool pav_violates(double Wp, int np, double Wc, int n
   return __dsqrt_rn(__ddiv_rn(Wp, static_cast<double>(np))) < __dsqrt_rn(__ddiv_rn(Wc, static_cast<double>(nc)));
 }
 
-// Pool adjacent violators over w[0..T) (Appendix F) into one lane's stack (element m of the stack
-// at index m * kCapLanes): a new block is merged with the one below it while the block below has
-// the smaller score sqrt(W / n); merged weights add as W_prev + W_last, in the order of the
-// sequential definition, so every block sum is the same double. Returns the number of blocks (-1
-// if *stop was set before the end).
-__device__ int pav_stack_dev(const double* w, int T, double* bW, int32_t* bn, const volatile int* stop = nullptr) {
-  // The top block stays in registers (Wt, nt); the blocks below it are in memory at [0, nb - 1).
-  // Memory is read only when a merge uncovers the block below.
-  int nb = 0;
-  double Wt = 0.0;
-  int nt = 0;
-  double wnext = T > 0 ? w[0] : 0.0;
-  for (int t0 = 0; t0 < T; t0 += 64) {
-    if (stop != nullptr && *stop) return -1;   // abandoned: the caller needs no answer
-    const int t1 = min(T, t0 + 64);
-    for (int t = t0; t < t1; ++t) {
-      if (t + 16 < T) asm volatile("prefetch.global.L1 [%0];" ::"l"(w + t + 16));
-      double Wc = wnext;
-      if (t + 1 < T) wnext = w[t + 1];
-      int nc = 1;
-      while (nb > 0 && pav_violates(Wt, nt, Wc, nc)) {
-        Wc = __dadd_rn(Wt, Wc);
-        nc += nt;
-        --nb;
-        if (nb > 0) {
-          Wt = bW[(nb - 1) * kCapLanes];
-          nt = bn[(nb - 1) * kCapLanes];
+// Float-float numbers (an unevaluated sum hi + lo of two floats, about 44 significant bits). Knuth's TwoSum
+// and the Dekker renormalisation.
+struct FF {
+  float hi, lo;
+};
+__device__ __forceinline__ FF ff_add(FF a, FF b) {
+  const float lo = a.lo + b.lo;
+  const float s = a.hi + b.hi;
+  const float bb = s - a.hi;
+  const float e = ((a.hi - (s - bb)) + (b.hi - bb)) + lo;
+  const float h = s + e;
+  return FF{h, e - (h - s)};
+}
+__device__ __forceinline__ FF ff_select(bool c, FF a, FF b) { return FF{c ? a.hi : b.hi, c ? a.lo : b.lo}; }
+
+__device__ __forceinline__ FF ff_shfl_up(FF v, int o) {
+  return FF{__shfl_up_sync(0xffffffffu, v.hi, o), __shfl_up_sync(0xffffffffu, v.lo, o)};
+}
+// a - b as a float (a relative error of about 2^-23 of the difference beside the sums' own).
+__device__ __forceinline__ float ff_diff(float2 a, float2 b) { return (a.x - b.x) + (a.y - b.y); }
+
+// About 1 ulp (PTX sqrt.approx.ftz.f32).
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// ---------------------------------------------------------------- pooling by convex-hull links
+// Pooling adjacent violators over weights w[s..T) one after another leaves, after t of them, blocks whose
+// means fall from left to right: the segments of the least concave majorant of the prefix sums. The last
+// block starts at link(t) = argmin_{a < t} (S_t - S_a) / (t - a), which every t can look for by itself, so the
+// CTA finds the links of kWin positions at a time (below) and no longer walks the chain of decisions with one
+// thread, whose every step costs 0.3 us or more: a dependent FP64 addition takes 64 cycles on GB300, and a
+// divergent loop's turn some 50 before its work. The design kernel, 8 prompts, T = 15350: 13.7 ms with the
+// one-thread walks (4.5 ms once their loops had no branches and decided in floats), 1.69 ms now; 2 prompts,
+// T = 3240: 2.59 against 0.33 ms. What is left, at T = 15350: 0.35 ms for each search of links, 0.1 for each
+// prefix sum, 0.7 for the sums by the links (rounds of a barrier and an FP64 addition), 0.1 for their check.
+constexpr int kWin = kDesignThreads;
+constexpr int kHullSmem = 14336;       // hull vertices in shared memory (deeper ones in the workspace)
+constexpr size_t kDesignDynSmem = kHullSmem * (sizeof(float2) + sizeof(int32_t));
+
+// S[u], u = 0..n: the sums of the first u values (float-float), times sign. value(i) is the i-th one.
+template <class F>
+__device__ void ff_prefix_sums(F value, int n, float sign, float2* S) {
+  __shared__ float2 warp_s[kDesignWarps];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  FF carry{0.f, 0.f};
+  if (tid == 0) S[0] = make_float2(0.f, 0.f);
+  for (int i0 = 0; i0 < n; i0 += kDesignThreads) {
+    const int i = i0 + tid;
+    FF v{0.f, 0.f};
+    if (i < n) v = value(i);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const FF y = ff_shfl_up(v, o);
+      if (lane >= o) v = ff_add(y, v);
+    }
+    if (lane == 31) warp_s[wid] = make_float2(v.hi, v.lo);
+    __syncthreads();
+    FF before = carry;
+    for (int k = 0; k < kDesignWarps; ++k) {
+      const FF x{warp_s[k].x, warp_s[k].y};
+      if (k < wid) before = ff_add(before, x);
+      carry = ff_add(carry, x);
+    }
+    v = ff_add(before, v);
+    if (i < n) S[i + 1] = make_float2(sign * v.hi, sign * v.lo);
+    __syncthreads();
+  }
+}
+
+// link[u] = argmin over v < u of (S[u] - S[v]) / (u - v) (the nearest v on ties), u = 1..n. The hull of
+// S[0..lo] is kept as a stack of its vertices; a window's positions lo < u <= lo + kWin look at every v of the
+// window themselves (at most 256 steps) and at the hull by bisection (along it the slope to u falls, then
+// rises); the walk from the window's end along the links then gives the next hull. Compared in float, so a
+// link may be another whose slope is within about 2^-22 of the smallest.
+__device__ void hull_links(const float2* S, int n, int32_t* link, float2* hull_S, int32_t* hull, int32_t* hull_deep) {
+  __shared__ float2 win_S[kWin + 1];
+  __shared__ int win_link[kWin], win_at[kWin], path[kWin];
+  __shared__ int path_n, path_base;
+  const int tid = threadIdx.x;
+  auto vertex = [&](int i) { return i < kHullSmem ? hull[i] : hull_deep[i]; };
+  auto vertex_S = [&](int i, int v) { return i < kHullSmem ? hull_S[i] : S[v]; };
+  if (tid == 0) {
+    hull[0] = 0;
+    hull_S[0] = S[0];
+  }
+  int depth = 1;
+  for (int lo = 0; lo < n; lo += kWin) {
+    const int m = min(kWin, n - lo);
+    for (int i = tid; i <= m; i += kDesignThreads) win_S[i] = S[lo + i];
+    __syncthreads();
+    if (tid < m) {
+      const int u = lo + 1 + tid;
+      const float2 Su = win_S[tid + 1];
+      int best = u - 1, at = -1;
+      float bd = ff_diff(Su, win_S[tid]), bn = 1.f;
+      float nv = 1.f;
+      for (int k = tid - 1; k >= 0; --k) {
+        const float dv = ff_diff(Su, win_S[k]);
+        nv += 1.f;
+        if (dv * bn < bd * nv) {
+          bd = dv;
+          bn = nv;
+          best = lo + k;
         }
       }
-      if (nb > 0) {
-        bW[(nb - 1) * kCapLanes] = Wt;
-        bn[(nb - 1) * kCapLanes] = nt;
+      int l = 0, r = depth - 1;   // the top vertex is lo itself
+      while (l < r) {
+        const int mid = (l + r) >> 1;
+        const int a = vertex(mid), b = vertex(mid + 1);
+        const float2 Sa = vertex_S(mid, a), Sb = vertex_S(mid + 1, b);
+        if (ff_diff(Sb, Sa) * static_cast<float>(u - a) > ff_diff(Su, Sa) * static_cast<float>(b - a)) l = mid + 1;
+        else r = mid;
       }
-      Wt = Wc;
-      nt = nc;
-      ++nb;
+      if (l < depth - 1) {
+        const int a = vertex(l);
+        if (ff_diff(Su, vertex_S(l, a)) * bn < bd * static_cast<float>(u - a)) {
+          best = a;
+          at = l;
+        }
+      }
+      win_link[tid] = best;
+      win_at[tid] = at;
+      link[u] = best;
     }
+    __syncthreads();
+    if (tid == 0) {
+      int cnt = 0, u = lo + m, base = depth;
+      while (u > lo) {
+        path[cnt++] = u;
+        const int i = u - lo - 1;
+        if (win_at[i] >= 0) base = win_at[i] + 1;
+        u = win_link[i];
+      }
+      path_n = cnt;
+      path_base = base;
+    }
+    __syncthreads();
+    depth = path_base + path_n;
+    for (int i = tid; i < path_n; i += kDesignThreads) {
+      const int v = path[path_n - 1 - i], j = path_base + i;
+      if (j < kHullSmem) {
+        hull[j] = v;
+        hull_S[j] = win_S[v - lo];
+      } else {
+        hull_deep[j] = v;
+      }
+    }
+    __syncthreads();
   }
-  if (nb > 0) {
-    bW[(nb - 1) * kCapLanes] = Wt;
-    bn[(nb - 1) * kCapLanes] = nt;
-  }
-  return nb;
 }
 
 // ---------------------------------------------------------------- capped design: locating the prefix
 // The capped design saturates the smallest prefix s whose suffix design (w[s..T), budget B - s)
 // starts at or below 1. Whether a prefix qualifies is not monotone in s, so it cannot be bisected;
-// instead one pass of pooling from the right gives every suffix's first value at once: once w[t]
-// has been pushed (and pooled with the blocks to its right while it violates the order), the stack
-// holds the pooled blocks of the suffix w[t..T), because the pooled solution of a suffix is unique
-// whatever order its violators are pooled in (only the rounding of the block sums depends on it).
-// With D(t) = sum over those blocks of n_m s_m = sqrt(n_m W_m), the suffix design starts at
-// g(t) = (B - t) s_front / D(t). The pass records whether g(t) is clearly above 1 (0), clearly
-// below (2) or within kCapBand of 1 (1); only the last kind, and the first clear one, are then
-// decided by the exact rounded sequence of the definition.
+// instead the links of the weights taken from the right give the first block [t, T - link) of every suffix
+// design at once. With D(t) = sum over a suffix's blocks of n_m s_m = sqrt(n_m W_m), which is its first block's
+// term plus D at that block's end, the suffix design starts at g(t) = (B - t) s_front / D(t). status[t] records
+// whether g(t) is clearly above 1 (0), clearly below (2) or within kCapBand of 1 (1); only the last kind, and
+// the first clear one, are then decided by the exact rounded sequence of the definition.
+// The first block's mean is the largest slope from t, hence at least Q_t / (T - t) with Q_t the sum of the
+// suffix, of which the float-float sums are off by 2^-45: its weight is off by 2^-45 (T - t) / n relative, 2^-21 at
+// the largest T. Roots, products and the comparison add a few 2^-24: far inside kCapBand.
 constexpr double kCapBand = 0x1p-16;
 constexpr int kMaxNearCap = 64;        // prefixes within the band decided exactly (beyond: the full scan)
-constexpr int kCapStackSmem = 8192;    // stack entries of the status pass held in shared memory
 
-// Float-float numbers (an unevaluated sum hi + lo of two floats, about 44 significant bits): the
-// status pass's block sums and D. Knuth's TwoSum and the Dekker renormalisation.
-struct FF {
-  float hi, lo;
-};
-__device__ __forceinline__ FF ff_add(FF a, FF b) {
-  const float s = a.hi + b.hi;
-  const float bb = s - a.hi;
-  const float e = (a.hi - (s - bb)) + (b.hi - bb) + a.lo + b.lo;
-  const float h = s + e;
-  return FF{h, e - (h - s)};
-}
-
-// One thread: status[t] for t = T-1 down to 0 (see above), in float arithmetic (the FP64 units are
-// far slower). ws[t] = w[t] / max_t w[t] as floats (g does not depend on the scale, and every
-// n W then lies in [1e-12, T]); block sums and D as float-float numbers, roots and the comparison
-// in float: g is within about 2e-7 relative of its exact value, far inside kCapBand. The stack keeps
-// its front block in registers, the next kCapStackSmem entries in shared memory (W, n and the
-// root r = sqrt(n W) of each block, so that a pooled block leaves D as it entered) and deeper ones
-// in gW / gn / gr with stride kCapLanes. Stops early once *stop is set.
-__device__ void cap_status_pass(const float* __restrict__ ws, int T, double B, float2* sW, int32_t* sn, float* sr,
-                                double* gW, int32_t* gn, double* gr, float* status, const volatile int* stop) {
-  int nb = 0;            // blocks below the front
-  FF Wf{0.f, 0.f};       // front block
-  int nf = 0;
-  float rf = 0.f;
-  FF D{0.f, 0.f};
+// S, link: of the weights from the right, u = T - t, S negated. D [T + 1] scratch.
+__device__ void cap_status(const float2* S, const int32_t* link, int T, double B, float2* D, float* status) {
+  __shared__ float2 acc_s[kWin];
+  __shared__ int ptr_s[kWin];
+  const int tid = threadIdx.x;
   const float hi_band = static_cast<float>(1.0 + kCapBand), lo_band = static_cast<float>(1.0 - kCapBand);
-  for (int t = T - 1; t >= 0; --t) {
-    if ((t & 255) == 0 && *stop) return;   // the prefix s = 0 already qualifies: no status is needed
-    if (t >= 32) asm volatile("prefetch.global.L1 [%0];" ::"l"(ws + t - 32));
-    FF Wc{ws[t], 0.f};
-    int nc = 1;
-    // the new block sits left of the front: pool while its mean is below the front's
-    while (nf > 0 && Wf.hi * static_cast<float>(nc) > Wc.hi * static_cast<float>(nf)) {
-      D = ff_add(D, FF{-rf, 0.f});
-      Wc = ff_add(Wc, Wf);
-      nc += nf;
-      if (nb > 0) {
-        --nb;
-        if (nb < kCapStackSmem) {
-          const float2 v = sW[nb];
-          Wf = FF{v.x, v.y};
-          nf = sn[nb];
-          rf = sr[nb];
-        } else {
-          const float2 v = reinterpret_cast<const float2*>(gW)[static_cast<int64_t>(nb) * kCapLanes];
-          Wf = FF{v.x, v.y};
-          nf = gn[static_cast<int64_t>(nb) * kCapLanes];
-          rf = static_cast<float>(gr[static_cast<int64_t>(nb) * kCapLanes]);
-        }
-      } else {
-        nf = 0;
+  // B - t as a float: B's whole part less t is exact, so the sum is within an ulp
+  const int B_whole = static_cast<int>(B);
+  const float B_rest = static_cast<float>(B - static_cast<double>(B_whole));
+  for (int lo = 0; lo < T; lo += kWin) {
+    const int m = min(kWin, T - lo), u = lo + 1 + tid;
+    int ptr = 0;
+    float n = 1.f, r = 0.f;
+    FF acc{0.f, 0.f};
+    if (tid < m) {
+      ptr = link[u];
+      n = static_cast<float>(u - ptr);
+      r = sqrt_approx(n * ff_diff(S[ptr], S[u]));
+      acc.hi = r;
+    }
+    // sums along the links inside the window, twice as far each round
+    while (__syncthreads_or(ptr > lo)) {
+      acc_s[tid] = make_float2(acc.hi, acc.lo);
+      ptr_s[tid] = ptr;
+      __syncthreads();
+      if (ptr > lo) {
+        const int i = ptr - lo - 1;
+        acc = ff_add(acc, FF{acc_s[i].x, acc_s[i].y});
+        ptr = ptr_s[i];
       }
     }
-    if (nf > 0) {
-      if (nb < kCapStackSmem) {
-        sW[nb] = make_float2(Wf.hi, Wf.lo);
-        sn[nb] = nf;
-        sr[nb] = rf;
-      } else {
-        reinterpret_cast<float2*>(gW)[static_cast<int64_t>(nb) * kCapLanes] = make_float2(Wf.hi, Wf.lo);
-        gn[static_cast<int64_t>(nb) * kCapLanes] = nf;
-        gr[static_cast<int64_t>(nb) * kCapLanes] = rf;
+    if (tid < m) {
+      if (ptr > 0) {
+        const float2 rest = D[ptr];
+        acc = ff_add(acc, FF{rest.x, rest.y});
       }
-      ++nb;
+      D[u] = make_float2(acc.hi, acc.lo);
+      const int t = T - u;
+      const float num = (static_cast<float>(B_whole - t) + B_rest) * r, den = acc.hi * n;
+      status[t] = num > hi_band * den ? 0.f : (num < lo_band * den ? 2.f : 1.f);
     }
-    Wf = Wc;
-    nf = nc;
-    rf = sqrtf(static_cast<float>(nc) * Wc.hi);
-    D = ff_add(D, FF{rf, 0.f});
-    const float num = static_cast<float>(B - static_cast<double>(t)) * rf, den = D.hi * static_cast<float>(nc);
-    status[t] = num > hi_band * den ? 0.f : (num < lo_band * den ? 2.f : 1.f);
+    __syncthreads();
   }
 }
 
-constexpr size_t kDesignDynSmem = kCapStackSmem * (sizeof(float2) + sizeof(int32_t) + sizeof(float));
+// ---------------------------------------------------------------- pooling in the definition's arithmetic
+// first[t], W[t] for s < t <= T: the last block [first[t], t) after the weights w[s..t) have been pooled one after
+// another, and its sum as the definition adds it: the new weight c, then W_prev + c for each block that it
+// violates the order with, from the nearest on. A block below the last one is the last one of an earlier t, so
+// the sums of many t can be taken at a time where the links say which blocks they merge; and every decision is
+// then checked on the sums themselves (pav_violates), which by induction over t makes the result the sequential
+// one whatever the links were. The first t whose decisions differ (a near-tie that the links' float slopes took
+// the wrong way) is redone alone and what follows it again; after kMaxRepairs of those one thread does the rest.
+constexpr int kMaxRepairs = 8;
+struct Pooled {
+  const double* w;
+  int s, T;
+  int32_t* link;     // [T - s + 1], relative to s
+  int32_t* first;    // [T + 1]
+  double* W;         // [T + 1]
 
-constexpr int kDesignThreads = 256;
+  __device__ __forceinline__ bool violates(int j, double c, int n) const {
+    return pav_violates(W[j], j - first[j], c, n);
+  }
+  // Position t as the definition does it, on the positions before it (one thread).
+  __device__ void step(int t) const {
+    double c = w[t - 1];
+    int j = t - 1;
+    while (j > s && violates(j, c, t - j)) {
+      c = __dadd_rn(W[j], c);
+      j = first[j];
+    }
+    W[t] = c;
+    first[t] = j;
+  }
+  // Positions t0..T by the links (the whole CTA).
+  __device__ void by_links(int t0) const {
+    __shared__ double W_s[kWin];
+    __shared__ int first_s[kWin];
+    __shared__ int ready_s[kWin];
+    const int tid = threadIdx.x;
+    for (int lo = t0 - 1; lo < T; lo += kWin) {
+      const int t = lo + 1 + tid;
+      const bool mine = t <= T;
+      double c = mine ? w[t - 1] : 0.0;
+      int j = t - 1;
+      const int target = mine ? s + link[t - s] : j;
+      bool done = !mine;
+      ready_s[tid] = 0;
+      __syncthreads();
+      while (true) {
+        bool fresh = false;
+        if (!done) {
+          while (j > target) {
+            const int k = j - lo - 1;
+            if (k < 0) {
+              c = __dadd_rn(W[j], c);
+              j = first[j];
+            } else {
+              if (!ready_s[k]) break;
+              c = __dadd_rn(W_s[k], c);
+              j = first_s[k];
+            }
+          }
+          if (j <= target) {
+            W_s[tid] = c;
+            first_s[tid] = j;
+            done = fresh = true;
+          }
+        }
+        __syncthreads();
+        if (fresh) ready_s[tid] = 1;
+        if (!__syncthreads_or(!done)) break;
+      }
+      if (mine) {
+        W[t] = c;
+        first[t] = j;
+      }
+      __syncthreads();
+    }
+  }
+  // The first position in t0..T whose decisions are not the definition's, T + 1 if none (the whole CTA).
+  __device__ int first_wrong(int t0) const {
+    __shared__ int wrong_s;
+    if (threadIdx.x == 0) wrong_s = T + 1;
+    __syncthreads();
+    for (int t = t0 + threadIdx.x; t <= T; t += kDesignThreads) {
+      double c = w[t - 1];
+      int j = t - 1;
+      const int f = first[t];
+      bool ok = true;
+      while (ok && j > f) {
+        ok = violates(j, c, t - j);
+        c = __dadd_rn(W[j], c);
+        j = first[j];
+      }
+      if (ok && j > s) ok = !violates(j, c, t - j);
+      if (!ok) atomicMin(&wrong_s, t);
+    }
+    __syncthreads();
+    const int r = wrong_s;
+    __syncthreads();
+    return r;
+  }
+  __device__ void run() const {
+    int t = s + 1;
+    for (int repairs = 0;; ++repairs) {
+      by_links(t);
+      t = first_wrong(t);
+      if (t > T) return;
+      if (threadIdx.x == 0) {
+        step(t);
+        link[t - s] = first[t] - s;
+        if (repairs == kMaxRepairs)
+          for (int k = t + 1; k <= T; ++k) step(k);
+      }
+      __syncthreads();
+      if (repairs == kMaxRepairs || ++t > T) return;
+    }
+  }
+  // The blocks after all weights, last one first: their ends in `ends`; returns their number (the whole CTA).
+  // A position is a block's end if no later one's block reaches over it.
+  __device__ int blocks(int32_t* ends) const {
+    __shared__ int min_s[kDesignWarps], cnt_s[kDesignWarps];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    int reach = T, count = 0;   // the smallest start among positions further right, and the ends found there
+    for (int t0 = T; t0 > s; t0 -= kDesignThreads) {
+      const int t = t0 - tid;   // thread order runs from right to left
+      const int f = t > s ? first[t] : T;
+      int low = f;              // smallest start among this and the earlier threads of the warp
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, low, o);
+        if (lane >= o) low = min(low, y);
+      }
+      if (lane == 31) min_s[wid] = low;
+      int right = __shfl_up_sync(0xffffffffu, low, 1);   // ... among the earlier threads alone
+      if (lane == 0) right = T;
+      __syncthreads();
+      right = min(right, reach);
+      for (int k = 0; k < kDesignWarps; ++k) {
+        if (k < wid) right = min(right, min_s[k]);
+        reach = min(reach, min_s[k]);
+      }
+      const bool end = t > s && right >= t;
+      const unsigned mask = __ballot_sync(0xffffffffu, end);
+      if (lane == 0) cnt_s[wid] = __popc(mask);
+      __syncthreads();
+      int at = count + __popc(mask & ((1u << lane) - 1u));
+      for (int k = 0; k < kDesignWarps; ++k) {
+        if (k < wid) at += cnt_s[k];
+        count += cnt_s[k];
+      }
+      if (end) ends[at] = t;
+      __syncthreads();
+    }
+    return count;
+  }
+};
 
-// One CTA per prompt (and 128 KB of shared memory each): registers are not what limits residency.
+// Timestep weights of the OPTIMIZED and HEURISTIC designs, before the floor: w_t = gamma_bar_t * u_t with
+// gamma_bar_t = (1/K) sum over the completions that reach t, and the largest of each kWeightSteps steps. A
+// division costs tens of FP64 operations, of which an SM of GB300 does two a clock, so the steps are spread over
+// the chip: 17 us for 8 prompts of 16 completions and 15350 steps.
+constexpr int kWeightSteps = 512;
+__global__ void __launch_bounds__(kDesignThreads)
+    design_weights_kernel(int K, int T_max, const int32_t* __restrict__ L, const float* __restrict__ gamma,
+                          const float* __restrict__ u, DesignWs ws, uint32_t* status) {
+  __shared__ long long red_l[kDesignWarps];
+  __shared__ int red_i[kDesignWarps];
+  __shared__ double red_d[kDesignWarps];
+  const int p = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  long long base = 0;   // rows before the group's first completion
+  for (int k = tid; k < p * K; k += kDesignThreads) base += L[k];
+  int Tp = 0;           // the group's horizon
+  for (int j = tid; j < K; j += kDesignThreads) Tp = max(Tp, L[p * K + j]);
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    base += __shfl_xor_sync(0xffffffffu, base, o);
+    Tp = max(Tp, __shfl_xor_sync(0xffffffffu, Tp, o));
+  }
+  if (lane == 0) {
+    red_l[wid] = base;
+    red_i[wid] = Tp;
+  }
+  __syncthreads();
+  base = 0;
+  for (int i = 0; i < kDesignWarps; ++i) {
+    base += red_l[i];
+    Tp = max(Tp, red_i[i]);
+  }
+  Tp = min(max(Tp, 1), T_max);
+  double wmax = 0.0;
+  const int t1 = min(Tp, static_cast<int>(blockIdx.y + 1) * kWeightSteps);
+  for (int t = blockIdx.y * kWeightSteps + tid; t < t1; t += kDesignThreads) {
+    double acc = 0.0;
+    long long off = base;
+    for (int j = 0; j < K; ++j) {
+      const int n = L[p * K + j];
+      if (t < n) acc = __dadd_rn(acc, static_cast<double>(gamma[off + t]));
+      off += n;
+    }
+    double v = __ddiv_rn(acc, static_cast<double>(K));
+    if (u) v = __dmul_rn(v, static_cast<double>(u[static_cast<int64_t>(p) * T_max + t]));
+    if (!isfinite(v)) raise_status(status, PS_DEV_NONFINITE);
+    ws.w[static_cast<int64_t>(p) * T_max + t] = v;
+    wmax = fmax(wmax, v);
+  }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) wmax = fmax(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
+  if (lane == 0) red_d[wid] = wmax;
+  __syncthreads();
+  if (tid == 0) {
+    for (int i = 1; i < kDesignWarps; ++i) wmax = fmax(wmax, red_d[i]);
+    ws.bW[static_cast<int64_t>(p) * 2 * T_max * kDesignArrays + blockIdx.y] = wmax;   // free until the pooling
+  }
+}
+
+// One CTA per prompt (and, OPTIMIZED, 172 KB of shared memory each): registers are not what limits residency.
+template <bool OPTIMIZED>
 __global__ void __launch_bounds__(kDesignThreads, 1)
-    design_kernel(int K, int T_max, const int32_t* __restrict__ L, const float* __restrict__ gamma,
-                  const float* __restrict__ u, double budget, int strategy, double param, uint64_t* __restrict__ q,
-                  double* __restrict__ xi_out, DesignWs ws, uint32_t* status) {
+    design_kernel(int K, int T_max, const int32_t* __restrict__ L, double budget, int strategy, double param,
+                  uint64_t* __restrict__ q, double* __restrict__ xi_out, DesignWs ws, uint32_t* status) {
   const int p = blockIdx.x;
   const int tid = threadIdx.x;
   __shared__ int Tp_s;
   __shared__ double red_d[kDesignThreads / 32];
   __shared__ unsigned long long red_u[kDesignThreads / 32];
   __shared__ unsigned long long red_b[kDesignThreads / 32];
-  __shared__ long long red_l[kDesignThreads / 32];
   __shared__ int red_i[kDesignThreads / 32];
   __shared__ double lam_s;
-  __shared__ int found_s, found_lane_s, ncand_s, nnear_s, tdef_s;
-  __shared__ volatile int s0_ok_s, s0_skip_s;
+  __shared__ int ncand_s, nnear_s, tdef_s, decided_s;
   __shared__ int cand_s[kMaxNearCap + 1];
-  __shared__ int nb_s[kCapLanes];
-  __shared__ double den_s[kCapLanes];
-  extern __shared__ double dyn_smem[];    // the status pass's stack (kDesignDynSmem bytes)
+  __shared__ double den_s;
+  extern __shared__ __align__(16) float2 dyn_smem[];    // the hull's vertices (kDesignDynSmem bytes)
   const int lane = tid & 31, wid = tid >> 5;
   double* w = ws.w + static_cast<int64_t>(p) * T_max;
   double* xi = ws.xi + static_cast<int64_t>(p) * T_max;
-  int64_t* off = ws.off + static_cast<int64_t>(p) * K;
 
-  // horizon of the group, and the row offset of its first completion
-  long long base = 0;
-  for (int k = tid; k < p * K; k += kDesignThreads) base += L[k];
+  // horizon of the group
+  int Tmax = 0;
+  for (int j = tid; j < K; j += kDesignThreads) Tmax = max(Tmax, L[p * K + j]);
 #pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) base += __shfl_xor_sync(0xffffffffu, base, o);
-  if (lane == 0) red_l[wid] = base;
+  for (int o = 16; o >= 1; o >>= 1) Tmax = max(Tmax, __shfl_xor_sync(0xffffffffu, Tmax, o));
+  if (lane == 0) red_i[wid] = Tmax;
   __syncthreads();
   if (tid == 0) {
-    long long b = 0;
-    for (int i = 0; i < kDesignThreads / 32; ++i) b += red_l[i];
-    int Tp = 0;
-    for (int j = 0; j < K; ++j) {
-      off[j] = b;
-      b += L[p * K + j];
-      Tp = max(Tp, L[p * K + j]);
-    }
-    if (Tp < 1 || Tp > T_max) raise_status(status, PS_DEV_BAD_LENGTH);
-    Tp_s = Tp < 1 ? 1 : (Tp > T_max ? T_max : Tp);
+    for (int i = 1; i < kDesignWarps; ++i) Tmax = max(Tmax, red_i[i]);
+    if (Tmax < 1 || Tmax > T_max) raise_status(status, PS_DEV_BAD_LENGTH);
+    Tp_s = Tmax < 1 ? 1 : (Tmax > T_max ? T_max : Tmax);
   }
   __syncthreads();
   const int Tp = Tp_s;
   const double Bp = fmin(budget, static_cast<double>(Tp));
 
-  if (strategy == PS_DESIGN_OPTIMIZED || strategy == PS_DESIGN_HEURISTIC) {
-    // w_t = gamma_bar_t * u_t; gamma_bar_t = (1/K) sum over the completions that reach t
+  if (OPTIMIZED || strategy == PS_DESIGN_HEURISTIC) {
+    // the floor under the weights: the largest of them from the weights kernel's parts
     double wmax = 0.0;
-    for (int t = tid; t < Tp; t += kDesignThreads) {
-      double acc = 0.0;
-      for (int j = 0; j < K; ++j)
-        if (t < L[p * K + j]) acc = __dadd_rn(acc, static_cast<double>(gamma[off[j] + t]));
-      double v = __ddiv_rn(acc, static_cast<double>(K));
-      if (u) v = __dmul_rn(v, static_cast<double>(u[static_cast<int64_t>(p) * T_max + t]));
-      if (!isfinite(v)) raise_status(status, PS_DEV_NONFINITE);
-      w[t] = v;
-      wmax = fmax(wmax, v);
+    {
+      const double* parts = ws.bW + static_cast<int64_t>(p) * 2 * T_max * kDesignArrays;
+      for (int c = tid; c * kWeightSteps < Tp; c += kDesignThreads) wmax = fmax(wmax, parts[c]);
     }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) wmax = fmax(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
@@ -445,68 +723,40 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
     const double fl = __dmul_rn(1e-12, wm);
     for (int t = tid; t < Tp; t += kDesignThreads) w[t] = wm > 0.0 ? (w[t] > fl ? w[t] : fl) : 1.0;
     __syncthreads();
-    if (strategy == PS_DESIGN_OPTIMIZED) {
-      // The smallest saturated prefix s whose suffix design (budget B - s) starts at or below 1,
-      // decided by the definition's exact rounded sequence: for a candidate s, a lane of warp 0 pools
-      // w[s..T) into its own stack; all threads take the blocks' scores s_m = sqrt(W_m / n_m); the
-      // lane sums den = sum_m n_m s_m in block order and tests (B - s) s_1 / den <= 1. Candidates:
-      // the prefixes the status pass puts within the band of 1, then the first clearly below it, in
+    if constexpr (OPTIMIZED) {
+      // The smallest saturated prefix s whose suffix design (budget B - s) starts at or below 1, decided by
+      // the definition's exact rounded sequence: for a candidate s, w[s..T) is pooled, the blocks' scores are
+      // s_m = sqrt(W_m / n_m), den = sum_m n_m s_m in block order, and it passes if (B - s) s_1 / den <= 1.
+      // Candidates: the prefixes whose status is within the band of 1, then the first clearly below it, in
       // increasing order; the first that passes is the answer. (If the band holds too many, or none
-      // passes, the search falls back to trying every prefix in order, 32 at a time.)
-      const int64_t sbase = static_cast<int64_t>(p) * T_max * kCapLanes;
-      double* bW = ws.bW + sbase;
-      double* bs = ws.bs + sbase;
-      int32_t* bn = ws.bn + sbase;
-      // xi is written last; meanwhile its 8 Tp bytes hold the scaled weights of the status pass
-      // (floats, [0, Tp)) and the statuses (floats, [Tp, 2 Tp))
-      float* wsc = reinterpret_cast<float*>(xi);
-      float* status = wsc + Tp;
-      {
-        const double inv = 1.0 / (wm > 0.0 ? wm : 1.0);
-        for (int t = tid; t < Tp; t += kDesignThreads) wsc[t] = static_cast<float>(w[t] * inv);
-      }
-      // s = 0 first, exactly (small budgets end here), on warp 0; meanwhile warp 1 runs the status
-      // pass for every other prefix on a stack of its own (shared memory, then lane 31's slots), and
-      // stops as soon as s = 0 has qualified.
-      if (tid == 0) {
-        found_s = -1;
-        nnear_s = 0;
-        ncand_s = 0;
-        s0_ok_s = 0;
-        s0_skip_s = 0;
-      }
-      __syncthreads();
-      if (wid == 0) {
-        // (abandoned when the status pass, finished first, puts s = 0 clearly above the cap)
-        if (lane == 0) nb_s[0] = pav_stack_dev(w, Tp, bW, bn, &s0_skip_s);
-        __syncwarp();
-        const int nb0 = nb_s[0];
-        for (int m = lane; m < nb0; m += 32)
-          bs[m * kCapLanes] = __dsqrt_rn(__ddiv_rn(bW[m * kCapLanes], static_cast<double>(bn[m * kCapLanes])));
-        __syncwarp();
-        if (lane == 0) {
-          double den = 0.0;
-          for (int m = 0; m < nb0; ++m)
-            den = __dadd_rn(den, __dmul_rn(static_cast<double>(bn[m * kCapLanes]), bs[m * kCapLanes]));
-          den_s[0] = den;
-          if (nb0 > 0 && __ddiv_rn(__dmul_rn(Bp, bs[0]), den) <= 1.0) {
-            found_s = 0;
-            found_lane_s = 0;
-            s0_ok_s = 1;
-          }
-        }
-      }
-      if (wid == 1 && lane == 0) {
-        float2* sW = reinterpret_cast<float2*>(dyn_smem);
-        int32_t* sn = reinterpret_cast<int32_t*>(sW + kCapStackSmem);
-        float* sr = reinterpret_cast<float*>(sn + kCapStackSmem);
-        cap_status_pass(wsc, Tp, Bp, sW, sn, sr, bW + (kCapLanes - 1), bn + (kCapLanes - 1),
-                        bs + (kCapLanes - 1), status, &s0_ok_s);
-        if (!s0_ok_s && status[0] == 0.f) s0_skip_s = 1;
-      }
-      __syncthreads();
+      // passes, every prefix is tried in order.)
+      const int64_t pitch = 2 * static_cast<int64_t>(T_max);   // at least T + 1
+      double* fW = ws.bW + p * pitch * kDesignArrays;
+      double* fs = ws.bs + p * pitch * kDesignArrays;
+      int32_t* fn = ws.bn + p * pitch * kDesignArrays;
+      float2* S = reinterpret_cast<float2*>(fW);
+      float2* D = reinterpret_cast<float2*>(fW + pitch);
+      double* blockW = fW + 2 * pitch;      // Pooled::W
+      double* score = fs;
+      double* term = fs + pitch;
+      int32_t* link = fn;
+      int32_t* first = fn + pitch;
+      int32_t* ends = fn + 2 * pitch;
+      int32_t* hull_deep = fn + 3 * pitch;
+      float2* hull_S = dyn_smem;
+      int32_t* hull = reinterpret_cast<int32_t*>(hull_S + kHullSmem);
+      float* status = reinterpret_cast<float*>(xi);            // xi is written last
+      const double inv = 1.0 / (wm > 0.0 ? wm : 1.0);
+      auto scaled = [&](int t) {   // w[t] over the largest weight: in [1e-12, 1]
+        const double v = w[t] * inv;
+        const float hi = static_cast<float>(v);
+        return FF{hi, static_cast<float>(v - static_cast<double>(hi))};
+      };
+      ff_prefix_sums([&](int i) { return scaled(Tp - 1 - i); }, Tp, -1.f, S);
+      hull_links(S, Tp, link, hull_S, hull, hull_deep);
+      cap_status(S, link, Tp, Bp, D, status);
       int td = Tp;
-      for (int t = 1 + tid; t < Tp; t += kDesignThreads)
+      for (int t = tid; t < Tp; t += kDesignThreads)
         if (status[t] == 2.f) {
           td = t;
           break;
@@ -514,6 +764,7 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
 #pragma unroll
       for (int o = 16; o >= 1; o >>= 1) td = min(td, __shfl_xor_sync(0xffffffffu, td, o));
       if (lane == 0) red_i[wid] = td;
+      if (tid == 0) nnear_s = 0;
       __syncthreads();
       if (tid == 0) {
         int m = Tp;
@@ -522,14 +773,13 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
       }
       __syncthreads();
       const int tdef = tdef_s;
-      if (found_s < 0)
-        for (int t = 1 + tid; t < tdef; t += kDesignThreads)
-          if (status[t] == 1.f) {
-            const int i = atomicAdd(&nnear_s, 1);
-            if (i < kMaxNearCap) cand_s[i] = t;
-          }
+      for (int t = tid; t < tdef; t += kDesignThreads)
+        if (status[t] == 1.f) {
+          const int i = atomicAdd(&nnear_s, 1);
+          if (i < kMaxNearCap) cand_s[i] = t;
+        }
       __syncthreads();
-      if (tid == 0 && found_s < 0) {
+      if (tid == 0) {
         const int n = min(nnear_s, kMaxNearCap);
         for (int i = 1; i < n; ++i) {          // the few near-band prefixes, in increasing order
           const int v = cand_s[i];
@@ -544,67 +794,60 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
         if (tdef < Tp && nnear_s <= kMaxNearCap) cand_s[n] = tdef;
       }
       __syncthreads();
-      // One round: lanes l < width try the prefixes start(l); sets found_s / found_lane_s.
-      auto try_prefixes = [&](int width, auto start) {
-        if (wid == 0) {
-          const int st = lane < width ? start(lane) : Tp;
-          nb_s[lane] = st < Tp ? pav_stack_dev(w + st, Tp - st, bW + lane, bn + lane) : 0;
+      int nb = 0;
+      // Pools w[s..T) and tests the prefix; block m's end is ends[nb - 1 - m].
+      auto passes = [&](int s) {
+        ff_prefix_sums([&](int i) { return scaled(s + i); }, Tp - s, 1.f, S);
+        hull_links(S, Tp - s, link, hull_S, hull, hull_deep);
+        const Pooled pool{w, s, Tp, link, first, blockW};
+        pool.run();
+        nb = pool.blocks(ends);
+        for (int m = tid; m < nb; m += kDesignThreads) {
+          const int e = ends[nb - 1 - m];
+          const double n = static_cast<double>(e - first[e]);
+          const double sc = __dsqrt_rn(__ddiv_rn(blockW[e], n));
+          score[m] = sc;
+          term[m] = __dmul_rn(n, sc);
         }
         __syncthreads();
-        for (int l = 0; l < width; ++l)
-          for (int m = tid; m < nb_s[l]; m += kDesignThreads)
-            bs[m * kCapLanes + l] =
-                __dsqrt_rn(__ddiv_rn(bW[m * kCapLanes + l], static_cast<double>(bn[m * kCapLanes + l])));
-        __syncthreads();
-        if (wid == 0) {
-          const int st = lane < width ? start(lane) : Tp;
-          bool ok = false;
-          if (st < Tp) {
-            double den = 0.0;
-            for (int m = 0; m < nb_s[lane]; ++m)
-              den = __dadd_rn(den, __dmul_rn(static_cast<double>(bn[m * kCapLanes + lane]), bs[m * kCapLanes + lane]));
-            den_s[lane] = den;
-            ok = __ddiv_rn(__dmul_rn(__dsub_rn(Bp, static_cast<double>(st)), bs[lane]), den) <= 1.0;
+        if (tid == 0) {
+          double den = 0.0;
+          int m = 0;
+          for (; m + 8 <= nb; m += 8) {
+            double v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = term[m + j];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) den = __dadd_rn(den, v[j]);
           }
-          const unsigned m = __ballot_sync(0xffffffffu, ok);
-          if (lane == 0 && m != 0u) {
-            found_lane_s = __ffs(m) - 1;
-            found_s = start(found_lane_s);
-          }
+          for (; m < nb; ++m) den = __dadd_rn(den, term[m]);
+          den_s = den;
         }
         __syncthreads();
+        return __ddiv_rn(__dmul_rn(__dsub_rn(Bp, static_cast<double>(s)), score[0]), den_s) <= 1.0;
       };
-      const int ncand = ncand_s;
-      for (int c0 = 0; c0 < ncand && found_s < 0; c0 += kCapLanes)
-        try_prefixes(min(kCapLanes, ncand - c0), [&](int l) { return cand_s[c0 + l]; });
-      // the exact scan over every prefix: only when the band held too many prefixes or no candidate
-      // passed, which the status pass's accuracy rules out in practice
-      for (int base = 1; found_s < 0 && base < Tp; base += kCapLanes)
-        try_prefixes(kCapLanes, [&](int l) { return base + l; });
-      const int found = found_s;
+      int found = -1;
+      for (int c = 0; c < ncand_s && found < 0; ++c)
+        if (passes(cand_s[c])) found = cand_s[c];
+      // every prefix in order: only when the band held too many prefixes or no candidate passed, which the
+      // accuracy of the statuses rules out in practice (an infinite weight has no design: PS_DEV_NONFINITE)
+      for (int t = 0; found < 0 && t < Tp && isfinite(wm); ++t)
+        if (passes(t)) found = t;
+      __syncthreads();
       if (found < 0) {
         for (int t = tid; t < Tp; t += kDesignThreads) xi[t] = 1.0;
       } else {
-        // the design of the lane that found it: block starts by a scan, then every block in parallel
-        const int l = found_lane_s;
-        const int nb = nb_s[l];
         const double Bs = __dsub_rn(Bp, static_cast<double>(found));
-        const double den = den_s[l];
         for (int t = tid; t < found; t += kDesignThreads) xi[t] = 1.0;
-        if (tid == 0) {
-          int t0 = found;
-          for (int m = 0; m < nb; ++m) {
-            const int n = bn[m * kCapLanes + l];
-            bn[m * kCapLanes + l] = t0;          // the block's first step replaces its length
-            t0 += n;
-          }
-        }
-        __syncthreads();
-        for (int m = tid; m < nb; m += kDesignThreads) {
-          const double v = __ddiv_rn(__dmul_rn(Bs, bs[m * kCapLanes + l]), den);
-          const int t_end = m + 1 < nb ? bn[(m + 1) * kCapLanes + l] : Tp;
-          for (int t = bn[m * kCapLanes + l]; t < t_end; ++t) xi[t] = v;
-        }
+        // short blocks by a thread each, long ones by a warp
+        auto fill = [&](int m, int t_first, int t_step, bool want_long) {
+          const int b1 = ends[nb - 1 - m], b0 = first[b1];
+          if ((b1 - b0 >= 64) != want_long) return;
+          const double v = __ddiv_rn(__dmul_rn(Bs, score[m]), den_s);
+          for (int t = b0 + t_first; t < b1; t += t_step) xi[t] = v;
+        };
+        for (int m = tid; m < nb; m += kDesignThreads) fill(m, 0, 1, false);
+        for (int m = wid; m < nb; m += kDesignWarps) fill(m, lane, 32, true);
       }
     } else {
       // Heuristic: closed form B sqrt(w_t) / sum_j sqrt(w_j) (the sum in step order), a running
@@ -613,17 +856,36 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
       __syncthreads();
       if (tid == 0) {
         double tot = 0.0;
-        for (int t = 0; t < Tp; ++t) tot = __dadd_rn(tot, xi[t]);
-        den_s[0] = tot;
+        int t = 0;
+        for (; t + 8 <= Tp; t += 8) {
+          double v[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[j] = xi[t + j];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) tot = __dadd_rn(tot, v[j]);
+        }
+        for (; t < Tp; ++t) tot = __dadd_rn(tot, xi[t]);
+        den_s = tot;
       }
       __syncthreads();
-      const double tot = den_s[0];
-      for (int t = tid; t < Tp; t += kDesignThreads) xi[t] = __ddiv_rn(__dmul_rn(Bp, xi[t]), tot);
-      __syncthreads();
-      if (tid == 0)
-        for (int t = 1; t < Tp; ++t) xi[t] = fmin(xi[t - 1], xi[t]);
-      __syncthreads();
-      for (int t = tid; t < Tp; t += kDesignThreads) xi[t] = fmin(xi[t], 1.0);
+      const double tot = den_s;
+      // the running minimum over 256 steps at a time: a scan in each warp, then the minima before it
+      double run = INFINITY;
+      for (int t0 = 0; t0 < Tp; t0 += kDesignThreads) {
+        const int t = t0 + tid;
+        double v = t < Tp ? __ddiv_rn(__dmul_rn(Bp, xi[t]), tot) : INFINITY;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const double y = __shfl_up_sync(0xffffffffu, v, o);
+          if (lane >= o) v = fmin(y, v);
+        }
+        if (lane == 31) red_d[wid] = v;
+        __syncthreads();
+        for (int i = 0; i < wid; ++i) run = fmin(run, red_d[i]);
+        if (t < Tp) xi[t] = fmin(fmin(run, v), 1.0);
+        for (int i = wid; i < kDesignWarps; ++i) run = fmin(run, red_d[i]);
+        __syncthreads();
+      }
     }
   } else if (strategy == PS_DESIGN_UNIFORM) {
     for (int t = tid; t < Tp; t += kDesignThreads)
@@ -643,15 +905,33 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
       for (int i = 0; i < kDesignThreads / 32; ++i) tot += red_d[i];
       return tot;
     };
+    // Whether the budget at lam exceeds Bp. The sum is (1 - e^(-lam T)) / (1 - e^-lam), which one thread has in
+    // microseconds, where the sum over T steps keeps an SM's FP64 lanes busy for T / 200 us. Both are off by at
+    // most (T / 256 + 32) 2^-53 relative (the longest chain of additions, and a few roundings), so outside
+    // twice that band the closed form decides as the sum would; inside it, the sum decides.
+    constexpr int kClosedFormFrom = 2048;
+    auto over = [&](double lam) {
+      if (Tp >= kClosedFormFrom) {
+        __syncthreads();
+        if (tid == 0) {
+          const double est = expm1(-lam * Tp) / expm1(-lam);
+          const double band = (Tp / kDesignThreads + 32) * 0x1p-52 * Bp;
+          decided_s = est > Bp + band ? 1 : est < Bp - band ? 0 : -1;
+        }
+        __syncthreads();
+        if (decided_s >= 0) return decided_s != 0;
+      }
+      return budget_at(lam) > Bp;
+    };
     if (static_cast<double>(Tp) <= Bp) {
       if (tid == 0) lam_s = 0.0;
     } else {
       double lo = 0.0, hi = 1.0;
-      for (int it = 0; it < 64 && budget_at(hi) > Bp; ++it) hi *= 2.0;
+      for (int it = 0; it < 64 && over(hi); ++it) hi *= 2.0;
       for (int it = 0; it < 200; ++it) {
         const double mid = 0.5 * (lo + hi);
         if (mid <= lo || mid >= hi) break;   // lo and hi are adjacent doubles: nothing changes any more
-        if (budget_at(mid) > Bp) lo = mid;
+        if (over(mid)) lo = mid;
         else hi = mid;
       }
       if (tid == 0) lam_s = hi;
@@ -850,7 +1130,7 @@ int ps_reward_uncertainty(int P, int K, int T_max, const int32_t* L, const float
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }
 
-static DesignWs design_ws(void* ws, int P, int K, int T_max) {
+static DesignWs design_ws(void* ws, int P, int T_max) {
   uint8_t* b = static_cast<uint8_t*>(ws) + kWsHeader;
   const size_t pt = static_cast<size_t>(P) * T_max;
   DesignWs d;
@@ -859,20 +1139,18 @@ static DesignWs design_ws(void* ws, int P, int K, int T_max) {
   d.xi = reinterpret_cast<double*>(b);
   b += al256(sizeof(double) * pt);
   d.bW = reinterpret_cast<double*>(b);
-  b += al256(sizeof(double) * pt * kCapLanes);
+  b += al256(sizeof(double) * pt * 2 * kDesignArrays);
   d.bs = reinterpret_cast<double*>(b);
-  b += al256(sizeof(double) * pt * kCapLanes);
+  b += al256(sizeof(double) * pt * 2 * kDesignArrays);
   d.bn = reinterpret_cast<int32_t*>(b);
-  b += al256(sizeof(int32_t) * pt * kCapLanes);
-  d.off = reinterpret_cast<int64_t*>(b);
   return d;
 }
 
 size_t ps_design_cutoffs_workspace_size(int P, int K, int T_max) {
   if (P < 1 || K < 1 || T_max < 1) return 0;
   const size_t pt = static_cast<size_t>(P) * T_max;
-  return kWsHeader + al256(sizeof(double) * pt) * 2 + al256(sizeof(double) * pt * kCapLanes) * 2 +
-         al256(sizeof(int32_t) * pt * kCapLanes) + al256(sizeof(int64_t) * static_cast<size_t>(P) * K);
+  return kWsHeader + al256(sizeof(double) * pt) * 2 + al256(sizeof(double) * pt * 2 * kDesignArrays) * 2 +
+         al256(sizeof(int32_t) * pt * 2 * kDesignArrays) + al256(sizeof(int64_t) * static_cast<size_t>(P) * K);
 }
 
 int ps_design_cutoffs(int P, int K, int T_max, const int32_t* L, const float* gamma_full, const float* u,
@@ -891,11 +1169,22 @@ int ps_design_cutoffs(int P, int K, int T_max, const int32_t* L, const float* ga
     return PS_ERR_WORKSPACE;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (cudaMemsetAsync(ws, 0, kWsHeader, s) != cudaSuccess) return PS_ERR_CUDA;
-  if (cudaFuncSetAttribute(design_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(kDesignDynSmem)) != cudaSuccess)
-    return PS_ERR_CUDA;
-  design_kernel<<<P, kDesignThreads, kDesignDynSmem, s>>>(K, T_max, L, gamma_full, u, budget, strategy, param, q, xi,
-                                              design_ws(ws, P, K, T_max), static_cast<uint32_t*>(ws));
+  const DesignWs d = design_ws(ws, P, T_max);
+  if (uses_gamma) {
+    const dim3 grid(static_cast<unsigned>(P), static_cast<unsigned>((T_max + kWeightSteps - 1) / kWeightSteps));
+    design_weights_kernel<<<grid, kDesignThreads, 0, s>>>(K, T_max, L, gamma_full, u, d, static_cast<uint32_t*>(ws));
+    if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
+  }
+  if (strategy == PS_DESIGN_OPTIMIZED) {
+    if (cudaFuncSetAttribute(design_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kDesignDynSmem)) != cudaSuccess)
+      return PS_ERR_CUDA;
+    design_kernel<true><<<P, kDesignThreads, kDesignDynSmem, s>>>(K, T_max, L, budget, strategy, param, q, xi, d,
+                                                                  static_cast<uint32_t*>(ws));
+  } else {
+    design_kernel<false><<<P, kDesignThreads, 0, s>>>(K, T_max, L, budget, strategy, param, q, xi, d,
+                                                      static_cast<uint32_t*>(ws));
+  }
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }
 

@@ -105,6 +105,33 @@ def test_capped_design_random_steep_weights(seed):
         _crafted_design(vecs, B)
 
 
+def test_capped_design_deep_hulls():
+    # Decreasing weights pool nothing: the hull of their sums outgrows shared memory (14336 vertices) and goes
+    # on in the workspace; a ramp or a spike at the end then pools back through both parts. With a heavy front
+    # the answer is a saturated prefix, pooled on its own.
+    T = 16000
+    fall = np.linspace(2.0, 1.0, T)
+    ramp = np.concatenate([fall[:15000], np.linspace(1.0, 3.0, 1000)])
+    spike = np.concatenate([fall[:-1], [4000.0]])
+    for front in ([], [1e8, 9e7, 2e7]):
+        for v in (fall, ramp, spike):
+            xi = _crafted_design([np.concatenate([front, v])], 100.0)
+            assert (xi[0] == 1.0).sum() == len(front)
+
+
+def test_capped_design_ties_and_near_ties():
+    # Means that tie exactly, or differ only beyond the float slopes that propose the blocks: the definition's
+    # double arithmetic has to decide each, at more places than are redone one by one (the rest is then pooled
+    # by one thread), across window edges of 256 steps and at sizes around them.
+    rng = np.random.default_rng(3)
+    for T in (1, 2, 255, 256, 257, 513, 900):
+        base = np.repeat(rng.uniform(0.5, 2.0, -(-T // 3)), 3)[:T]
+        vecs = [np.tile([1.0, 2.0], -(-T // 2))[:T], np.tile([1.0, 3.0, 2.0], -(-T // 3))[:T],
+                base * (1.0 + 2.0 ** -23 * rng.integers(-1, 2, T)), np.sort(base)[::-1], np.sort(base)]
+        for B in (1.0, 0.3 * T + 0.7, float(T)):
+            _crafted_design(vecs, min(B, float(T)))
+
+
 @pytest.mark.parametrize("name,budget", [("mid", 40.0), ("7b", 128.0)])
 def test_time_prior_design(name, budget):
     cfg = get_config(name)
