@@ -47,9 +47,14 @@ static uint32_t* ticket_word(void* ws) { return static_cast<uint32_t*>(ws) + 1; 
 constexpr uint64_t kCutoffKeyTag = 0x5053505030303031ull;  // "PSPP0001"
 
 // ================================================================== K1: cutoff sampler
-// One CTA per prompt. Saturating block scan of the masses gives U[h]; S[t] = 2^62 - U[t-1];
-// the thread that owns h decides every completion whose draw x lies in [U[h-1], U[h]).
-constexpr int kSampThreads = 1024;
+// Saturating scans of the masses give U[h]; S[t] = 2^62 - U[t-1]; the thread that owns bucket h decides every
+// completion whose draw x lies in [U[h-1], U[h]).
+// A prompt's steps are shared by blockIdx.y of the grid: what costs is a step's f64 division (an SM of GB300 does
+// two FP64 operations a clock), so one CTA per prompt took 81 us for 2 prompts x 16384 steps and 36 us for one of
+// 7220, against 14 and 8.4 us with 64 and 29 CTAs each. Every CTA adds up the whole row of masses itself
+// (integers, from L2) rather than wait for the CTAs before it; kSampMaxParts bounds that reading.
+constexpr int kSampThreads = 256;
+constexpr int kSampMaxParts = 64;
 constexpr uint64_t kSatCap = kOne62 + 1;   // any prefix above 2^62 is invalid; saturate just past it
 
 __device__ __forceinline__ uint64_t sat_add(uint64_t a, uint64_t b) {
@@ -62,56 +67,74 @@ __global__ void __launch_bounds__(kSampThreads)
                           uint64_t seed, uint64_t step, int64_t traj_base, int mode, int32_t* __restrict__ H,
                           int32_t* __restrict__ n, float* __restrict__ w_tab, uint32_t* status) {
   extern __shared__ uint64_t xs[];  // [K] draws
-  __shared__ uint64_t warp_tot[32];
-  __shared__ uint64_t carry_s, total_s;
+  constexpr int kWarps = kSampThreads / 32;
+  __shared__ uint64_t warp_tot[kWarps], warp_before[kWarps];
   const int p = blockIdx.x;
   const int tid = threadIdx.x;
+  const bool first_part = blockIdx.y == 0;
   const int64_t wrow = static_cast<int64_t>(p) * T_max;
+  // this CTA's steps [t_begin, t_end): whole tiles of kSampThreads
+  const int64_t tiles = (T_max + kSampThreads - 1) / kSampThreads;
+  const int t_begin = static_cast<int>(tiles * blockIdx.y / gridDim.y * kSampThreads);
+  const int t_end = min(T_max, static_cast<int>(tiles * (blockIdx.y + 1) / gridDim.y * kSampThreads));
 
   for (int j = tid; j < K; j += blockDim.x) {
     const int k = p * K + j;
-    const int Lk = L[k];
-    if (Lk < 1 || Lk > T_max) raise_status(status, PS_DEV_BAD_LENGTH);
-    if (mode == PS_MODE_FULL) {
-      H[k] = Lk;
-      n[k] = Lk;
-    } else {
-      H[k] = 0;
-      n[k] = 0;
+    if (first_part) {
+      const int Lk = L[k];
+      if (Lk < 1 || Lk > T_max) raise_status(status, PS_DEV_BAD_LENGTH);
+      if (mode == PS_MODE_FULL) {
+        H[k] = Lk;
+        n[k] = Lk;
+      }
+    }
+    if (mode != PS_MODE_FULL) {
       uint64_t c[4] = {static_cast<uint64_t>(traj_base + k), step, 0ull, 0ull};
       philox4x64_10(c, seed, kCutoffKeyTag);
       xs[j] = c[0] >> 2;
     }
   }
   if (mode == PS_MODE_FULL) {
-    for (int t = tid; t < T_max; t += blockDim.x) w_tab[wrow + t] = 1.0f;
+    for (int t = t_begin + tid; t < t_end; t += blockDim.x) w_tab[wrow + t] = 1.0f;
     return;
   }
   const int lane = tid & 31, wid = tid >> 5;
-  // Total mass U[T] (saturating). Exact mode requires 2^62; in the H = 0 mode the deficit
-  // 2^62 - U[T] is Pr(H = 0) and the survival is S[t] = U[T] - U[t-1].
-  {
-    uint64_t part = 0;
-    for (int t = tid; t < T_max; t += blockDim.x) {
-      const uint64_t m = q[wrow + t];
-      part = sat_add(part, m > kOne62 ? kSatCap : m);
-    }
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) part = sat_add(part, __shfl_xor_sync(0xffffffffu, part, o));
-    if (lane == 0) warp_tot[wid] = part;
-    __syncthreads();
-    if (tid == 0) {
-      uint64_t tot = 0;
-      for (int w = 0; w < kSampThreads / 32; ++w) tot = sat_add(tot, warp_tot[w]);
-      total_s = tot;
-      if (tot > kOne62 || (mode == PS_MODE_TRUNC && tot != kOne62)) raise_status(status, PS_DEV_BAD_PMF);
-    }
+  // Total mass U[T] and the mass before this CTA's steps (saturating). Exact mode requires U[T] = 2^62; in the
+  // H = 0 mode the deficit 2^62 - U[T] is Pr(H = 0) and the survival is S[t] = U[T] - U[t-1].
+  uint64_t part = 0, before = 0;
+#pragma unroll 4
+  for (int t = tid; t < T_max; t += kSampThreads) {
+    const uint64_t m = q[wrow + t];
+    part = sat_add(part, m > kOne62 ? kSatCap : m);
+    if (t < t_begin) before = part;   // (a tile lies on one side of t_begin)
   }
-  if (tid == 0) carry_s = 0;
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    part = sat_add(part, __shfl_xor_sync(0xffffffffu, part, o));
+    before = sat_add(before, __shfl_xor_sync(0xffffffffu, before, o));
+  }
+  if (lane == 0) {
+    warp_tot[wid] = part;
+    warp_before[wid] = before;
+  }
   __syncthreads();
-  const uint64_t total = total_s > kOne62 ? kOne62 : total_s;
+  uint64_t mass = 0, carry = 0;
+  for (int w = 0; w < kWarps; ++w) {
+    mass = sat_add(mass, warp_tot[w]);
+    carry = sat_add(carry, warp_before[w]);
+  }
+  if (first_part) {
+    if (tid == 0 && (mass > kOne62 || (mode == PS_MODE_TRUNC && mass != kOne62))) raise_status(status, PS_DEV_BAD_PMF);
+    for (int j = tid; j < K; j += blockDim.x)   // a draw at or above U[T]
+      if (xs[j] >= mass) {
+        H[p * K + j] = 0;
+        n[p * K + j] = 0;
+      }
+  }
+  const uint64_t total = mass > kOne62 ? kOne62 : mass;
 
-  for (int base = 0; base < T_max; base += kSampThreads) {
+  for (int base = t_begin; base < t_end; base += kSampThreads) {
+    __syncthreads();
     const int t = base + tid;  // 0-based: bucket h = t + 1
     uint64_t m = t < T_max ? q[wrow + t] : 0ull;
     if (m > kOne62) {
@@ -126,20 +149,14 @@ __global__ void __launch_bounds__(kSampThreads)
     }
     if (lane == 31) warp_tot[wid] = v;
     __syncthreads();
-    if (wid == 0) {
-      uint64_t w = warp_tot[lane];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint64_t y = __shfl_up_sync(0xffffffffu, w, o);
-        if (lane >= o) w = sat_add(w, y);
-      }
-      warp_tot[lane] = w;  // inclusive over warps
+    uint64_t prior = carry;          // up to this warp
+    for (int w = 0; w < kWarps; ++w) {
+      if (w < wid) prior = sat_add(prior, warp_tot[w]);
+      carry = sat_add(carry, warp_tot[w]);
     }
-    __syncthreads();
-    const uint64_t carry = carry_s;
-    const uint64_t before = wid > 0 ? warp_tot[wid - 1] : 0ull;
-    const uint64_t incl = sat_add(carry, sat_add(before, v));  // U[h]
-    const uint64_t excl = sat_add(carry, sat_add(before, v - m > kSatCap ? kSatCap : v - m));
+    const uint64_t incl = sat_add(prior, v);  // U[h]
+    const uint64_t left = __shfl_up_sync(0xffffffffu, v, 1);
+    const uint64_t excl = lane > 0 ? sat_add(prior, left) : prior;   // U[h-1]
     if (t < T_max) {
       // S[t+1] = U[T] - U[t]; weight 2^62 / S (f64 divide, rounded once to f32)
       float wt;
@@ -151,22 +168,19 @@ __global__ void __launch_bounds__(kSampThreads)
         wt = __double2float_rn(__ddiv_rn(4611686018427387904.0, S));
       }
       w_tab[wrow + t] = wt;
-      if (m > 0 && incl <= kOne62) {
+      if (m > 0) {
+        const bool valid = incl <= kOne62;   // a bucket past 2^62 (an invalid row) decides nothing
         for (int j = 0; j < K; ++j) {
           const uint64_t x = xs[j];
           if (x >= excl && x < incl) {
             const int k = p * K + j;
-            H[k] = t + 1;
-            n[k] = min(t + 1, L[k]);
+            H[k] = valid ? t + 1 : 0;
+            n[k] = valid ? min(t + 1, L[k]) : 0;
           }
         }
       }
     }
-    __syncthreads();
-    if (tid == kSampThreads - 1) carry_s = incl;
-    __syncthreads();
   }
-  // (the total was checked before the scan; a draw at or above U[T] leaves H = n = 0)
 }
 
 // ================================================================== K2: packing
@@ -187,82 +201,104 @@ static PackWs pack_ws(void* ws, int B) {
   return w;
 }
 
-// One CTA: scans of L and n, group advantages (sequential f64 sums per group, no FMA
-// contraction, so the result is the correctly rounded sequence of the stated operations).
-__global__ void __launch_bounds__(1024)
+// CTA 0: scans of L and n. The others: group advantages, a warp per prompt (sequential f64 sums per group, no FMA
+// contraction, so the result is the correctly rounded sequence of the stated operations; the divisions, one per
+// completion, by its lanes). Latency-bound: with one CTA that scanned through 20 barriers and a thread per prompt
+// that divided one completion after another it took 14.6 us for 2 prompts x 16, now 4.1.
+constexpr int kMetaThreads = 1024;
+constexpr int kAdvWarps = 4;   // per CTA: more would wait for each other's double operations
+__global__ void __launch_bounds__(kMetaThreads)
     pack_meta_kernel(int P, int K, int T_max, const int32_t* __restrict__ L, const int32_t* __restrict__ n,
                      const float* __restrict__ R, int adv_mode, int64_t capacity, int32_t* __restrict__ cu_seqlens,
                      PackWs w, uint32_t* status) {
+  constexpr int kWarps = kMetaThreads / 32;
   const int B = P * K;
-  __shared__ int64_t sl[1024], sn[1024];
-  __shared__ int64_t carry_l, carry_n;
-  if (threadIdx.x == 0) {
-    carry_l = 0;
-    carry_n = 0;
-  }
-  __syncthreads();
-  for (int base = 0; base < B; base += 1024) {
-    const int k = base + threadIdx.x;
-    int64_t lk = 0, nk = 0;
-    if (k < B) {
-      lk = L[k];
-      nk = n[k];
-      if (lk < 1 || lk > T_max || nk < 0 || nk > lk) {
-        raise_status(status, PS_DEV_BAD_LENGTH);
-        lk = lk < 0 ? 0 : lk;
-        nk = nk < 0 ? 0 : (nk > lk ? lk : nk);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (blockIdx.x == 0) {
+    __shared__ int64_t warp_l[kWarps], warp_n[kWarps];
+    int64_t carry_l = 0, carry_n = 0;
+    for (int base = 0; base < B; base += kMetaThreads) {
+      const int k = base + threadIdx.x;
+      int64_t lk = 0, nk = 0;
+      if (k < B) {
+        lk = L[k];
+        nk = n[k];
+        if (lk < 1 || lk > T_max || nk < 0 || nk > lk) {
+          raise_status(status, PS_DEV_BAD_LENGTH);
+          lk = lk < 0 ? 0 : lk;
+          nk = nk < 0 ? 0 : (nk > lk ? lk : nk);
+        }
       }
-    }
-    sl[threadIdx.x] = lk;
-    sn[threadIdx.x] = nk;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {  // Hillis-Steele inclusive scan
-      const int64_t al = threadIdx.x >= o ? sl[threadIdx.x - o] : 0;
-      const int64_t an = threadIdx.x >= o ? sn[threadIdx.x - o] : 0;
+      int64_t sl = lk, sn = nk;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int64_t yl = __shfl_up_sync(0xffffffffu, sl, o), yn = __shfl_up_sync(0xffffffffu, sn, o);
+        if (lane >= o) {
+          sl += yl;
+          sn += yn;
+        }
+      }
+      if (lane == 31) {
+        warp_l[wid] = sl;
+        warp_n[wid] = sn;
+      }
       __syncthreads();
-      sl[threadIdx.x] += al;
-      sn[threadIdx.x] += an;
+      // the warps' sums, scanned by every warp for itself
+      int64_t tl = warp_l[lane], tn = warp_n[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int64_t yl = __shfl_up_sync(0xffffffffu, tl, o), yn = __shfl_up_sync(0xffffffffu, tn, o);
+        if (lane >= o) {
+          tl += yl;
+          tn += yn;
+        }
+      }
+      const int64_t before_l = __shfl_sync(0xffffffffu, tl, wid - 1), before_n = __shfl_sync(0xffffffffu, tn, wid - 1);
+      if (wid > 0) {
+        sl += before_l;
+        sn += before_n;
+      }
+      if (k < B) {
+        w.off_L[k] = carry_l + sl - lk;
+        const int64_t cu = carry_n + sn - nk;
+        cu_seqlens[k] = static_cast<int32_t>(cu > INT32_MAX ? INT32_MAX : cu);
+      }
+      carry_l += __shfl_sync(0xffffffffu, tl, 31);
+      carry_n += __shfl_sync(0xffffffffu, tn, 31);
       __syncthreads();
     }
-    if (k < B) {
-      w.off_L[k] = carry_l + sl[threadIdx.x] - lk;
-      const int64_t cu = carry_n + sn[threadIdx.x] - nk;
-      cu_seqlens[k] = static_cast<int32_t>(cu > INT32_MAX ? INT32_MAX : cu);
+    if (threadIdx.x == 0) {
+      w.off_L[B] = carry_l;
+      int64_t N = carry_n;
+      if (N > capacity || N > INT32_MAX || carry_l > INT32_MAX) {
+        raise_status(status, PS_DEV_CAPACITY);
+        N = 0;  // write no rows
+      }
+      cu_seqlens[B] = static_cast<int32_t>(carry_n > INT32_MAX ? INT32_MAX : carry_n);
+      *w.N = N;
     }
-    __syncthreads();
-    if (threadIdx.x == 1023) {
-      carry_l += sl[1023];
-      carry_n += sn[1023];
-    }
-    __syncthreads();
+    return;
   }
-  if (threadIdx.x == 0) {
-    w.off_L[B] = carry_l;
-    int64_t N = carry_n;
-    if (N > capacity || N > INT32_MAX || carry_l > INT32_MAX) {
-      raise_status(status, PS_DEV_CAPACITY);
-      N = 0;  // write no rows
-    }
-    cu_seqlens[B] = static_cast<int32_t>(carry_n > INT32_MAX ? INT32_MAX : carry_n);
-    *w.N = N;
-  }
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
+  if (wid >= kAdvWarps) return;
+  const int warps = (gridDim.x - 1) * kAdvWarps;
+  for (int p = (blockIdx.x - 1) * kAdvWarps + wid; p < P; p += warps) {
+    const float* Rp = R + static_cast<int64_t>(p) * K;
+    double* Ap = w.A + static_cast<int64_t>(p) * K;
     double s = 0.0;
-    for (int j = 0; j < K; ++j) s = __dadd_rn(s, static_cast<double>(R[p * K + j]));
+    for (int j = 0; j < K; ++j) s = __dadd_rn(s, static_cast<double>(Rp[j]));
     const double mu = __ddiv_rn(s, static_cast<double>(K));
     if (adv_mode == PS_ADV_CENTERED) {
-      for (int j = 0; j < K; ++j) w.A[p * K + j] = __dsub_rn(static_cast<double>(R[p * K + j]), mu);
+      for (int j = lane; j < K; j += 32) Ap[j] = __dsub_rn(static_cast<double>(Rp[j]), mu);
       continue;
     }
     double ss = 0.0;
     for (int j = 0; j < K; ++j) {
-      const double dv = __dsub_rn(static_cast<double>(R[p * K + j]), mu);
+      const double dv = __dsub_rn(static_cast<double>(Rp[j]), mu);
       ss = __dadd_rn(ss, __dmul_rn(dv, dv));
     }
     const double sigma = __dsqrt_rn(__ddiv_rn(ss, static_cast<double>(K)));
     const double den = __dadd_rn(sigma, 1e-6);
-    for (int j = 0; j < K; ++j)
-      w.A[p * K + j] = __ddiv_rn(__dsub_rn(static_cast<double>(R[p * K + j]), mu), den);
+    for (int j = lane; j < K; j += 32) Ap[j] = __ddiv_rn(__dsub_rn(static_cast<double>(Rp[j]), mu), den);
   }
 }
 
@@ -625,7 +661,13 @@ int ps_sample_cutoffs(int P, int K, int T_max, const uint64_t* q, const int32_t*
   if (cudaFuncSetAttribute(sample_cutoffs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(smem)) != cudaSuccess)
     return PS_ERR_CUDA;
-  sample_cutoffs_kernel<<<P, kSampThreads, smem, s>>>(K, T_max, q, L, seed, step, traj_base, mode, H, n, w_tab,
+  // parts of a prompt: one per tile of steps while that leaves no more than two CTAs per SM
+  int64_t parts = (T_max + kSampThreads - 1) / kSampThreads;
+  const int64_t most = 2 * static_cast<int64_t>(num_sms_current()) / P;
+  if (parts > most) parts = most > 0 ? most : 1;
+  if (parts > kSampMaxParts) parts = kSampMaxParts;
+  const dim3 grid(static_cast<unsigned>(P), static_cast<unsigned>(parts));
+  sample_cutoffs_kernel<<<grid, kSampThreads, smem, s>>>(K, T_max, q, L, seed, step, traj_base, mode, H, n, w_tab,
                                                       status_word(ws));
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }
@@ -654,10 +696,13 @@ int ps_pack_prefixes(int P, int K, int T_max, int d, int dtype, const int32_t* L
   if (rc != PS_OK) return rc;
   const int B = P * K;
   PackWs pw = pack_ws(ws, B);
-  pack_meta_kernel<<<1, 1024, 0, s>>>(P, K, T_max, L, n, R, adv_mode, capacity, cu_seqlens, pw, status_word(ws));
+  const int sms = num_sms_current();
+  const int adv_ctas = P < kAdvWarps * sms ? (P + kAdvWarps - 1) / kAdvWarps : sms;
+  pack_meta_kernel<<<1 + adv_ctas, kMetaThreads, 0, s>>>(P, K, T_max, L, n, R, adv_mode, capacity, cu_seqlens, pw,
+                                                         status_word(ws));
   if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
   const int64_t row_vec = hid_full ? static_cast<int64_t>(d) * elem_size(dtype) / 16 : 0;
-  const int grid = num_sms_current() * 8;
+  const int grid = sms * 8;
   pack_rows_kernel<<<grid, kPackThreads, 0, s>>>(B, K, T_max, cu_seqlens, pw, w_tab, tok_full, oldlogp_full,
                                                  static_cast<const uint4*>(hid_full), row_vec, src_row, row_traj,
                                                  row_pos, tok, oldlogp, w, adv, static_cast<uint4*>(hid_packed));
