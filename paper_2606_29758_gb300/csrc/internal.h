@@ -34,10 +34,13 @@ int fwd_gemm_f32(int64_t N, int d, int V, const float* Hpk, const float* W, cons
 int proxy_gemm_bf16(int64_t N, int d, int V, const void* Hrows, const void* W, const int32_t* tok, float4* part,
                     float* ztok, int splits, uint32_t* status, cudaStream_t s);
 
-// Score proxy plus the 16 largest logits per row and vocabulary range (contiguous ranges, at most
-// 16): topk [splits][N][16] (logit, column bits).
+// Score proxy plus the 16 largest logits per row and list: part [lists][N], topk [lists][N][16] (logit,
+// column bits), lists = ranges x lists_per_range, `ranges` contiguous vocabulary ranges. A workspace of
+// `lists` lists takes proxy_topk_lists_bf16() per range.
+int proxy_topk_lists_bf16(int64_t N, int d, int lists);
 int proxy_topk_gemm_bf16(int64_t N, int d, int V, const void* Hrows, const void* W, const int32_t* tok,
-                         float4* part, float2* topk, float* ztok, int splits, uint32_t* status, cudaStream_t s);
+                         float4* part, float2* topk, float* ztok, int ranges, int lists_per_range, uint32_t* status,
+                         cudaStream_t s);
 
 // Backward for one chunk of rows [0, rc) of already offset pointers: recompute dZ into
 // dz ([rc][ldz], operand dtype), then dH = dZ W and dW (+)= dZ^T Hpk. With tok_base, W holds

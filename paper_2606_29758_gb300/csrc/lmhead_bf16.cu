@@ -240,9 +240,11 @@ struct FwdProxyEpi {
 // FwdProxyEpi plus the 16 largest logits of the unit's vocabulary range (Appendix I: u_t uses
 // the top 16 next tokens). The list stays sorted (descending, lower column first on ties) in
 // registers; only the values of a 32-column slice above the current 16th value are inserted.
+// With 8 epilogue warps a row has two lists per range, one per column group.
 constexpr int kTopK = 16;
+template <int EPI_WARPS>
 struct FwdProxyTopkEpi {
-  static constexpr int kEpiWarps = 4;
+  static constexpr int kEpiWarps = EPI_WARPS;
   static constexpr bool kTmaStore = false;
   static constexpr int kStageBytes = 0;
   struct Params {
@@ -284,9 +286,10 @@ struct FwdProxyTopkEpi {
       float x = pick32(r, j);
       if (!(x > st.v[kTopK - 1])) continue;   // the threshold rose since the mask was taken
       int c = col0 + j;
+      bool take = false;   // from its place on, every entry moves down one (an equal one too: it came first)
 #pragma unroll
       for (int i = 0; i < kTopK; ++i) {
-        const bool take = x > st.v[i];
+        take = take || x > st.v[i];
         const float tv = st.v[i];
         const int ti = st.id[i];
         st.v[i] = take ? x : tv;
@@ -850,17 +853,34 @@ int proxy_gemm_bf16(int64_t N, int d, int V, const void* Hrows, const void* W, c
   return launch_gemm_single<false, false, FwdProxyEpi, 2>(ta, tb, ta, N, V, d, splits, band, ep, status, s);
 }
 
-int proxy_topk_gemm_bf16(int64_t N, int d, int V, const void* Hrows, const void* W, const int32_t* tok,
-                         float4* part, float2* topk, float* ztok, int splits, uint32_t* status, cudaStream_t s) {
+// The top-16 epilogue is long (per row and tile some 2500 instructions on 4 warps), and it hides under the next
+// tile's MMAs only from about d = 1300 on: below, 8 warps with two lists per range are faster though the workspace's
+// 16 lists then make half as many ranges, as long as those still give every SM a unit. Score proxy, 4 warps and 16
+// ranges / 8 warps and 8: 21840 rows, d = 512, V = 151936 4297 / 3281 us; d = 1024, V = 32000 1513 / 1309; d = 1536,
+// V = 151936 6266 / 6805. (256 x 256 tiles with 8 warps: 4615, 1788 and 7976 us.)
+int proxy_topk_lists_bf16(int64_t N, int d, int lists) {
+  return d < 1280 && lists >= 2 && (N + kBM - 1) / kBM * (lists / 2) >= num_sms_current() ? 2 : 1;
+}
+
+template <int EPI_WARPS>
+static int proxy_topk_gemm(int64_t N, int d, int V, const void* Hrows, const void* W, const int32_t* tok, float4* part,
+                           float2* topk, float* ztok, int ranges, uint32_t* status, cudaStream_t s) {
   CUtensorMap ta, tb;
   if (!map_kmajor(&ta, Hrows, N, d, d, kBM) || !map_kmajor(&tb, W, V, d, d, kBRowsBox)) return PS_ERR_INVALID_ARG;
-  FwdProxyTopkEpi::Params ep{tok, static_cast<int>(N), V, part, topk, ztok};
+  typename FwdProxyTopkEpi<EPI_WARPS>::Params ep{tok, static_cast<int>(N), V, part, topk, ztok};
   // Units are contiguous vocabulary ranges; a band of row blocks whose rows fill the forward's L2
   // share walks them range by range, so W is read from DRAM about once per band.
   const int workers = num_sms_current();
   int band = static_cast<int>(kFwdBandL2Bytes / (static_cast<double>(kBM) * d * 2.0));
-  if (band < (workers + splits - 1) / splits) band = (workers + splits - 1) / splits;
-  return launch_gemm_single<false, false, FwdProxyTopkEpi, 1>(ta, tb, ta, N, V, d, splits, band, ep, status, s);
+  if (band < (workers + ranges - 1) / ranges) band = (workers + ranges - 1) / ranges;
+  return launch_gemm_single<false, false, FwdProxyTopkEpi<EPI_WARPS>, 1>(ta, tb, ta, N, V, d, ranges, band, ep, status,
+                                                                         s);
+}
+int proxy_topk_gemm_bf16(int64_t N, int d, int V, const void* Hrows, const void* W, const int32_t* tok,
+                         float4* part, float2* topk, float* ztok, int ranges, int lists_per_range, uint32_t* status,
+                         cudaStream_t s) {
+  return lists_per_range == 2 ? proxy_topk_gemm<8>(N, d, V, Hrows, W, tok, part, topk, ztok, ranges, status, s)
+                              : proxy_topk_gemm<4>(N, d, V, Hrows, W, tok, part, topk, ztok, ranges, status, s);
 }
 
 int bwd_chunk_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, const int32_t* tok,

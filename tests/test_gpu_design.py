@@ -429,3 +429,34 @@ def test_proxy_and_top16_at_full_size(name):
     zk = np.sort(z, axis=1)[:, ::-1]
     clear = (zk[:, k - 1] - zk[:, k]) > 1e-3
     assert np.array_equal(np.sort(gi[clear], axis=1), np.sort(ridx[clear], axis=1))
+
+
+@pytest.mark.parametrize("N,d,V,k", [(2600, 64, 5000, 16), (5200, 1272, 2049, 16), (9800, 128, 600, 5)])
+def test_topk_of_two_column_groups_orders_equal_logits_by_column(N, d, V, k):
+    # Many rows of a narrow head: a row's top tokens come as two lists per vocabulary range, which interleave
+    # columns. Every fourth of the head's rows repeats, so logits are equal in exact fours across lists, ranges
+    # and tiles: the lower columns come first. Probabilities against float64 softmax (the tolerance of the other
+    # proxy tests); rows whose distinct logits come within 1e-4 may order them either way and are left out.
+    from paper_2606_29758_gb300 import _binding as B
+    g = torch.Generator(device="cuda").manual_seed(N + V)
+    base = -(-V // 4)
+    W = torch.randn(base, d, device="cuda", generator=g).bfloat16().repeat(4, 1)[:V].contiguous()
+    H = (torch.randn(N, d, device="cuda", generator=g) * d ** -0.5 * 2).bfloat16()
+    tok = torch.randint(0, V, (N,), device="cuda", generator=g, dtype=torch.int32)
+    gamma, logp = torch.empty(N, device="cuda"), torch.empty(N, device="cuda")
+    idx = torch.full((N, k), -7, dtype=torch.int32, device="cuda")
+    prob = torch.empty(N, k, device="cuda")
+    ws = torch.empty(B.ps_lmhead_score_proxy_workspace_size(N, d, V, B.PS_DTYPE_BF16, k), dtype=torch.uint8,
+                     device="cuda")
+    B.ps_lmhead_score_proxy(N, d, V, B.PS_DTYPE_BF16, H, W, tok, gamma, logp, ws, k, idx, prob)
+    assert B.ps_workspace_status(ws)[0] == B.PS_OK
+    z = H.double() @ W.double().t()
+    ref_v, ref_i = torch.sort(z, dim=1, descending=True, stable=True)
+    gap = ref_v[:, :-1] - ref_v[:, 1:]
+    clear = ((gap[:, :k] == 0) | (gap[:, :k] > 1e-4)).all(1)
+    assert clear.float().mean() > 0.5
+    assert torch.equal(idx[clear].long(), ref_i[clear, :k])
+    p = torch.exp(ref_v[:, :k] - torch.logsumexp(z, 1, keepdim=True))
+    assert ((prob.double() - p).abs() <= 2e-4 * p).all()
+    lp = z.gather(1, tok[:, None].long())[:, 0] - torch.logsumexp(z, 1)
+    assert ((logp.double() - lp).abs() <= 1e-4 * lp.abs() + 2e-4).all()
