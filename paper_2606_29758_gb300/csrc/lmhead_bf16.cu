@@ -681,29 +681,41 @@ static int splitk_clusters_at_once(int ranks) {
   return n;
 }
 
-// Ranks per output tile (1: the persistent kernel) of a product with `tiles` output tiles and num_kb
-// k-blocks: the fewest rounds of (k-blocks per rank + the exchange). dH of a few rows has few tiles and
-// the vocabulary as its K loop. Measured, one CTA per tile against 2 / 4 / 8 ranks (us):
+// Ranks per output tile (1: the persistent kernel) and the tile's height for an M x N product of num_kb k-blocks: the
+// fewest rounds of (k-blocks per rank + the exchange), in hundredths of a wide tile's k-block (0.55 us). dH of a few
+// rows has few tiles and the vocabulary as its K loop. Measured, one CTA per tile against 2 / 4 / 8 ranks (us):
 //   d = 3584, V = 152064: 185 rows (14 tiles) 1353 / 688 / 363 / 217; 400 (28) 1332 / 676 / 357 / 412;
 //     1000 (56) 1326 / 660 / 710 / 832; 2048 (112) 1297 / 1342 / 1408 / 1668; 3000 (168) 2639 / 2010 /
 //     1770 / 2503; 4000 (224) 2631 / 1999 / 2482 / 3169.
-//   d = 392, V = 2000: 185 rows (2) 22.9 / 18.5 / 14.7 / 12.3; 4000 (32) 27.0 / 23.3 / 20.2 / 41.9.
-// Over 54 such sizes the rule picked the fastest of the four or one within 3% of it, but for one (600 rows,
-// d = 3584, V = 32000: 172 us with 8 ranks, 158 with 2). From two
-// tiles per SM on the persistent kernel's last round costs less than a third, and the split is off, so
-// that whole batches and their shards (hundreds of tiles each) add dH up in the same order.
-constexpr int kSplitOverheadKb = 12;   // the exchange and the launch, in k-blocks of a wide tile (0.55 us each)
-static int choose_splitk(int64_t tiles, int num_kb) {
-  if (tiles >= 2 * num_sms_current()) return 1;
-  auto cost = [&](int S) {
-    const int64_t at_once = S == 1 ? num_sms_current() : splitk_clusters_at_once(S);
-    return (tiles + at_once - 1) / at_once * ((num_kb + S - 1) / S + (S > 1 ? kSplitOverheadKb : 0));
-  };
-  int best = 1;
-  for (int S = 2; S <= 8 && S <= num_kb; S *= 2)
-    if (cost(S) * 100 < cost(best) * 97) best = S;
+//   d = 392, V = 2000: 185 rows (2) 22.9 / 18.5 / 14.7 / 12.3; 4000 (32) 27.0 / 23.3 / 20.2 / 41.9. 571 rows
+//     with 8 ranks take 17.6 us on wide tiles and 11.4 on 128-row ones, which exchange one half each.
+// Over 54 such sizes on wide tiles the rule picked the fastest of the four or one within 3% of it, but for one (600
+// rows, d = 3584, V = 32000: 172 us with 8 ranks, 158 with 2). From two wide tiles per SM on the persistent kernel's
+// last round costs less than a third, and the split is off, so that whole batches and their shards (hundreds of
+// tiles each) add dH up in the same order.
+struct SplitK {
+  int ranks, halves;
+};
+static SplitK choose_splitk(int64_t M, int64_t N, int num_kb) {
+  const int sms = num_sms_current();
+  const int64_t nb = (N + kBN - 1) / kBN;
+  const int64_t tiles[3] = {0, (M + kBM - 1) / kBM * nb, (M + 2 * kBM - 1) / (2 * kBM) * nb};
+  SplitK best{1, 2};
+  if (tiles[2] >= 2 * sms) return best;
+  int64_t best_cost = (tiles[2] + sms - 1) / sms * num_kb * 100;
+  for (int halves = 2; halves >= 1; --halves)
+    for (int S = 2; S <= 8 && S <= num_kb; S *= 2) {
+      const int64_t at_once = splitk_clusters_at_once(S);
+      const int64_t c = (tiles[halves] + at_once - 1) / at_once *
+                        ((num_kb + S - 1) / S * (halves == 2 ? 100 : 54) + (halves == 2 ? 1200 : 700));
+      if (c * 100 < best_cost * 97) {
+        best = SplitK{S, halves};
+        best_cost = c;
+      }
+    }
   return best;
 }
+
 template <bool A_MN, bool B_MN, int HALVES>
 static int launch_gemm_splitk(const CUtensorMap& ta, const CUtensorMap& tb, int64_t M, int64_t N, int64_t K, int ranks,
                               const SplitOut& o, uint32_t* status, cudaStream_t s) {
@@ -759,16 +771,35 @@ static int choose_splits(int64_t m_blocks, int64_t n_blocks, int workers, int mi
 // 256-row B tile. (The CTA-pair kernel, reached only through the GEMM test hook, has each CTA
 // load half of it, 128 rows; see gemm_bf16.)
 constexpr uint32_t kBRowsBox = kBN;
-// Tile height of the logit recompute in 128-row halves (see GemmCfg). The wide tile moves a third
-// fewer operand bytes per FLOP (about 0.8 vs 0.95 pJ per FLOP at the power cap) but does not overlap
-// its epilogue with the next tile; with dZ stored through TMA it is the faster of the two (7B-shaped
-// backward 381.4 vs 382.8 ms, and 387.7 ms with per-thread stores of 128-row tiles, back to back).
-constexpr int kRecHalves = 2;
-// The forward's (and score proxy's) tile height depends on the hidden size: its K loop is d long,
-// while the epilogue of a wide tile overlaps the next tile only in part (one TMEM half at a time).
-// Measured back to back with the current epilogue: at d = 1536 the wide tile is 3% faster (56.5 vs
-// 58.2 ms per 191k-row forward); below d = 1024 the K loop is short enough to keep 128-row tiles.
+// Tile height in 128-row halves (see GemmCfg) of a GEMM whose units are M x N tiles. The wide tile moves a third
+// fewer operand bytes per FLOP (about 0.8 vs 0.95 pJ per FLOP at the power cap) and takes 1.8-1.95 times as long as
+// a 128 x 256 one, so it is the faster of the two unless the narrow one needs clearly fewer than twice its rounds
+// over the SMs: when few rows leave its last row block half empty, or few tiles its last round. limit: the most
+// narrow rounds per 10 wide ones. Measured, narrow / wide (us):
+//   logits recomputed, limit 18: 60 rows, d = 3584, V = 152064 (4 rounds / 4) 174 / 198; 571 rows, d = 512, V =
+//     151936 (20 / 12) 88 / 98; 571 rows, d = 392, V = 2000 (1 / 1) 14.2 / 17.2; 200 rows, d = 3584 (8 / 4) 224 / 203
+//   forward, limit 18: 60 rows, d = 1536, V = 151936 (4 / 4) 95 / 108; 1200 rows, d = 1024, V = 32000 (9 / 5) 72 / 74;
+//     20000 rows, d = 128, V = 9000 (38 / 19) 105 / 89; 3000 rows, d = 768, V = 32000 (20 / 10) 115 / 108
+//   forward from d = 2048 on, limit 16: 571 rows, d = 3584 with a store (20 / 12) 495 / 490
+//   dW, limit 17: 571 rows, d = 392, V = 2000 (1 / 1) 11.7 / 14.5; 20000 rows, d = 128, V = 9000 (1 / 1) 118 / 190; 1200
+//     rows, d = 768, V = 32000 (5 / 3) 59 / 63; 8000 rows, d = 1024, V = 32000 (7 / 4) 338 / 325
+static int tile_halves(int64_t M, int64_t N, int limit) {
+  const int64_t sms = num_sms_current(), nb = (N + kBN - 1) / kBN;
+  const int64_t narrow = ((M + kBM - 1) / kBM * nb + sms - 1) / sms;
+  const int64_t wide = ((M + 2 * kBM - 1) / (2 * kBM) * nb + sms - 1) / sms;
+  return narrow * 10 <= wide * limit ? 1 : 2;
+}
+
+// The forward's tile height. With fewer partials than vocabulary tiles (and for the score proxy), units are
+// ranges of tiles and the height depends on the hidden size, the K loop: below d = 1024 it is short enough to keep
+// 128-row tiles. A storing forward of at most 3 k-blocks keeps them too: its wide epilogue takes longer than they do
+// (20000 rows, d = 128, V = 9000: 149 us on narrow tiles, 162 on wide ones).
 static int fwd_halves(int d) { return d < 1024 ? 1 : 2; }
+static int fwd_halves(int64_t N, int d, int V, int splits, bool store) {
+  if (splits != fwd_tile_splits_bf16(V)) return fwd_halves(d);
+  if (store && d <= 3 * kBK) return 1;
+  return tile_halves(N, V, d < 2048 ? 18 : 16);
+}
 
 // The forward keeps one band of row blocks in flight; every CTA re-reads its row block for
 // every vocabulary tile, so the band's hidden rows must stay in L2 (129 MB) next to the W
@@ -776,8 +807,8 @@ static int fwd_halves(int d) { return d < 1024 ? 1 : 2; }
 // forward than 20 MB or 43 MB, and 64-86 MB were slower still).
 constexpr double kFwdBandL2Bytes = 30e6;
 
-static int fwd_band_max(int d) {
-  const double block_bytes = static_cast<double>(kBM * fwd_halves(d)) * d * 2.0;
+static int fwd_band_max(int d, int halves) {
+  const double block_bytes = static_cast<double>(kBM * halves) * d * 2.0;
   const int b = static_cast<int>(kFwdBandL2Bytes / block_bytes);
   return b < 1 ? 1 : b;
 }
@@ -790,20 +821,21 @@ int choose_fwd_splits_bf16(int64_t N, int d, int V, int num_sms, int max_splits)
   const int nb = fwd_tile_splits_bf16(V);
   if (max_splits >= nb) return nb;
   const int rows = kBM * fwd_halves(d);
-  int lo = (num_sms + fwd_band_max(d) - 1) / fwd_band_max(d);
+  const int band = fwd_band_max(d, fwd_halves(d));
+  int lo = (num_sms + band - 1) / band;
   if (lo > max_splits) lo = max_splits;
   return choose_splits((N + rows - 1) / rows, nb, num_sms, lo, max_splits);
 }
 
 int fwd_gemm_bf16(int64_t N, int d, int V, const void* Hpk, const void* W, const int32_t* tok, float2* part,
                   float* ztok, int splits, uint32_t* status, cudaStream_t s, int tok_base) {
-  const int halves = fwd_halves(d);
+  const int halves = fwd_halves(N, d, V, splits, false);
   CUtensorMap ta, tb;
   if (!map_kmajor(&ta, Hpk, N, d, d, kBM * halves) || !map_kmajor(&tb, W, V, d, d, kBRowsBox))
     return PS_ERR_INVALID_ARG;
   FwdLseEpi::Params ep{tok, static_cast<int>(N), V, part, ztok, tok_base};
   const int workers = num_sms_current();
-  const int band = splits == fwd_tile_splits_bf16(V) ? fwd_band_max(d) : (workers + splits - 1) / splits;
+  const int band = splits == fwd_tile_splits_bf16(V) ? fwd_band_max(d, halves) : (workers + splits - 1) / splits;
   if (halves == 1)
     return launch_gemm_single<false, false, FwdLseEpi, 1>(ta, tb, ta, N, V, d, splits, band, ep, status, s);
   return launch_gemm_single<false, false, FwdLseEpi, 2>(ta, tb, ta, N, V, d, splits, band, ep, status, s);
@@ -817,14 +849,14 @@ int fwd_gemm_bf16(int64_t N, int d, int V, const void* Hpk, const void* W, const
 int fwd_gemm_store_bf16(int64_t N, int d, int V, const void* Hpk, const void* W, const int32_t* tok, float2* part,
                         float* ztok, int splits, void* store, int64_t ldz, float* scale, uint32_t* status,
                         cudaStream_t s, int tok_base) {
-  const int halves = fwd_halves(d);
+  const int halves = fwd_halves(N, d, V, splits, true);
   CUtensorMap ta, tb, tc;
   if (!map_kmajor(&ta, Hpk, N, d, d, kBM * halves) || !map_kmajor(&tb, W, V, d, d, kBRowsBox)) return PS_ERR_INVALID_ARG;
   if (!make_map(&tc, store, V, N, ldz * 2, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_DATA_TYPE_FLOAT16))
     return PS_ERR_INVALID_ARG;
   FwdLseStoreEpi::Params ep{tok, static_cast<int>(N), V, part, ztok, scale, N, tok_base};
   const int workers = num_sms_current();
-  const int band = splits == fwd_tile_splits_bf16(V) ? fwd_band_max(d) : (workers + splits - 1) / splits;
+  const int band = splits == fwd_tile_splits_bf16(V) ? fwd_band_max(d, halves) : (workers + splits - 1) / splits;
   if (halves == 1)
     return launch_gemm_single<false, false, FwdLseStoreEpi, 1>(ta, tb, tc, N, V, d, splits, band, ep, status, s);
   return launch_gemm_single<false, false, FwdLseStoreEpi, 2>(ta, tb, tc, N, V, d, splits, band, ep, status, s);
@@ -847,7 +879,7 @@ int proxy_gemm_bf16(int64_t N, int d, int V, const void* Hrows, const void* W, c
     return PS_ERR_INVALID_ARG;
   FwdProxyEpi::Params ep{tok, static_cast<int>(N), V, part, ztok};
   const int workers = num_sms_current();
-  const int band = splits == fwd_tile_splits_bf16(V) ? fwd_band_max(d) : (workers + splits - 1) / splits;
+  const int band = splits == fwd_tile_splits_bf16(V) ? fwd_band_max(d, halves) : (workers + splits - 1) / splits;
   if (halves == 1)
     return launch_gemm_single<false, false, FwdProxyEpi, 1>(ta, tb, ta, N, V, d, splits, band, ep, status, s);
   return launch_gemm_single<false, false, FwdProxyEpi, 2>(ta, tb, ta, N, V, d, splits, band, ep, status, s);
@@ -889,14 +921,17 @@ int bwd_chunk_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, con
   int rcode;
   {
     CUtensorMap ta, tb;
-    if (!map_kmajor(&ta, Hpk, rc, d, d, kBM * kRecHalves) || !map_kmajor(&tb, W, V, d, d, kBRowsBox))
+    const int halves = tile_halves(rc, V, 18);
+    if (!map_kmajor(&ta, Hpk, rc, d, d, kBM * halves) || !map_kmajor(&tb, W, V, d, d, kBRowsBox))
       return PS_ERR_INVALID_ARG;
     // dZ [rc][ldz] bf16, written in 32 x 32 boxes from 64-byte-swizzled staging
     CUtensorMap tz;
     if (!make_map(&tz, dz, V, rc, ldz * 2, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B)) return PS_ERR_INVALID_ARG;
     BwdDzEpi::Params ep{tok, lse, coef, static_cast<int>(rc), V, tok_base};
-    rcode = launch_gemm_single<false, false, BwdDzEpi, kRecHalves>(ta, tb, tz, rc, V, d, 0,
-                                                                    kBandRecompute / kRecHalves, ep, status, s);
+    if (halves == 1)
+      rcode = launch_gemm_single<false, false, BwdDzEpi, 1>(ta, tb, tz, rc, V, d, 0, kBandRecompute, ep, status, s);
+    else
+      rcode = launch_gemm_single<false, false, BwdDzEpi, 2>(ta, tb, tz, rc, V, d, 0, kBandRecompute / 2, ep, status, s);
     if (rcode != PS_OK) return rcode;
   }
   return bwd_grads_bf16(rc, d, V, Hpk, W, dH, dW, dw_accumulate, dz, ldz, status, s, dh_accumulate, n_call);
@@ -913,15 +948,14 @@ int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, flo
     if (!map_kmajor(&ta, dz, rc, V, ldz, 2 * kBM) || !map_mnmajor(&tb, W, V, d, d) || !map_out_f32(&tc, dH, rc, d, d))
       return PS_ERR_INVALID_ARG;
     StoreF32Epi::Params ep{d, dh_accumulate};
-    const int64_t tiles = ((n_call + 2 * kBM - 1) / (2 * kBM)) * ((d + kBN - 1) / kBN);
-    const int ranks = choose_splitk(tiles, (V + kBK - 1) / kBK);
-    if (ranks > 1) {
+    const SplitK split = choose_splitk(n_call, d, (V + kBK - 1) / kBK);
+    if (split.ranks > 1) {
       const SplitOut o{dH, d, static_cast<int>(rc), d, dh_accumulate};
-      if (rc > kBM) {
-        rcode = launch_gemm_splitk<false, true, 2>(ta, tb, rc, d, V, ranks, o, status, s);
-      } else {   // one 128-row half holds every row
+      if (split.halves == 2) {
+        rcode = launch_gemm_splitk<false, true, 2>(ta, tb, rc, d, V, split.ranks, o, status, s);
+      } else {
         if (!map_kmajor(&ta, dz, rc, V, ldz, kBM)) return PS_ERR_INVALID_ARG;
-        rcode = launch_gemm_splitk<false, true, 1>(ta, tb, rc, d, V, ranks, o, status, s);
+        rcode = launch_gemm_splitk<false, true, 1>(ta, tb, rc, d, V, split.ranks, o, status, s);
       }
     } else
       rcode = launch_gemm_single<false, true, StoreF32Epi, 2>(ta, tb, tc, rc, d, V, 0, kBandGrad, ep, status, s);
@@ -932,7 +966,14 @@ int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, flo
     if (!map_mnmajor(&ta, dz, rc, V, ldz) || !map_mnmajor(&tb, Hpk, rc, d, d) || !map_out_f32(&tc, dW, V, d, d))
       return PS_ERR_INVALID_ARG;
     StoreF32Epi::Params ep{d, dw_accumulate};
-    rcode = launch_gemm_single<true, true, StoreF32Epi, 2>(ta, tb, tc, V, d, rc, 0, kBandGrad, ep, status, s);
+    // dW of 65 to 256 rows (2 to 4 k-blocks) is bound by its stores, which the narrow tile's epilogue overlaps whole
+    // with the next tile (200 rows, V = 152064: d = 3584 407 us narrow / 443 wide, d = 1536 183 / 200; 571 rows
+    // 610 / 592).
+    const int kb = static_cast<int>((rc + kBK - 1) / kBK);
+    if ((kb >= 2 && kb <= 4) || tile_halves(V, d, 17) == 1)
+      rcode = launch_gemm_single<true, true, StoreF32Epi, 1>(ta, tb, tc, V, d, rc, 0, 2 * kBandGrad, ep, status, s);
+    else
+      rcode = launch_gemm_single<true, true, StoreF32Epi, 2>(ta, tb, tc, V, d, rc, 0, kBandGrad, ep, status, s);
     if (rcode != PS_OK) return rcode;
   }
   return PS_OK;
