@@ -29,7 +29,8 @@ static size_t al256(size_t x) { return (x + 255) / 256 * 256; }
 
 // ================================================================== score proxy
 __global__ void row_sqnorm_kernel(int64_t N, int d, int is_bf16, const void* __restrict__ H,
-                                  float* __restrict__ out) {
+                                  float* __restrict__ out, uint32_t* status) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) clear_status(status);   // the call's first kernel
   const int lane = threadIdx.x & 31;
   const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < N; i += warps) {
@@ -253,8 +254,10 @@ __global__ void __launch_bounds__(kUncWarps * 32)
 }
 
 // One warp: exclusive scan of L.
-__global__ void group_offsets_kernel(int B, const int32_t* __restrict__ L, int64_t* __restrict__ off) {
+__global__ void group_offsets_kernel(int B, const int32_t* __restrict__ L, int64_t* __restrict__ off,
+                                     uint32_t* status) {
   const int lane = threadIdx.x;
+  if (lane == 0) clear_status(status);   // the call's first kernel
   int64_t carry = 0;
   for (int k0 = 0; k0 < B; k0 += 32) {
     const int64_t n = k0 + lane < B ? L[k0 + lane] : 0;
@@ -1132,15 +1135,14 @@ int ps_lmhead_score_proxy(int64_t N, int d, int V, int dtype, const void* Hrows,
   }
   if (ws_bytes < fixed) return PS_ERR_WORKSPACE;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(ws, 0, kWsHeader, s) != cudaSuccess) return PS_ERR_CUDA;
-  if (N == 0) return PS_OK;
+  if (N == 0) return cudaMemsetAsync(ws, 0, kWsHeader, s) == cudaSuccess ? PS_OK : PS_ERR_CUDA;
   uint8_t* base = static_cast<uint8_t*>(ws);
   float* ztok = reinterpret_cast<float*>(base + kWsHeader);
   float* hn = reinterpret_cast<float*>(base + kWsHeader + al256(sizeof(float) * N));
   float4* part = reinterpret_cast<float4*>(base + fixed);
   float2* tpart = reinterpret_cast<float2*>(base + fixed + sizeof(float4) * static_cast<size_t>(S) * N);
   uint32_t* status = static_cast<uint32_t*>(ws);
-  row_sqnorm_kernel<<<num_sms_current() * 8, 256, 0, s>>>(N, d, 1, Hrows, hn);
+  row_sqnorm_kernel<<<num_sms_current() * 8, 256, 0, s>>>(N, d, 1, Hrows, hn, status);
   if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
   // With the top-k lists, as many vocabulary ranges as the workspace holds (up to 16): shorter
   // ranges keep the CTAs of a band closer together along W (16 ranges measured 4% faster than
@@ -1184,9 +1186,8 @@ int ps_reward_uncertainty(int P, int K, int T_max, const int32_t* L, const float
       ws_bytes < ps_reward_uncertainty_workspace_size(P, K))
     return PS_ERR_WORKSPACE;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(ws, 0, kWsHeader, s) != cudaSuccess) return PS_ERR_CUDA;
   int64_t* off = reinterpret_cast<int64_t*>(static_cast<uint8_t*>(ws) + kWsHeader);
-  group_offsets_kernel<<<1, 32, 0, s>>>(P * K, L, off);
+  group_offsets_kernel<<<1, 32, 0, s>>>(P * K, L, off, static_cast<uint32_t*>(ws));
   if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
   const size_t smem = (sizeof(int32_t) + sizeof(double)) * kUncWarps * unc_entries(K, topk);
   if (cudaFuncSetAttribute(uncertainty_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

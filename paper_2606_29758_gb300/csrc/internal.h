@@ -46,10 +46,11 @@ int proxy_topk_gemm_bf16(int64_t N, int d, int V, const void* Hrows, const void*
 // dz ([rc][ldz], operand dtype), then dH = dZ W and dW (+)= dZ^T Hpk. With tok_base, W holds
 // vocabulary rows [tok_base, tok_base + V) and the one-hot term applies where tok - tok_base is in [0, V);
 // dh_accumulate adds dH to what the buffer holds. n_call: rows of the whole call, which decide how dH's K
-// loop is split over CTAs, so that dH does not depend on the chunking.
+// loop is split over CTAs, so that dH does not depend on the chunking. clear: the call's first chunk, whose first
+// kernel zeroes the status (the forwards' GEMMs and dz_from_store always do).
 int bwd_chunk_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, const int32_t* tok,
                    const float* lse, const float* coef, float* dH, float* dW, int dw_accumulate, void* dz,
-                   int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call);
+                   int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, bool clear);
 // dH = dZ W and dW (+)= dZ^T Hpk from dZ [rc][ldz] bf16 already in memory.
 int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, float* dH, float* dW, int dw_accumulate,
                    const void* dz, int64_t ldz, uint32_t* status, cudaStream_t s, int dh_accumulate, int64_t n_call);
@@ -58,11 +59,11 @@ int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, flo
 // tok_base, the store holds vocabulary columns [tok_base, tok_base + V) and the one-hot term applies
 // where tok - tok_base is in [0, V).
 int dz_from_store_bf16(int64_t N, int V, void* store, int64_t ldz, const float* scale, int64_t lds,
-                       const int32_t* tok, const float* lse, const float* logp, const float* coef, cudaStream_t s,
-                       int tok_base = 0);
+                       const int32_t* tok, const float* lse, const float* logp, const float* coef, uint32_t* status,
+                       cudaStream_t s, int tok_base = 0);
 int bwd_chunk_f32(int64_t rc, int d, int V, const float* Hpk, const float* W, const int32_t* tok,
                   const float* lse, const float* coef, float* dH, float* dW, int dw_accumulate, float* dz,
-                  int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call);
+                  int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, bool clear);
 
 // Plain tensor-core GEMM (test hook): C[M][N] (+)= sum_k A(m,k) B(k,n), f32 out. variant: 0 one
 // CTA per 128 x 256 tile, 1 a CTA pair per 256 x 256 tile, 2 one CTA per 256 x 256 tile.

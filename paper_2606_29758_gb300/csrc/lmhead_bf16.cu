@@ -469,7 +469,8 @@ __global__ void __launch_bounds__(kDzThreads) dz_from_store_kernel(int64_t N, in
                                                                    const float* scale, int64_t lds,
                                                                    const int32_t* tok, int tok_base,
                                                                    const float* lse, const float* logp,
-                                                                   const float* coef) {
+                                                                   const float* coef, uint32_t* status) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) clear_status(status);   // the call's first kernel
   __shared__ float f_s[kDzCols / 32][kDzRows];   // -coef 2^(m - lse log2 e) per slice and row
   __shared__ float one_s[kDzRows];               // coef (1 - p_o)
   __shared__ int tok_s[kDzRows];
@@ -584,8 +585,9 @@ static bool map_mnmajor(CUtensorMap* m, const void* base, int64_t K, int64_t MN,
 template <bool A_MN, bool B_MN, class Epi, int HALVES = 1>
 static int launch_gemm_single(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, int64_t M,
                               int64_t N, int64_t K, int splits, int band_m, const typename Epi::Params& ep,
-                              uint32_t* status, cudaStream_t s) {
+                              uint32_t* status, cudaStream_t s, bool clear = false) {
   Sched sc;
+  sc.clear = clear ? 1 : 0;
   sc.m_blocks = static_cast<int>((M + kBM * HALVES - 1) / (kBM * HALVES));
   sc.n_blocks = static_cast<int>((N + kBN - 1) / kBN);
   sc.splits = splits > 0 ? splits : sc.n_blocks;
@@ -632,6 +634,7 @@ static int launch_gemm_pair(const CUtensorMap& ta, const CUtensorMap& tb, int64_
                             int splits, int band_m, const typename Epi::Params& ep, uint32_t* status,
                             cudaStream_t s) {
   Sched sc;
+  sc.clear = 0;
   sc.m_blocks = static_cast<int>((M + 255) / 256);
   sc.n_blocks = static_cast<int>((N + kBN - 1) / kBN);
   sc.splits = splits > 0 ? splits : sc.n_blocks;
@@ -837,8 +840,10 @@ int fwd_gemm_bf16(int64_t N, int d, int V, const void* Hpk, const void* W, const
   const int workers = num_sms_current();
   const int band = splits == fwd_tile_splits_bf16(V) ? fwd_band_max(d, halves) : (workers + splits - 1) / splits;
   if (halves == 1)
-    return launch_gemm_single<false, false, FwdLseEpi, 1>(ta, tb, ta, N, V, d, splits, band, ep, status, s);
-  return launch_gemm_single<false, false, FwdLseEpi, 2>(ta, tb, ta, N, V, d, splits, band, ep, status, s);
+    return launch_gemm_single<false, false, FwdLseEpi, 1>(ta, tb, ta, N, V, d, splits, band, ep, status, s,
+                                                              true);
+  return launch_gemm_single<false, false, FwdLseEpi, 2>(ta, tb, ta, N, V, d, splits, band, ep, status, s,
+                                                              true);
 }
 
 // The forward that keeps its logits: f16 e [N][ldz] through TMA (32 x 32 boxes from 64-byte-swizzled
@@ -858,8 +863,10 @@ int fwd_gemm_store_bf16(int64_t N, int d, int V, const void* Hpk, const void* W,
   const int workers = num_sms_current();
   const int band = splits == fwd_tile_splits_bf16(V) ? fwd_band_max(d, halves) : (workers + splits - 1) / splits;
   if (halves == 1)
-    return launch_gemm_single<false, false, FwdLseStoreEpi, 1>(ta, tb, tc, N, V, d, splits, band, ep, status, s);
-  return launch_gemm_single<false, false, FwdLseStoreEpi, 2>(ta, tb, tc, N, V, d, splits, band, ep, status, s);
+    return launch_gemm_single<false, false, FwdLseStoreEpi, 1>(ta, tb, tc, N, V, d, splits, band, ep, status, s,
+                                                              true);
+  return launch_gemm_single<false, false, FwdLseStoreEpi, 2>(ta, tb, tc, N, V, d, splits, band, ep, status, s,
+                                                              true);
 }
 
 // Bands (row blocks walked together) of the backward GEMMs. Recompute: 32 row blocks of 128 rows
@@ -917,7 +924,7 @@ int proxy_topk_gemm_bf16(int64_t N, int d, int V, const void* Hrows, const void*
 
 int bwd_chunk_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, const int32_t* tok,
                    const float* lse, const float* coef, float* dH, float* dW, int dw_accumulate, void* dz,
-                   int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call) {
+                   int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, bool clear) {
   int rcode;
   {
     CUtensorMap ta, tb;
@@ -929,9 +936,11 @@ int bwd_chunk_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, con
     if (!make_map(&tz, dz, V, rc, ldz * 2, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B)) return PS_ERR_INVALID_ARG;
     BwdDzEpi::Params ep{tok, lse, coef, static_cast<int>(rc), V, tok_base};
     if (halves == 1)
-      rcode = launch_gemm_single<false, false, BwdDzEpi, 1>(ta, tb, tz, rc, V, d, 0, kBandRecompute, ep, status, s);
+      rcode = launch_gemm_single<false, false, BwdDzEpi, 1>(ta, tb, tz, rc, V, d, 0, kBandRecompute, ep, status, s,
+                                                               clear);
     else
-      rcode = launch_gemm_single<false, false, BwdDzEpi, 2>(ta, tb, tz, rc, V, d, 0, kBandRecompute / 2, ep, status, s);
+      rcode = launch_gemm_single<false, false, BwdDzEpi, 2>(ta, tb, tz, rc, V, d, 0, kBandRecompute / 2, ep, status, s,
+                                                               clear);
     if (rcode != PS_OK) return rcode;
   }
   return bwd_grads_bf16(rc, d, V, Hpk, W, dH, dW, dw_accumulate, dz, ldz, status, s, dh_accumulate, n_call);
@@ -980,12 +989,12 @@ int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, flo
 }
 
 int dz_from_store_bf16(int64_t N, int V, void* store, int64_t ldz, const float* scale, int64_t lds,
-                       const int32_t* tok, const float* lse, const float* logp, const float* coef, cudaStream_t s,
-                       int tok_base) {
+                       const int32_t* tok, const float* lse, const float* logp, const float* coef, uint32_t* status,
+                       cudaStream_t s, int tok_base) {
   if (N == 0) return PS_OK;
   const dim3 grid(static_cast<unsigned>((N + kDzRows - 1) / kDzRows), static_cast<unsigned>((V + kDzCols - 1) / kDzCols));
   dz_from_store_kernel<<<grid, kDzThreads, 0, s>>>(N, V, static_cast<uint16_t*>(store), ldz, scale, lds, tok,
-                                                   tok_base, lse, logp, coef);
+                                                   tok_base, lse, logp, coef, status);
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }
 

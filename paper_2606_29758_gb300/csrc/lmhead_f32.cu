@@ -102,7 +102,9 @@ struct SlabLoader {
 // shared memory by the rank that stores their rows.
 template <class Cfg, bool A_K, bool B_K, class Epi, bool SPLIT>
 __global__ void __launch_bounds__(Cfg::kThreads, Cfg::kMinBlocks)
-    simt_gemm_kernel(int64_t M, int64_t N, int64_t K, Operand A, Operand B, typename Epi::Params ep) {
+    simt_gemm_kernel(int64_t M, int64_t N, int64_t K, Operand A, Operand B, typename Epi::Params ep, uint32_t* clear) {
+  // the call's first kernel zeroes the status (no CTA of this one sets a bit)
+  if (clear != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) clear_status(clear);
   constexpr int TM = Cfg::TM, TN = Cfg::TN, BK = Cfg::BK, PD = Cfg::PD, GM = Cfg::GM, GN = Cfg::GN;
   struct Slabs {
     float a[2][BK][TM + 4];
@@ -311,7 +313,7 @@ static int64_t simt_tiles(int64_t M, int64_t N) {
 
 template <class Cfg, bool A_K, bool B_K, class Epi>
 static int launch_simt_cfg(int64_t M, int64_t N, int64_t K, int ranks, Operand A, Operand B,
-                           const typename Epi::Params& ep, cudaStream_t s) {
+                           const typename Epi::Params& ep, cudaStream_t s, uint32_t* clear = nullptr) {
   const dim3 grid(static_cast<unsigned>((N + Cfg::TN - 1) / Cfg::TN), static_cast<unsigned>((M + Cfg::TM - 1) / Cfg::TM),
                   static_cast<unsigned>(ranks));
   if constexpr (A_K && !B_K) {   // dH
@@ -327,12 +329,13 @@ static int launch_simt_cfg(int64_t M, int64_t N, int64_t K, int ranks, Operand A
       cfg.stream = s;
       cfg.attrs = attr;
       cfg.numAttrs = 1;
-      return cudaLaunchKernelEx(&cfg, simt_gemm_kernel<Cfg, A_K, B_K, Epi, true>, M, N, K, A, B, ep) == cudaSuccess
+      return cudaLaunchKernelEx(&cfg, simt_gemm_kernel<Cfg, A_K, B_K, Epi, true>, M, N, K, A, B, ep,
+                                nullptr) == cudaSuccess
                  ? PS_OK
                  : PS_ERR_CUDA;
     }
   }
-  simt_gemm_kernel<Cfg, A_K, B_K, Epi, false><<<grid, Cfg::kThreads, 0, s>>>(M, N, K, A, B, ep);
+  simt_gemm_kernel<Cfg, A_K, B_K, Epi, false><<<grid, Cfg::kThreads, 0, s>>>(M, N, K, A, B, ep, clear);
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }
 
@@ -343,12 +346,12 @@ static bool simt_fits(int64_t M) { return (M + kSB - 1) / kSB <= 65535; }
 // tiles 32 / 28 us), medium ones below (small ones were never faster).
 template <class Epi>
 static int launch_z(int64_t M, int64_t N, int64_t K, Operand A, Operand B, const typename Epi::Params& ep,
-                    cudaStream_t s) {
+                    cudaStream_t s, uint32_t* clear) {
   if (M == 0 || N == 0) return PS_OK;
   if (!simt_fits(M)) return PS_ERR_UNSUPPORTED;
   if (2 * simt_tiles<SimtLarge>(M, N) >= 3 * num_sms_current())
-    return launch_simt_cfg<SimtLarge, true, true, Epi>(M, N, K, 1, A, B, ep, s);
-  return launch_simt_cfg<SimtMedium, true, true, Epi>(M, N, K, 1, A, B, ep, s);
+    return launch_simt_cfg<SimtLarge, true, true, Epi>(M, N, K, 1, A, B, ep, s, clear);
+  return launch_simt_cfg<SimtMedium, true, true, Epi>(M, N, K, 1, A, B, ep, s, clear);
 }
 
 // dW = dZ^T H, its k steps (the rows) in one CTA: small tiles where medium ones would leave half of the SMs
@@ -393,16 +396,16 @@ static int launch_dh(int64_t M, int64_t N, int64_t K, int64_t n_call, Operand A,
 int fwd_splits_f32(int V) { return (V + kSB - 1) / kSB; }
 
 int fwd_gemm_f32(int64_t N, int d, int V, const float* Hpk, const float* W, const int32_t* tok, float2* part,
-                 float* ztok, uint32_t*, cudaStream_t s, int tok_base) {
+                 float* ztok, uint32_t* status, cudaStream_t s, int tok_base) {
   return launch_z<SimtFwdEpi>(N, V, d, Operand{Hpk, d}, Operand{W, d}, SimtFwdEpi::Params{tok, part, ztok, tok_base},
-                              s);
+                              s, status);
 }
 
 int bwd_chunk_f32(int64_t rc, int d, int V, const float* Hpk, const float* W, const int32_t* tok,
                   const float* lse, const float* coef, float* dH, float* dW, int dw_accumulate, float* dz,
-                  int64_t ldz, uint32_t*, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call) {
+                  int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, bool clear) {
   int r = launch_z<SimtDzEpi>(rc, V, d, Operand{Hpk, d}, Operand{W, d},
-                              SimtDzEpi::Params{tok, lse, coef, dz, ldz, tok_base}, s);
+                              SimtDzEpi::Params{tok, lse, coef, dz, ldz, tok_base}, s, clear ? status : nullptr);
   if (r != PS_OK) return r;
   if (dH) {  // dH(m=i, n=c) = sum_v dz[i][v] W[v][c]
     r = launch_dh(rc, d, V, n_call, Operand{dz, ldz}, Operand{W, d}, SimtStoreEpi::Params{dH, d, dh_accumulate}, s);

@@ -21,6 +21,13 @@ __device__ __forceinline__ void raise_status(uint32_t* status, uint32_t bits) {
   if (status) atomicOr(status, bits);
 }
 
+// The status word and the count of finished blocks beside it, zeroed at a call's start: by the call's first
+// kernel where none of its CTAs sets a bit early (a memset of its own costs a launch), else by a memset.
+__device__ __forceinline__ void clear_status(uint32_t* status) {
+  status[0] = 0u;
+  status[1] = 0u;
+}
+
 __device__ __forceinline__ uint64_t globaltimer_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

@@ -33,9 +33,14 @@ int device_is_sm103() {
   return major == 10 && minor == 3;
 }
 
-static int begin_call(void* ws, size_t ws_bytes, size_t need, cudaStream_t s) {
+static int check_ws(const void* ws, size_t ws_bytes, size_t need) {
   if (ws == nullptr || (reinterpret_cast<uintptr_t>(ws) & 255)) return PS_ERR_WORKSPACE;
-  if (ws_bytes < need) return PS_ERR_WORKSPACE;
+  return ws_bytes < need ? PS_ERR_WORKSPACE : PS_OK;
+}
+// The workspace checked and its status zeroed. (Calls whose first kernel zeroes it use check_ws alone.)
+static int begin_call(void* ws, size_t ws_bytes, size_t need, cudaStream_t s) {
+  const int rc = check_ws(ws, ws_bytes, need);
+  if (rc != PS_OK) return rc;
   if (cudaMemsetAsync(ws, 0, kWsHeader, s) != cudaSuccess) return PS_ERR_CUDA;
   return PS_OK;
 }
@@ -217,6 +222,8 @@ __global__ void __launch_bounds__(kMetaThreads)
   if (blockIdx.x == 0) {
     __shared__ int64_t warp_l[kWarps], warp_n[kWarps];
     int64_t carry_l = 0, carry_n = 0;
+    if (threadIdx.x == 0) clear_status(status);   // the call's first kernel; only this CTA sets bits
+    __syncthreads();
     for (int base = 0; base < B; base += kMetaThreads) {
       const int k = base + threadIdx.x;
       int64_t lk = 0, nk = 0;
@@ -692,7 +699,7 @@ int ps_pack_prefixes(int P, int K, int T_max, int d, int dtype, const int32_t* L
     if (!hid_packed || !d_ok(d, dtype) || !al16(hid_full) || !al16(hid_packed)) return PS_ERR_INVALID_ARG;
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  int rc = begin_call(ws, ws_bytes, ps_pack_prefixes_workspace_size(P, K), s);
+  const int rc = check_ws(ws, ws_bytes, ps_pack_prefixes_workspace_size(P, K));
   if (rc != PS_OK) return rc;
   const int B = P * K;
   PackWs pw = pack_ws(ws, B);
@@ -757,7 +764,7 @@ static int lmhead_fwd_impl(int64_t N, int d, int V, int dtype, const void* Hpk, 
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   FwdWs f = fwd_ws(ws, N, V, dtype, ws_bytes);
   if (N > 0 && f.splits < 1) return PS_ERR_WORKSPACE;
-  int rc = begin_call(ws, ws_bytes, f.bytes, s);
+  int rc = N == 0 ? begin_call(ws, ws_bytes, f.bytes, s) : check_ws(ws, ws_bytes, f.bytes);
   if (rc != PS_OK) return rc;
   if (N == 0) return cudaMemsetAsync(loss, 0, sizeof(double), s) == cudaSuccess ? PS_OK : PS_ERR_CUDA;
   int splits;
@@ -799,7 +806,7 @@ static int bwd_from_store_impl(int64_t N, int d, int V, int64_t tok_base, int dt
   if (N > 0 && store_bytes < store_layout(N, V).bytes) return PS_ERR_WORKSPACE;
   if (!device_is_sm103()) return PS_ERR_UNSUPPORTED;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  int rc = begin_call(ws, ws_bytes, kWsHeader, s);
+  int rc = N == 0 ? begin_call(ws, ws_bytes, kWsHeader, s) : check_ws(ws, ws_bytes, kWsHeader);
   if (rc != PS_OK) return rc;
   if (N == 0) {
     if (dW && !(flags & PS_DW_ACCUMULATE))
@@ -813,7 +820,8 @@ static int bwd_from_store_impl(int64_t N, int d, int V, int64_t tok_base, int dt
   // 267.3 / 269.2 ms, back to back), so the parts run in turn.
   const StoreLayout L = store_layout(N, V);
   const float* scale = reinterpret_cast<const float*>(static_cast<const uint8_t*>(store) + L.scale_off);
-  rc = dz_from_store_bf16(N, V, store, L.ldz, scale, N, tok, lse, logp, coef, s, static_cast<int>(tok_base));
+  rc = dz_from_store_bf16(N, V, store, L.ldz, scale, N, tok, lse, logp, coef, status_word(ws), s,
+                          static_cast<int>(tok_base));
   if (rc != PS_OK) return rc;
   return bwd_grads_bf16(N, d, V, Hpk, W, dH, dW, (flags & PS_DW_ACCUMULATE) ? 1 : 0, store, L.ldz, status_word(ws),
                         s, (flags & PS_DH_ACCUMULATE) ? 1 : 0, N);
@@ -889,7 +897,7 @@ static int logit_stats_impl(int64_t N, int d, int Vs, int64_t v0, int dtype, con
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   FwdWs f = fwd_ws(ws, N, Vs, dtype, ws_bytes);
   if (N > 0 && f.splits < 1) return PS_ERR_WORKSPACE;
-  int rc = begin_call(ws, ws_bytes, f.bytes, s);
+  int rc = N == 0 ? begin_call(ws, ws_bytes, f.bytes, s) : check_ws(ws, ws_bytes, f.bytes);
   if (rc != PS_OK || N == 0) return rc;
   int splits;
   if (dtype == PS_DTYPE_BF16) {
@@ -987,7 +995,8 @@ static int lmhead_bwd_impl(int64_t N, int d, int V, int64_t tok_base, int dtype,
   if ((N > 0 && (!al16(Hpk) || !al16(W))) || (dH && !al16(dH)) || (dW && !al16(dW))) return PS_ERR_INVALID_ARG;
   if (dtype == PS_DTYPE_BF16 && !device_is_sm103()) return PS_ERR_UNSUPPORTED;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  int rc = begin_call(ws, ws_bytes, ps_lmhead_ppo_bwd_workspace_size(N, d, V, dtype, 128), s);
+  const size_t need = ps_lmhead_ppo_bwd_workspace_size(N, d, V, dtype, 128);
+  int rc = N == 0 ? begin_call(ws, ws_bytes, need, s) : check_ws(ws, ws_bytes, need);
   if (rc != PS_OK) return rc;
   if (N == 0) {
     if (dW && !(flags & PS_DW_ACCUMULATE))
@@ -1012,12 +1021,12 @@ static int lmhead_bwd_impl(int64_t N, int d, int V, int64_t tok_base, int dtype,
     if (dtype == PS_DTYPE_BF16) {
       const uint16_t* h = static_cast<const uint16_t*>(Hpk) + r0 * d;
       rc = bwd_chunk_bf16(rcn, d, V, h, W, tok + r0, lse + r0, coef + r0, dH ? dH + r0 * d : nullptr, dW, acc, dz,
-                          ldz, status_word(ws), s, static_cast<int>(tok_base), hacc, N);
+                          ldz, status_word(ws), s, static_cast<int>(tok_base), hacc, N, r0 == 0);
     } else {
       const float* h = static_cast<const float*>(Hpk) + r0 * d;
       rc = bwd_chunk_f32(rcn, d, V, h, static_cast<const float*>(W), tok + r0, lse + r0, coef + r0,
                          dH ? dH + r0 * d : nullptr, dW, acc, static_cast<float*>(dz), ldz, status_word(ws), s,
-                         static_cast<int>(tok_base), hacc, N);
+                         static_cast<int>(tok_base), hacc, N, r0 == 0);
     }
     if (rc != PS_OK) return rc;
   }

@@ -40,6 +40,7 @@ struct Sched {
   int band_m;     // m blocks per band
   int num_units;  // m_blocks * splits
   int num_kb;     // ceil(K / 64)
+  int clear;      // this launch opens a library call: it zeroes the status words
 
   __device__ __forceinline__ void unit(int u, int& m_blk, int& split, int& n0, int& n1) const {
     const int per_band = band_m * splits;
@@ -125,6 +126,8 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
   const int lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
+    // (a CTA of this kernel sets a bit only once a wait of seconds has run out)
+    if (sched.clear && blockIdx.x == 0) clear_status(status);
     for (int s = 0; s < S; ++s) {
       mbar_init(&sm.full[s], 1);
       mbar_init(&sm.empty[s], 1);
