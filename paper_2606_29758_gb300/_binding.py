@@ -8,6 +8,7 @@ no fallback, and importing this module without the built library raises.
 from __future__ import annotations
 
 import ctypes
+import threading
 import os
 from typing import Optional
 
@@ -140,7 +141,24 @@ def _stream(stream=None) -> Optional[int]:
     if stream is not None:
         return int(stream) if isinstance(stream, int) else stream.cuda_stream
     import torch
-    return torch.cuda.current_stream().cuda_stream
+    # the current stream's handle without building a Stream object around it (4 of them a pass took 8 us)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(torch.cuda.current_device()) if raw is not None else torch.cuda.current_stream().cuda_stream
+
+
+_tls = threading.local()
+
+
+def _row_count():
+    """This thread's host word for the number of packed rows: page-locked (the copy then needs no
+    staging), written and read within one ps_pack_prefixes call."""
+    if not hasattr(_tls, "rows"):
+        import torch
+        if not torch.cuda.is_available():
+            return ctypes.c_int64(-1)
+        _tls.rows_mem = torch.zeros(1, dtype=torch.int64).pin_memory()
+        _tls.rows = ctypes.c_int64.from_address(_tls.rows_mem.data_ptr())
+    return _tls.rows
 
 
 def _check(rc: int, where: str) -> None:
@@ -195,7 +213,7 @@ def ps_pack_prefixes_workspace_size(P: int, K: int) -> int:
 def ps_pack_prefixes(P, K, T_max, d, dtype, L, n, R, adv_mode, w_tab, tok_full, oldlogp_full, hid_full,
                      capacity, cu_seqlens, src_row, row_traj, row_pos, tok, oldlogp, w, adv, hid_packed, ws,
                      return_num_rows=True, stream=None) -> Optional[int]:
-    nrows = ctypes.c_int64(-1)
+    nrows = _row_count() if return_num_rows else None
     rc = lib().ps_pack_prefixes(P, K, T_max, d, dtype, _ptr(L), _ptr(n), _ptr(R), adv_mode, _ptr(w_tab),
                                 _ptr(tok_full), _ptr(oldlogp_full), _ptr(hid_full), capacity, _ptr(cu_seqlens),
                                 _ptr(src_row), _ptr(row_traj), _ptr(row_pos), _ptr(tok), _ptr(oldlogp), _ptr(w),

@@ -665,8 +665,8 @@ int ps_sample_cutoffs(int P, int K, int T_max, const uint64_t* q, const int32_t*
   int rc = begin_call(ws, ws_bytes, ps_sample_cutoffs_workspace_size(P, K, T_max), s);
   if (rc != PS_OK) return rc;
   const size_t smem = sizeof(uint64_t) * K;
-  if (cudaFuncSetAttribute(sample_cutoffs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(smem)) != cudaSuccess)
+  if (smem > 47 * 1024 && cudaFuncSetAttribute(sample_cutoffs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               static_cast<int>(smem)) != cudaSuccess)
     return PS_ERR_CUDA;
   // parts of a prompt: one per tile of steps while that leaves no more than two CTAs per SM
   int64_t parts = (T_max + kSampThreads - 1) / kSampThreads;
@@ -715,10 +715,12 @@ int ps_pack_prefixes(int P, int K, int T_max, int d, int dtype, const int32_t* L
                                                  row_pos, tok, oldlogp, w, adv, static_cast<uint4*>(hid_packed));
   if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
   if (h_num_rows) {
-    int32_t nr = 0;
-    if (cudaMemcpyAsync(&nr, cu_seqlens + B, sizeof(nr), cudaMemcpyDeviceToHost, s) != cudaSuccess) return PS_ERR_CUDA;
+    // straight into the caller's word (its low half: both hosts are little-endian), so that a page-locked one
+    // is copied to without the driver's staging
+    *h_num_rows = 0;
+    if (cudaMemcpyAsync(h_num_rows, cu_seqlens + B, sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+      return PS_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return PS_ERR_CUDA;
-    *h_num_rows = nr;
   }
   return PS_OK;
 }
