@@ -34,7 +34,7 @@ static __device__ __forceinline__ float pick32(const uint32_t (&r)[32], int j) {
 
 struct FwdLseEpi {
   static constexpr int kEpiWarps = 8;   // two column groups per row: two (max, sum) partials per unit
-  static constexpr bool kTmaStore = false;
+  static constexpr bool kTmaStore = false, kReadAhead = false;
   static constexpr int kStageBytes = 0;
   struct Params {
     const int32_t* tok;
@@ -96,7 +96,7 @@ struct FwdLseEpi {
 // The backward turns e into dZ = coef (1[v = o] - e 2^(m - lse log2 e)) in place.
 struct FwdLseStoreEpi {
   static constexpr int kEpiWarps = 8;   // as FwdLseEpi
-  static constexpr bool kTmaStore = true;
+  static constexpr bool kTmaStore = true, kReadAhead = false;
   static constexpr int kStageBytes = 32 * 64;   // 32 rows of 32 2-byte elements
   struct Params {
     const int32_t* tok;
@@ -170,7 +170,7 @@ struct FwdLseStoreEpi {
 // (1 - 2 p(o) + ||p||^2 would cancel there).
 struct FwdProxyEpi {
   static constexpr int kEpiWarps = 4;
-  static constexpr bool kTmaStore = false;
+  static constexpr bool kTmaStore = false, kReadAhead = false;
   static constexpr int kStageBytes = 0;
   struct Params {
     const int32_t* tok;
@@ -245,7 +245,7 @@ constexpr int kTopK = 16;
 template <int EPI_WARPS>
 struct FwdProxyTopkEpi {
   static constexpr int kEpiWarps = EPI_WARPS;
-  static constexpr bool kTmaStore = false;
+  static constexpr bool kTmaStore = false, kReadAhead = false;
   static constexpr int kStageBytes = 0;
   struct Params {
     const int32_t* tok;
@@ -318,7 +318,7 @@ struct FwdProxyTopkEpi {
 // the store itself).
 struct BwdDzEpi {
   static constexpr int kEpiWarps = 8;   // no per-row state: the two column groups store their own slices
-  static constexpr bool kTmaStore = true;
+  static constexpr bool kTmaStore = true, kReadAhead = false;
   static constexpr int kStageBytes = 32 * 64;   // 32 rows of 32 2-byte elements
   struct Params {
     const int32_t* tok;
@@ -393,7 +393,7 @@ struct BwdDzEpi {
 // registers; a step of 7.8k rows gained 2%.
 struct StoreF32Epi {
   static constexpr int kEpiWarps = 8;
-  static constexpr bool kTmaStore = true;
+  static constexpr bool kTmaStore = true, kReadAhead = true;
   static constexpr int kStageBytes = 32 * 128;
   struct Params {
     int N;
