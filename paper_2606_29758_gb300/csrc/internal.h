@@ -46,14 +46,15 @@ int proxy_topk_gemm_bf16(int64_t N, int d, int V, const void* Hrows, const void*
 // dz ([rc][ldz], operand dtype), then dH = dZ W and dW (+)= dZ^T Hpk. With tok_base, W holds
 // vocabulary rows [tok_base, tok_base + V) and the one-hot term applies where tok - tok_base is in [0, V);
 // dh_accumulate adds dH to what the buffer holds. n_call: rows of the whole call, which decide how dH's K
-// loop is split over CTAs, so that dH does not depend on the chunking. clear: the call's first chunk, whose first
+// loop is split over CTAs, so that dH does not depend on the chunking; v_call: the whole head's vocabulary (of which
+// W may be a shard), which decides for dW, so that a shard's rows are the whole head's. clear: the call's first chunk, whose first
 // kernel zeroes the status (the forwards' GEMMs and dz_from_store always do).
 int bwd_chunk_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, const int32_t* tok,
                    const float* lse, const float* coef, float* dH, float* dW, int dw_accumulate, void* dz,
-                   int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, bool clear);
+                   int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, int64_t v_call, bool clear);
 // dH = dZ W and dW (+)= dZ^T Hpk from dZ [rc][ldz] bf16 already in memory.
 int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, float* dH, float* dW, int dw_accumulate,
-                   const void* dz, int64_t ldz, uint32_t* status, cudaStream_t s, int dh_accumulate, int64_t n_call);
+                   const void* dz, int64_t ldz, uint32_t* status, cudaStream_t s, int dh_accumulate, int64_t n_call, int64_t v_call);
 // The logit store of the forward turned into dZ in place (f16 e -> bf16 dZ), rows [0, N) of already
 // offset pointers; scale [c][lds] (lds: the store's row count, the pitch of its slice maxima). With
 // tok_base, the store holds vocabulary columns [tok_base, tok_base + V) and the one-hot term applies
@@ -63,7 +64,7 @@ int dz_from_store_bf16(int64_t N, int V, void* store, int64_t ldz, const float* 
                        cudaStream_t s, int tok_base = 0);
 int bwd_chunk_f32(int64_t rc, int d, int V, const float* Hpk, const float* W, const int32_t* tok,
                   const float* lse, const float* coef, float* dH, float* dW, int dw_accumulate, float* dz,
-                  int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, bool clear);
+                  int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, int64_t v_call, bool clear);
 
 // Plain tensor-core GEMM (test hook): C[M][N] (+)= sum_k A(m,k) B(k,n), f32 out. variant: 0 one
 // CTA per 128 x 256 tile, 1 a CTA pair per 256 x 256 tile, 2 one CTA per 256 x 256 tile.

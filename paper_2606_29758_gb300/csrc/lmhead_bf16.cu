@@ -6,6 +6,7 @@
 // TMEM. Backward: the same product is recomputed per chunk of rows and turned into
 // dZ = coef (onehot - softmax) in bf16; dH = dZ W and dW = dZ^T Hpk are two more
 // tensor-core products over that chunk.
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 
@@ -699,13 +700,15 @@ static int splitk_clusters_at_once(int ranks) {
 struct SplitK {
   int ranks, halves;
 };
-static SplitK choose_splitk(int64_t M, int64_t N, int num_kb) {
+// narrow_too: the unsplit product may run on 128-row tiles (54 hundredths a k-block).
+static SplitK choose_splitk(int64_t M, int64_t N, int num_kb, bool narrow_too) {
   const int sms = num_sms_current();
   const int64_t nb = (N + kBN - 1) / kBN;
   const int64_t tiles[3] = {0, (M + kBM - 1) / kBM * nb, (M + 2 * kBM - 1) / (2 * kBM) * nb};
   SplitK best{1, 2};
   if (tiles[2] >= 2 * sms) return best;
   int64_t best_cost = (tiles[2] + sms - 1) / sms * num_kb * 100;
+  if (narrow_too) best_cost = std::min(best_cost, (tiles[1] + sms - 1) / sms * num_kb * 54);
   for (int halves = 2; halves >= 1; --halves)
     for (int S = 2; S <= 8 && S <= num_kb; S *= 2) {
       const int64_t at_once = splitk_clusters_at_once(S);
@@ -924,7 +927,7 @@ int proxy_topk_gemm_bf16(int64_t N, int d, int V, const void* Hrows, const void*
 
 int bwd_chunk_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, const int32_t* tok,
                    const float* lse, const float* coef, float* dH, float* dW, int dw_accumulate, void* dz,
-                   int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, bool clear) {
+                   int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, int64_t v_call, bool clear) {
   int rcode;
   {
     CUtensorMap ta, tb;
@@ -943,21 +946,22 @@ int bwd_chunk_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, con
                                                                clear);
     if (rcode != PS_OK) return rcode;
   }
-  return bwd_grads_bf16(rc, d, V, Hpk, W, dH, dW, dw_accumulate, dz, ldz, status, s, dh_accumulate, n_call);
+  return bwd_grads_bf16(rc, d, V, Hpk, W, dH, dW, dw_accumulate, dz, ldz, status, s, dh_accumulate, n_call,
+                        v_call);
 }
 
 // dH = dZ W and dW (+)= dZ^T H over rc rows of dZ [rc][ldz] bf16. Both have long K loops (V and rc):
 // one CTA computes a 256 x 256 tile as two M = 128 halves that share each B stage (a third fewer
 // operand bytes per FLOP); a call of few rows splits dH's K loop over clusters (choose_splitk).
 int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, float* dH, float* dW, int dw_accumulate,
-                   const void* dz, int64_t ldz, uint32_t* status, cudaStream_t s, int dh_accumulate, int64_t n_call) {
+                   const void* dz, int64_t ldz, uint32_t* status, cudaStream_t s, int dh_accumulate, int64_t n_call, int64_t v_call) {
   int rcode;
   if (dH) {
     CUtensorMap ta, tb, tc;
     if (!map_kmajor(&ta, dz, rc, V, ldz, 2 * kBM) || !map_mnmajor(&tb, W, V, d, d) || !map_out_f32(&tc, dH, rc, d, d))
       return PS_ERR_INVALID_ARG;
     StoreF32Epi::Params ep{d, dh_accumulate};
-    const SplitK split = choose_splitk(n_call, d, (V + kBK - 1) / kBK);
+    const SplitK split = choose_splitk(n_call, d, (V + kBK - 1) / kBK, false);
     if (split.ranks > 1) {
       const SplitOut o{dH, d, static_cast<int>(rc), d, dh_accumulate};
       if (split.halves == 2) {
@@ -975,10 +979,18 @@ int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, flo
     if (!map_mnmajor(&ta, dz, rc, V, ldz) || !map_mnmajor(&tb, Hpk, rc, d, d) || !map_out_f32(&tc, dW, V, d, d))
       return PS_ERR_INVALID_ARG;
     StoreF32Epi::Params ep{d, dw_accumulate};
+    const int kb = static_cast<int>((rc + kBK - 1) / kBK);
+    const SplitK split = choose_splitk(v_call, d, kb, true);
+    if (split.ranks > 1) {
+      // a small vocabulary has few tiles, and many rows as their K loop: 8000 rows, d = 128, V = 1024 47 us unsplit, 14
+      // split; d = 392, V = 2000 65 / 27; 100000 rows 737 / 256; d = 128, V = 9000 53 / 37
+      const SplitOut o{dW, d, V, d, dw_accumulate};
+      return split.halves == 2 ? launch_gemm_splitk<true, true, 2>(ta, tb, V, d, rc, split.ranks, o, status, s)
+                               : launch_gemm_splitk<true, true, 1>(ta, tb, V, d, rc, split.ranks, o, status, s);
+    }
     // dW of 65 to 256 rows (2 to 4 k-blocks) is bound by its stores, which the narrow tile's epilogue overlaps whole
     // with the next tile (200 rows, V = 152064: d = 3584 407 us narrow / 443 wide, d = 1536 183 / 200; 571 rows
     // 610 / 592).
-    const int kb = static_cast<int>((rc + kBK - 1) / kBK);
     if ((kb >= 2 && kb <= 4) || tile_halves(V, d, 17) == 1)
       rcode = launch_gemm_single<true, true, StoreF32Epi, 1>(ta, tb, tc, V, d, rc, 0, 2 * kBandGrad, ep, status, s);
     else

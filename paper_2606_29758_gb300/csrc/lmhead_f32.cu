@@ -7,6 +7,8 @@
 // hands 4 x 4 blocks of its tile to an epilogue: the forward's per-row (max, sum of exp)
 // over 64 columns (rows reduced across the 16 threads that share them with warp shuffles),
 // the backward's dZ, or a plain store.
+#include <type_traits>
+
 #include "internal.h"
 #include "ps_common.cuh"
 
@@ -316,7 +318,7 @@ static int launch_simt_cfg(int64_t M, int64_t N, int64_t K, int ranks, Operand A
                            const typename Epi::Params& ep, cudaStream_t s, uint32_t* clear = nullptr) {
   const dim3 grid(static_cast<unsigned>((N + Cfg::TN - 1) / Cfg::TN), static_cast<unsigned>((M + Cfg::TM - 1) / Cfg::TM),
                   static_cast<unsigned>(ranks));
-  if constexpr (A_K && !B_K) {   // dH
+  if constexpr (std::is_same<Epi, SimtStoreEpi>::value) {
     if (ranks > 1) {
       cudaLaunchConfig_t cfg = {};
       cudaLaunchAttribute attr[1];
@@ -354,43 +356,38 @@ static int launch_z(int64_t M, int64_t N, int64_t K, Operand A, Operand B, const
   return launch_simt_cfg<SimtMedium, true, true, Epi>(M, N, K, 1, A, B, ep, s, clear);
 }
 
-// dW = dZ^T H, its k steps (the rows) in one CTA: small tiles where medium ones would leave half of the SMs
-// idle (560 rows, d = 128, V = 1024: 12.0 against 17.7 us), else medium ones (d = 256, V = 3000: 28.7 against
-// 30.8 us for small ones).
-static int launch_dw(int64_t M, int64_t N, int64_t K, Operand A, Operand B, const SimtStoreEpi::Params& ep,
-                     cudaStream_t s) {
+// dH = dZ W (its k steps are the vocabulary) and dW = dZ^T H (the rows) may have few tiles: the CTAs of a cluster
+// then share the k steps where that shortens the longest SM's queue. n tiles on an SM take about 2.2, 2.5, 3, 4, 5,
+// ... times the steps of one (three are resident), and the exchange costs about 60 such steps. Measured, 1 / 2 / 4 / 8
+// ranks (us): dH at d = 768, V = 8192, 200 rows 265 / 167 / 113 / 83, 560 rows 271 / 221 / 160 / 184, 1200 rows 419 /
+// 328 / 359 / 347, 2500 rows 855 / 741 / 684 / 697; dW unsplit / by this rule, 8000 rows: d = 128, V = 1024 139 / 57,
+// d = 256, V = 3000 389 / 288, and (282 tiles, not split) d = 128, V = 9000 387 against 402 split.
+// Below 32 tiles, small ones with 8 ranks (dH of 560 rows, d = 128, V = 1024: 10.0 us against 11.8 on medium tiles and
+// 38.1 unsplit), and small ones too where an unsplit product would leave half of the SMs idle (dW there: 12.0 against
+// 17.7 us).
+// m_call: the rows of the whole call (dH) or of the whole vocabulary (dW), which decide, so that dH does not depend on
+// how the call is cut into chunks and a vocabulary shard's dW rows are the whole head's.
+template <bool A_K, bool B_K>
+static int launch_grad(int64_t M, int64_t N, int64_t K, int64_t m_call, Operand A, Operand B,
+                       const SimtStoreEpi::Params& ep, cudaStream_t s) {
   if (M == 0 || N == 0) return PS_OK;
   if (!simt_fits(M)) return PS_ERR_UNSUPPORTED;
-  if (2 * simt_tiles<SimtMedium>(M, N) < num_sms_current())
-    return launch_simt_cfg<SimtSmall, false, false, SimtStoreEpi>(M, N, K, 1, A, B, ep, s);
-  return launch_simt_cfg<SimtMedium, false, false, SimtStoreEpi>(M, N, K, 1, A, B, ep, s);
-}
-
-// dH = dZ W has few tiles and the vocabulary as its k steps: the CTAs of a cluster share them where that
-// shortens the longest SM's queue. n tiles on an SM take about 2.2, 2.5, 3, 4, 5, ... times the steps of one
-// (three are resident), and the exchange costs about 60 such steps. Measured, 1 / 2 / 4 / 8 ranks (us), d = 768,
-// V = 8192: 200 rows 265 / 167 / 113 / 83, 560 rows 271 / 221 / 160 / 184, 1200 rows 419 / 328 / 359 / 347, 2500
-// rows 855 / 741 / 684 / 697. Below 32 tiles, small ones with 8 ranks (560 rows, d = 128, V = 1024: 10.0 us
-// against 11.8 on medium tiles and 38.1 unsplit). The choice goes by the rows of the whole call, so
-// that dH does not depend on how the call is cut into chunks.
-static int launch_dh(int64_t M, int64_t N, int64_t K, int64_t n_call, Operand A, Operand B,
-                     const SimtStoreEpi::Params& ep, cudaStream_t s) {
-  if (M == 0 || N == 0) return PS_OK;
-  if (!simt_fits(M)) return PS_ERR_UNSUPPORTED;
-  const int64_t tiles = simt_tiles<SimtMedium>(n_call, N);
+  const int64_t tiles = simt_tiles<SimtMedium>(m_call, N);
+  const int sms = num_sms_current();
   int ranks = 1;
   if (tiles < 32) {
     while (ranks < 8 && K >= 8 * ranks * SimtSmall::BK) ranks *= 2;
-    return launch_simt_cfg<SimtSmall, true, false, SimtStoreEpi>(M, N, K, ranks, A, B, ep, s);
+    return launch_simt_cfg<SimtSmall, A_K, B_K, SimtStoreEpi>(M, N, K, ranks, A, B, ep, s);
   }
-  const int sms = num_sms_current();
   auto cost = [&](int r) {
     const int64_t n = (tiles * r + sms - 1) / sms, tenths = n == 1 ? 22 : n == 2 ? 25 : 10 * n;
     return tenths * ((K + SimtMedium::BK - 1) / SimtMedium::BK) / r + (r > 1 ? 600 : 0);
   };
-  for (int r = 2; r <= 8 && K >= 4 * r * SimtMedium::BK; r *= 2)
+  const int64_t most = A_K ? 4 * sms : 3 * sms / 2;   // from there on the exchanges cost what the last round gains
+  for (int r = 2; r <= 8 && K >= 4 * r * SimtMedium::BK && tiles < most; r *= 2)
     if (cost(r) < cost(ranks)) ranks = r;
-  return launch_simt_cfg<SimtMedium, true, false, SimtStoreEpi>(M, N, K, ranks, A, B, ep, s);
+  if (ranks == 1 && 2 * tiles < sms) return launch_simt_cfg<SimtSmall, A_K, B_K, SimtStoreEpi>(M, N, K, 1, A, B, ep, s);
+  return launch_simt_cfg<SimtMedium, A_K, B_K, SimtStoreEpi>(M, N, K, ranks, A, B, ep, s);
 }
 
 int fwd_splits_f32(int V) { return (V + kSB - 1) / kSB; }
@@ -403,16 +400,18 @@ int fwd_gemm_f32(int64_t N, int d, int V, const float* Hpk, const float* W, cons
 
 int bwd_chunk_f32(int64_t rc, int d, int V, const float* Hpk, const float* W, const int32_t* tok,
                   const float* lse, const float* coef, float* dH, float* dW, int dw_accumulate, float* dz,
-                  int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, bool clear) {
+                  int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, int64_t v_call, bool clear) {
   int r = launch_z<SimtDzEpi>(rc, V, d, Operand{Hpk, d}, Operand{W, d},
                               SimtDzEpi::Params{tok, lse, coef, dz, ldz, tok_base}, s, clear ? status : nullptr);
   if (r != PS_OK) return r;
   if (dH) {  // dH(m=i, n=c) = sum_v dz[i][v] W[v][c]
-    r = launch_dh(rc, d, V, n_call, Operand{dz, ldz}, Operand{W, d}, SimtStoreEpi::Params{dH, d, dh_accumulate}, s);
+    r = launch_grad<true, false>(rc, d, V, n_call, Operand{dz, ldz}, Operand{W, d},
+                                 SimtStoreEpi::Params{dH, d, dh_accumulate}, s);
     if (r != PS_OK) return r;
   }
   if (dW) {  // dW(m=v, n=c) = sum_i dz[i][v] H[i][c]
-    r = launch_dw(V, d, rc, Operand{dz, ldz}, Operand{Hpk, d}, SimtStoreEpi::Params{dW, d, dw_accumulate}, s);
+    r = launch_grad<false, false>(V, d, rc, v_call, Operand{dz, ldz}, Operand{Hpk, d},
+                                  SimtStoreEpi::Params{dW, d, dw_accumulate}, s);
   }
   return r;
 }

@@ -795,7 +795,8 @@ static int lmhead_fwd_impl(int64_t N, int d, int V, int dtype, const void* Hpk, 
 }
 
 // The backward from a logit store of V vocabulary columns whose first is global token id tok_base.
-static int bwd_from_store_impl(int64_t N, int d, int V, int64_t tok_base, int dtype, const void* Hpk, const void* W,
+// v_call: the whole head's vocabulary.
+static int bwd_from_store_impl(int64_t N, int d, int V, int64_t tok_base, int64_t v_call, int dtype, const void* Hpk, const void* W,
                                const int32_t* tok, const float* lse, const float* logp, const float* coef,
                                void* store, size_t store_bytes, float* dH, float* dW, int flags, void* ws,
                                size_t ws_bytes, ps_stream_t stream) {
@@ -826,7 +827,7 @@ static int bwd_from_store_impl(int64_t N, int d, int V, int64_t tok_base, int dt
                           static_cast<int>(tok_base));
   if (rc != PS_OK) return rc;
   return bwd_grads_bf16(N, d, V, Hpk, W, dH, dW, (flags & PS_DW_ACCUMULATE) ? 1 : 0, store, L.ldz, status_word(ws),
-                        s, (flags & PS_DH_ACCUMULATE) ? 1 : 0, N);
+                        s, (flags & PS_DH_ACCUMULATE) ? 1 : 0, N, v_call);
 }
 
 extern "C" {
@@ -862,7 +863,7 @@ int ps_lmhead_ppo_bwd_from_store(int64_t N, int d, int V, int dtype, const void*
                                  void* store, size_t store_bytes, float* dH, float* dW, int flags, void* ws,
                                  size_t ws_bytes, ps_stream_t stream) {
   NvtxRange nvtx_range("ps_lmhead_ppo_bwd_from_store");
-  return bwd_from_store_impl(N, d, V, 0, dtype, Hpk, W, tok, lse, logp, coef, store, store_bytes, dH, dW, flags, ws,
+  return bwd_from_store_impl(N, d, V, 0, V, dtype, Hpk, W, tok, lse, logp, coef, store, store_bytes, dH, dW, flags, ws,
                              ws_bytes, stream);
 }
 
@@ -873,7 +874,7 @@ int ps_lmhead_ppo_bwd_vocab_shard_from_store(int64_t N, int d, int Vs, int64_t v
                                              ps_stream_t stream) {
   NvtxRange nvtx_range("ps_lmhead_ppo_bwd_vocab_shard_from_store");
   if (Vs < 1 || v0 < 0 || V < 1 || v0 + Vs > V) return PS_ERR_INVALID_ARG;
-  return bwd_from_store_impl(N, d, Vs, v0, dtype, Hpk, W_shard, tok, lse, logp, coef, store, store_bytes, dH,
+  return bwd_from_store_impl(N, d, Vs, v0, V, dtype, Hpk, W_shard, tok, lse, logp, coef, store, store_bytes, dH,
                              dW_shard, flags, ws, ws_bytes, stream);
 }
 
@@ -987,8 +988,8 @@ size_t ps_lmhead_ppo_bwd_workspace_size(int64_t N, int d, int V, int dtype, int6
 }  // extern "C"
 
 // The backward over a head of V vocabulary rows whose first is global token id tok_base (0 for the
-// whole head, v0 for one shard of a vocabulary-parallel head).
-static int lmhead_bwd_impl(int64_t N, int d, int V, int64_t tok_base, int dtype, const void* Hpk, const void* W,
+// whole head, v0 for one shard of a vocabulary-parallel head of v_call rows in all).
+static int lmhead_bwd_impl(int64_t N, int d, int V, int64_t tok_base, int64_t v_call, int dtype, const void* Hpk, const void* W,
                            const int32_t* tok, const float* lse, const float* coef, float* dH, float* dW, int flags,
                            void* ws, size_t ws_bytes, ps_stream_t stream) {
   if (N < 0 || N > INT32_MAX || V < 1 || !dtype_ok(dtype) || !d_ok(d, dtype)) return PS_ERR_INVALID_ARG;
@@ -1023,12 +1024,12 @@ static int lmhead_bwd_impl(int64_t N, int d, int V, int64_t tok_base, int dtype,
     if (dtype == PS_DTYPE_BF16) {
       const uint16_t* h = static_cast<const uint16_t*>(Hpk) + r0 * d;
       rc = bwd_chunk_bf16(rcn, d, V, h, W, tok + r0, lse + r0, coef + r0, dH ? dH + r0 * d : nullptr, dW, acc, dz,
-                          ldz, status_word(ws), s, static_cast<int>(tok_base), hacc, N, r0 == 0);
+                          ldz, status_word(ws), s, static_cast<int>(tok_base), hacc, N, v_call, r0 == 0);
     } else {
       const float* h = static_cast<const float*>(Hpk) + r0 * d;
       rc = bwd_chunk_f32(rcn, d, V, h, static_cast<const float*>(W), tok + r0, lse + r0, coef + r0,
                          dH ? dH + r0 * d : nullptr, dW, acc, static_cast<float*>(dz), ldz, status_word(ws), s,
-                         static_cast<int>(tok_base), hacc, N, r0 == 0);
+                         static_cast<int>(tok_base), hacc, N, v_call, r0 == 0);
     }
     if (rc != PS_OK) return rc;
   }
@@ -1041,7 +1042,7 @@ int ps_lmhead_ppo_bwd(int64_t N, int d, int V, int dtype, const void* Hpk, const
                       const float* lse, const float* coef, float* dH, float* dW, int flags, void* ws,
                       size_t ws_bytes, ps_stream_t stream) {
   NvtxRange nvtx_range("ps_lmhead_ppo_bwd");
-  return lmhead_bwd_impl(N, d, V, 0, dtype, Hpk, W, tok, lse, coef, dH, dW, flags, ws, ws_bytes, stream);
+  return lmhead_bwd_impl(N, d, V, 0, V, dtype, Hpk, W, tok, lse, coef, dH, dW, flags, ws, ws_bytes, stream);
 }
 
 int ps_lmhead_ppo_bwd_vocab_shard(int64_t N, int d, int Vs, int64_t v0, int V, int dtype, const void* Hpk,
@@ -1050,7 +1051,7 @@ int ps_lmhead_ppo_bwd_vocab_shard(int64_t N, int d, int Vs, int64_t v0, int V, i
                                   ps_stream_t stream) {
   NvtxRange nvtx_range("ps_lmhead_ppo_bwd_vocab_shard");
   if (Vs < 1 || v0 < 0 || V < 1 || v0 + Vs > V) return PS_ERR_INVALID_ARG;
-  return lmhead_bwd_impl(N, d, Vs, v0, dtype, Hpk, W_shard, tok, lse, coef, dH, dW_shard, flags, ws, ws_bytes,
+  return lmhead_bwd_impl(N, d, Vs, v0, V, dtype, Hpk, W_shard, tok, lse, coef, dH, dW_shard, flags, ws, ws_bytes,
                          stream);
 }
 

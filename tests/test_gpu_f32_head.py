@@ -6,7 +6,7 @@ pass's own lse, dZ = coef (onehot - exp(z - lse)) is then off by at most |coef| 
 (the subtraction and the exponential round too) plus 2^-23 |dZ|, and an entry of dH or dW by that error
 carried through the product plus its own accumulation. The sum of V exponentials has relative error of at most
 V 2^-24 + max e_z + 2^-21, which is the bound on lse beside its rounding to f32. Sizes: one row and one column;
-d and V that end inside a 4-vector, a k step and a tile; few tiles (dH split over clusters of 2, 4 and 8) and
+d and V that end inside a 4-vector, a k step and a tile; few tiles (dH and dW split over clusters of 2, 4 and 8) and
 hundreds; rows cut into chunks, which must not change dH.
 """
 import pytest
@@ -17,7 +17,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("N,d,V", [(1, 8, 1), (3, 12, 5), (33, 20, 63), (64, 132, 65), (65, 64, 129), (200, 100, 1001),
                                    (191, 392, 2003), (700, 68, 3001), (129, 768, 4097), (1500, 260, 2050),
-                                   (5000, 128, 514)])
+                                   (5000, 128, 514),
+                                   (2600, 392, 1400)])
 def test_products_of_the_f32_head(N, d, V):
     from paper_2606_29758_gb300 import _binding as B
     F = B.PS_DTYPE_F32
