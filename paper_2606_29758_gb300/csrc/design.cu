@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(16 * kProxyRows)
                           float* __restrict__ top_prob, uint32_t* status) {
   __shared__ double s1_s[kProxyRows], s2_s[kProxyRows], tot_s[kProxyRows];
   __shared__ float m_s[kProxyRows];
+  wait_for_previous_kernel();
   const int sub = threadIdx.x & 15, r = threadIdx.x >> 4;
   const int64_t i = static_cast<int64_t>(blockIdx.x) * kProxyRows + r;
   const bool live = i < N;
@@ -170,6 +171,7 @@ __global__ void __launch_bounds__(kUncWarps * 32)
                        int topk, const int32_t* __restrict__ top_idx, const float* __restrict__ top_prob,
                        const int64_t* __restrict__ off, float* __restrict__ u) {
   extern __shared__ __align__(16) uint8_t smem[];
+  wait_for_previous_kernel();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int cap = unc_entries(K, topk);
   int32_t* etok = reinterpret_cast<int32_t*>(smem) + wid * cap;
@@ -1157,9 +1159,11 @@ int ps_lmhead_score_proxy(int64_t N, int d, int V, int dtype, const void* Hrows,
     rc = proxy_gemm_bf16(N, d, V, Hrows, W, tok, part, ztok, splits, status, s);
   }
   if (rc != PS_OK) return rc;
-  proxy_finalize_kernel<<<static_cast<unsigned>((N + kProxyRows - 1) / kProxyRows), 16 * kProxyRows, 0, s>>>(
-      N, V, splits, part, ztok, hn, tok, gamma, logp, topk, tpart, top_idx, top_prob, status);
-  return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
+  return launch_after(proxy_finalize_kernel, dim3(static_cast<unsigned>((N + kProxyRows - 1) / kProxyRows)), 16 * kProxyRows,
+                      0, s, 1, 1, true, N, V, splits, part, ztok, hn, tok, gamma, logp, topk, tpart, top_idx, top_prob,
+                      status) == cudaSuccess
+             ? PS_OK
+             : PS_ERR_CUDA;
 }
 
 size_t ps_reward_uncertainty_workspace_size(int P, int K) {
@@ -1194,9 +1198,10 @@ int ps_reward_uncertainty(int P, int K, int T_max, const int32_t* L, const float
                            static_cast<int>(smem)) != cudaSuccess)
     return PS_ERR_CUDA;
   const int64_t tasks = static_cast<int64_t>(P) * T_max;
-  uncertainty_kernel<<<static_cast<unsigned>((tasks + kUncWarps - 1) / kUncWarps), kUncWarps * 32, smem, s>>>(
-      P, K, T_max, L, R, topk, top_idx, top_prob, off, u);
-  return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
+  return launch_after(uncertainty_kernel, dim3(static_cast<unsigned>((tasks + kUncWarps - 1) / kUncWarps)), kUncWarps * 32,
+                      smem, s, 1, 1, true, P, K, T_max, L, R, topk, top_idx, top_prob, off, u) == cudaSuccess
+             ? PS_OK
+             : PS_ERR_CUDA;
 }
 
 static DesignWs design_ws(void* ws, int P, int T_max) {

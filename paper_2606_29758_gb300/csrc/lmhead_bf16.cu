@@ -604,8 +604,10 @@ static int launch_gemm_single(const CUtensorMap& ta, const CUtensorMap& tb, cons
       cudaSuccess)
     return PS_ERR_CUDA;
   const int grid = sc.num_units < num_sms_current() ? sc.num_units : num_sms_current();
-  kern<<<grid, 64 + 32 * EW, smem, s>>>(ta, tb, tc, sc, ep, status, kDefaultTimeoutNs);
-  return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
+  return launch_after(kern, dim3(static_cast<unsigned>(grid)), 64 + 32 * EW, smem, s, 1, 1, !clear, ta, tb, tc, sc, ep,
+                      status, kDefaultTimeoutNs) == cudaSuccess
+             ? PS_OK
+             : PS_ERR_CUDA;
 }
 
 // Number of CTA pairs of the pair kernel that fit on the device at once.
@@ -731,20 +733,9 @@ static int launch_gemm_splitk(const CUtensorMap& ta, const CUtensorMap& tb, int6
   constexpr size_t smem = sizeof(GemmSplitSmem<HALVES>) + 1024;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
     return PS_ERR_CUDA;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned>(ranks);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(static_cast<unsigned>(m_blocks * n_blocks * ranks), 1, 1);
-  cfg.blockDim = dim3(kSplitThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, ta, tb, n_blocks, static_cast<int>((K + kBK - 1) / kBK), o, status,
-                            kDefaultTimeoutNs) == cudaSuccess
+  return launch_after(kern, dim3(static_cast<unsigned>(m_blocks * n_blocks * ranks)), kSplitThreads, smem, s,
+                      static_cast<unsigned>(ranks), 1, true, ta, tb, n_blocks, static_cast<int>((K + kBK - 1) / kBK), o,
+                      status, kDefaultTimeoutNs) == cudaSuccess
              ? PS_OK
              : PS_ERR_CUDA;
 }
@@ -1032,15 +1023,15 @@ int gemm_bf16(int M, int N, int K, int a_mn, int b_mn, const void* A, int64_t ld
   if (!map_out_f32(&tc, C, M, N, ldc)) return PS_ERR_INVALID_ARG;
   E::Params ep{N, accumulate};
   if (variant == 2) {
-    if (!a_mn && !b_mn) return launch_gemm_single<false, false, E, 2>(ta, tb, tc, M, N, K, 0, 16, ep, status, s);
-    if (!a_mn && b_mn) return launch_gemm_single<false, true, E, 2>(ta, tb, tc, M, N, K, 0, 16, ep, status, s);
-    if (a_mn && b_mn) return launch_gemm_single<true, true, E, 2>(ta, tb, tc, M, N, K, 0, 16, ep, status, s);
-    return launch_gemm_single<true, false, E, 2>(ta, tb, tc, M, N, K, 0, 16, ep, status, s);
+    if (!a_mn && !b_mn) return launch_gemm_single<false, false, E, 2>(ta, tb, tc, M, N, K, 0, 16, ep, status, s, true);
+    if (!a_mn && b_mn) return launch_gemm_single<false, true, E, 2>(ta, tb, tc, M, N, K, 0, 16, ep, status, s, true);
+    if (a_mn && b_mn) return launch_gemm_single<true, true, E, 2>(ta, tb, tc, M, N, K, 0, 16, ep, status, s, true);
+    return launch_gemm_single<true, false, E, 2>(ta, tb, tc, M, N, K, 0, 16, ep, status, s, true);
   }
-  if (!a_mn && !b_mn) return launch_gemm_single<false, false, E, 1>(ta, tb, tc, M, N, K, 0, 16, ep, status, s);
-  if (!a_mn && b_mn) return launch_gemm_single<false, true, E, 1>(ta, tb, tc, M, N, K, 0, 16, ep, status, s);
-  if (a_mn && b_mn) return launch_gemm_single<true, true, E, 1>(ta, tb, tc, M, N, K, 0, 16, ep, status, s);
-  return launch_gemm_single<true, false, E, 1>(ta, tb, tc, M, N, K, 0, 16, ep, status, s);
+  if (!a_mn && !b_mn) return launch_gemm_single<false, false, E, 1>(ta, tb, tc, M, N, K, 0, 16, ep, status, s, true);
+  if (!a_mn && b_mn) return launch_gemm_single<false, true, E, 1>(ta, tb, tc, M, N, K, 0, 16, ep, status, s, true);
+  if (a_mn && b_mn) return launch_gemm_single<true, true, E, 1>(ta, tb, tc, M, N, K, 0, 16, ep, status, s, true);
+  return launch_gemm_single<true, false, E, 1>(ta, tb, tc, M, N, K, 0, 16, ep, status, s, true);
 }
 
 // ----------------------------------------------------------------------------- wait probe

@@ -105,6 +105,7 @@ struct SlabLoader {
 template <class Cfg, bool A_K, bool B_K, class Epi, bool SPLIT>
 __global__ void __launch_bounds__(Cfg::kThreads, Cfg::kMinBlocks)
     simt_gemm_kernel(int64_t M, int64_t N, int64_t K, Operand A, Operand B, typename Epi::Params ep, uint32_t* clear) {
+  wait_for_previous_kernel();
   // the call's first kernel zeroes the status (no CTA of this one sets a bit)
   if (clear != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) clear_status(clear);
   constexpr int TM = Cfg::TM, TN = Cfg::TN, BK = Cfg::BK, PD = Cfg::PD, GM = Cfg::GM, GN = Cfg::GN;
@@ -319,26 +320,16 @@ static int launch_simt_cfg(int64_t M, int64_t N, int64_t K, int ranks, Operand A
   const dim3 grid(static_cast<unsigned>((N + Cfg::TN - 1) / Cfg::TN), static_cast<unsigned>((M + Cfg::TM - 1) / Cfg::TM),
                   static_cast<unsigned>(ranks));
   if constexpr (std::is_same<Epi, SimtStoreEpi>::value) {
-    if (ranks > 1) {
-      cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = 1;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = static_cast<unsigned>(ranks);
-      cfg.gridDim = grid;
-      cfg.blockDim = dim3(Cfg::kThreads, 1, 1);
-      cfg.stream = s;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      return cudaLaunchKernelEx(&cfg, simt_gemm_kernel<Cfg, A_K, B_K, Epi, true>, M, N, K, A, B, ep,
-                                nullptr) == cudaSuccess
+    if (ranks > 1)
+      return launch_after(simt_gemm_kernel<Cfg, A_K, B_K, Epi, true>, grid, Cfg::kThreads, 0, s, 1,
+                          static_cast<unsigned>(ranks), true, M, N, K, A, B, ep, nullptr) == cudaSuccess
                  ? PS_OK
                  : PS_ERR_CUDA;
-    }
   }
-  simt_gemm_kernel<Cfg, A_K, B_K, Epi, false><<<grid, Cfg::kThreads, 0, s>>>(M, N, K, A, B, ep, clear);
-  return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
+  return launch_after(simt_gemm_kernel<Cfg, A_K, B_K, Epi, false>, grid, Cfg::kThreads, 0, s, 1, 1, clear == nullptr, M, N,
+                      K, A, B, ep, clear) == cudaSuccess
+             ? PS_OK
+             : PS_ERR_CUDA;
 }
 
 // M tiles of 64 rows past the grid's y limit are refused.

@@ -319,6 +319,7 @@ __global__ void __launch_bounds__(kPackThreads)
                      int32_t* __restrict__ src_row, int32_t* __restrict__ row_traj, int32_t* __restrict__ row_pos,
                      int32_t* __restrict__ tok, float* __restrict__ oldlogp, float* __restrict__ wout,
                      float* __restrict__ adv, uint4* __restrict__ hid_packed) {
+  wait_for_previous_kernel();
   const int64_t N = *w.N;
   const int lane = threadIdx.x & 31;
   const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
@@ -495,6 +496,7 @@ __global__ void __launch_bounds__(kMergeRows* kMergeSlices)
                         float* __restrict__ ratio, float* __restrict__ coef, float* __restrict__ row_loss,
                         uint32_t* ticket, uint32_t* status) {
   __shared__ bool last;
+  wait_for_previous_kernel();
   const int64_t i = static_cast<int64_t>(blockIdx.x) * kMergeRows + (threadIdx.x & 31);
   const float2 ms = merge_parts_block(part + i, splits, N, i < N);
   if (threadIdx.x < 32) {
@@ -526,6 +528,7 @@ __global__ void __launch_bounds__(kMergeRows* kMergeSlices)
     stats_merge_kernel(int64_t N, int splits, const float2* __restrict__ part, const float* __restrict__ ztok_ws,
                        const int32_t* __restrict__ tok, int64_t tok_base, int Vs, float2* __restrict__ stats,
                        float* __restrict__ ztok) {
+  wait_for_previous_kernel();
   const int64_t i = static_cast<int64_t>(blockIdx.x) * kMergeRows + (threadIdx.x & 31);
   const float2 ms = merge_parts_block(part + i, splits, N, i < N);
   if (threadIdx.x >= 32 || i >= N) return;
@@ -560,6 +563,7 @@ __global__ void __launch_bounds__(kFinThreads)
 
 __global__ void __launch_bounds__(1024) loss_reduce_kernel(int64_t nblocks, const double* __restrict__ part,
                                                            double* __restrict__ loss) {
+  wait_for_previous_kernel();
   double v = 0.0;
   for (int64_t b = threadIdx.x; b < nblocks; b += 1024) v += part[b];
   v = block_sum(v);
@@ -710,10 +714,10 @@ int ps_pack_prefixes(int P, int K, int T_max, int d, int dtype, const int32_t* L
   if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
   const int64_t row_vec = hid_full ? static_cast<int64_t>(d) * elem_size(dtype) / 16 : 0;
   const int grid = sms * 8;
-  pack_rows_kernel<<<grid, kPackThreads, 0, s>>>(B, K, T_max, cu_seqlens, pw, w_tab, tok_full, oldlogp_full,
-                                                 static_cast<const uint4*>(hid_full), row_vec, src_row, row_traj,
-                                                 row_pos, tok, oldlogp, w, adv, static_cast<uint4*>(hid_packed));
-  if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
+  if (launch_after(pack_rows_kernel, dim3(static_cast<unsigned>(grid)), kPackThreads, 0, s, 1, 1, true, B, K, T_max,
+                   cu_seqlens, pw, w_tab, tok_full, oldlogp_full, static_cast<const uint4*>(hid_full), row_vec, src_row,
+                   row_traj, row_pos, tok, oldlogp, w, adv, static_cast<uint4*>(hid_packed)) != cudaSuccess)
+    return PS_ERR_CUDA;
   if (h_num_rows) {
     // straight into the caller's word (its low half: both hosts are little-endian), so that a page-locked one
     // is copied to without the driver's staging
@@ -788,10 +792,11 @@ static int lmhead_fwd_impl(int64_t N, int d, int V, int dtype, const void* Hpk, 
                       status_word(ws), s);
   }
   if (rc != PS_OK) return rc;
-  fwd_finalize_kernel<<<merge_blocks(N), kMergeRows * kMergeSlices, 0, s>>>(
-      N, V, splits, f.part, f.ztok, tok, oldlogp, adv, w, eps, loss_scale, loss, lse, logp, ratio, coef, row_loss,
-      ticket_word(ws), status_word(ws));
-  return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
+  return launch_after(fwd_finalize_kernel, dim3(merge_blocks(N)), kMergeRows * kMergeSlices, 0, s, 1, 1, true, N, V, splits,
+                      f.part, f.ztok, tok, oldlogp, adv, w, eps, loss_scale, loss, lse, logp, ratio, coef, row_loss,
+                      ticket_word(ws), status_word(ws)) == cudaSuccess
+             ? PS_OK
+             : PS_ERR_CUDA;
 }
 
 // The backward from a logit store of V vocabulary columns whose first is global token id tok_base.
@@ -922,9 +927,10 @@ static int logit_stats_impl(int64_t N, int d, int Vs, int64_t v0, int dtype, con
                       f.ztok, status_word(ws), s, static_cast<int>(v0));
   }
   if (rc != PS_OK) return rc;
-  stats_merge_kernel<<<merge_blocks(N), kMergeRows * kMergeSlices, 0, s>>>(N, splits, f.part, f.ztok, tok, v0, Vs,
-                                                                           reinterpret_cast<float2*>(stats), ztok);
-  return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
+  return launch_after(stats_merge_kernel, dim3(merge_blocks(N)), kMergeRows * kMergeSlices, 0, s, 1, 1, true, N, splits,
+                      f.part, f.ztok, tok, v0, Vs, reinterpret_cast<float2*>(stats), ztok) == cudaSuccess
+             ? PS_OK
+             : PS_ERR_CUDA;
 }
 
 extern "C" {
@@ -971,8 +977,9 @@ int ps_lmhead_ppo_fwd_from_stats(int64_t N, int S, int64_t ld, int V, const floa
       N, S, ld, V, reinterpret_cast<const float2*>(stats), ztok, tok, oldlogp, adv, w, eps, loss_scale, lse, logp, ratio,
       coef, row_loss, block_loss, status_word(ws));
   if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
-  loss_reduce_kernel<<<1, 1024, 0, s>>>(nb, block_loss, loss);
-  return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
+  return launch_after(loss_reduce_kernel, dim3(1), 1024, 0, s, 1, 1, true, nb, block_loss, loss) == cudaSuccess
+             ? PS_OK
+             : PS_ERR_CUDA;
 }
 
 size_t ps_lmhead_ppo_bwd_workspace_size(int64_t N, int d, int V, int dtype, int64_t chunk_rows) {

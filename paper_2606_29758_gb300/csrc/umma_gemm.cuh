@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  wait_for_previous_kernel();
   const uint32_t tmem_base = sm.tmem_base;
   volatile int* abort = &sm.abort;
 
@@ -672,6 +673,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  wait_for_previous_kernel();
   const uint32_t tmem_base = sm.tmem_base;
   volatile int* abort = &sm.abort;
 
