@@ -4,9 +4,9 @@
 // inputs run here with exact f32 products and f32 accumulation, every output element over
 // its k in increasing order. One tiled kernel computes C(m, n) = sum_k A(m, k) B(k, n) for
 // operands whose k or whose m (n) is contiguous (Z = H W^T, dH = dZ W and dW = dZ^T H) and
-// hands 4 x 4 blocks of its tile to an epilogue: the forward's per-row (max, sum of exp)
-// over 64 columns (rows reduced across the 16 threads that share them with warp shuffles),
-// the backward's dZ, or a plain store.
+// hands blocks of its tile to an epilogue: the forward's per-row (max, sum of exp) over 64
+// columns (rows reduced across the 8 lanes that share them with warp shuffles), the
+// backward's dZ, or a plain store.
 #include <type_traits>
 
 #include "internal.h"
@@ -37,25 +37,26 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
   return d;
 }
 
-// A tile of TM x TN outputs by 16 x TY threads, in k steps of BK. A thread owns rows 4 ty + i + 4 TY g
-// and columns 4 tx + j + 64 h (i, j < 4): the 16 threads of a row sit in one half-warp, and its operands
-// are 16-byte shared loads. PD: k steps whose global loads are in flight while one is computed (they wait
-// in registers; shared memory holds two steps).
-template <int TM_, int TN_, int TY_, int BK_, int PD_, int MIN_BLOCKS>
+// A tile of TM x TN outputs by WM x WN warps, in k steps of BK. A warp owns 16 GM x 32 GN outputs, its lanes (ly, lx)
+// of 4 x 8 the rows 4 ly + i + 16 g and the columns 4 lx + j + 32 h (i, j < 4) of them, so that its operands are 16-byte
+// shared loads; neighbouring lanes differ in ly. PD: k steps whose global loads are in flight while one is computed (they
+// wait in registers; shared memory holds two steps).
+template <int TM_, int TN_, int WM_, int WN_, int BK_, int PD_, int MIN_BLOCKS>
 struct SimtCfg {
-  static constexpr int TM = TM_, TN = TN_, TY = TY_, BK = BK_, PD = PD_, kMinBlocks = MIN_BLOCKS;
-  static constexpr int kThreads = 16 * TY;
-  static constexpr int GM = TM / (4 * TY), GN = TN / 64;   // 4 x 4 blocks per thread
+  static constexpr int TM = TM_, TN = TN_, WN = WN_, BK = BK_, PD = PD_, kMinBlocks = MIN_BLOCKS;
+  static constexpr int kThreads = 32 * WM_ * WN_;
+  static constexpr int GM = TM / (16 * WM_), GN = TN / (32 * WN_);   // 4 x 4 blocks per thread
 };
 // The FP32 pipes are what bounds a product of many tiles; FFMA2 leaves issue slots for the shared loads
 // (the same kernel on single FMAs was 7-20% slower). 6330 rows at d = 768, V = 8192 (79.6 GFLOP each): Z
-// 1348 us on large tiles and 1600 on medium ones, dH 1567 and dW 1497 us on medium ones (large: 1861,
-// 1661), i.e. 51-59 TFLOP/s of the 80.5 that 152 SMs x 128 lanes have at 2070 MHz, against 3960, 2500 and
-// 3390 us for unpipelined 64 x 64 tiles with scalar loads. (128 x 64 and 128 x 128 tiles: Z 1589 / 1434, dH
-// 1546 / 1539, dW 1707 / 1768.) Few tiles are bound by the latency of their k steps instead.
-using SimtLarge = SimtCfg<64, 128, 8, 16, 1, 3>;
-using SimtMedium = SimtCfg<64, 64, 8, 16, 2, 3>;
-using SimtSmall = SimtCfg<32, 64, 8, 32, 2, 3>;
+// 1322 us on large tiles and 1452 on medium ones, dH 1425 and dW 1436 us on medium ones (large: 1839, 1581),
+// i.e. 55-60 TFLOP/s of the 80.5 that 152 SMs x 128 lanes have at 2070 MHz. (With 2 x 16 lanes to a warp,
+// and on medium tiles 8 x 4 outputs to a thread, Z 1334 / 1580, dH 1564, dW 1497; unpipelined 64 x 64 tiles with
+// scalar loads 3960, 2500 and 3390 us. 8 x 16 and 16 x 8 outputs to a thread: Z 1349 and 1414, dH 1539 and 1497, dW
+// 1643 and 1634.) Few tiles are bound by the latency of their k steps instead.
+using SimtLarge = SimtCfg<64, 128, 2, 2, 16, 1, 3>;
+using SimtMedium = SimtCfg<64, 64, 4, 1, 16, 2, 3>;
+using SimtSmall = SimtCfg<32, 64, 2, 2, 32, 2, 3>;
 
 // The T x BK slab of an operand that starts at row i0 and k0, through registers into s[BK][T + 4].
 template <int T, int BK, int THREADS, bool KMAJOR>
@@ -116,7 +117,9 @@ __global__ void __launch_bounds__(Cfg::kThreads, Cfg::kMinBlocks)
   __shared__ __align__(16) unsigned char smem[sizeof(Slabs)];
   Slabs& sm = *reinterpret_cast<Slabs*>(smem);
   const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
+  const int lane = tid & 31, warp = tid >> 5;
+  const int r0 = warp / Cfg::WN * 16 * GM + 4 * ((lane & 1) | ((lane >> 4) << 1));   // the thread's first row and column
+  const int c0 = warp % Cfg::WN * 32 * GN + 4 * ((lane >> 1) & 7);                   // of the tile
   const int64_t m0 = static_cast<int64_t>(blockIdx.y) * TM;
   const int64_t n0 = static_cast<int64_t>(blockIdx.x) * TN;
   int64_t kfirst = 0, steps = (K + BK - 1) / BK;
@@ -153,9 +156,9 @@ __global__ void __launch_bounds__(Cfg::kThreads, Cfg::kMinBlocks)
       for (int k = 0; k < BK; ++k) {
         float4 a[GM], b[GN];
 #pragma unroll
-        for (int g = 0; g < GM; ++g) a[g] = *reinterpret_cast<const float4*>(&sm.a[buf][k][ty * 4 + 4 * Cfg::TY * g]);
+        for (int g = 0; g < GM; ++g) a[g] = *reinterpret_cast<const float4*>(&sm.a[buf][k][r0 + 16 * g]);
 #pragma unroll
-        for (int h = 0; h < GN; ++h) b[h] = *reinterpret_cast<const float4*>(&sm.b[buf][k][tx * 4 + 64 * h]);
+        for (int h = 0; h < GN; ++h) b[h] = *reinterpret_cast<const float4*>(&sm.b[buf][k][c0 + 32 * h]);
 #pragma unroll
         for (int g = 0; g < GM; ++g) {
           const float av[4] = {a[g].x, a[g].y, a[g].z, a[g].w};
@@ -184,7 +187,7 @@ __global__ void __launch_bounds__(Cfg::kThreads, Cfg::kMinBlocks)
     for (int i = 0; i < 4 * GM; ++i)
 #pragma unroll
       for (int h = 0; h < GN; ++h)
-        *reinterpret_cast<float4*>(&part[(i & 3) + ty * 4 + 4 * Cfg::TY * (i >> 2)][tx * 4 + 64 * h]) =
+        *reinterpret_cast<float4*>(&part[r0 + (i & 3) + 16 * (i >> 2)][c0 + 32 * h]) =
             make_float4(acc[i][2 * h].x, acc[i][2 * h].y, acc[i][2 * h + 1].x, acc[i][2 * h + 1].y);
     cluster_sync_all();   // every rank's partial is in its shared memory
     const int ranks = gridDim.z, rank = blockIdx.z;
@@ -201,20 +204,19 @@ __global__ void __launch_bounds__(Cfg::kThreads, Cfg::kMinBlocks)
     cluster_sync_all();   // no rank exits while another reads its partial
   } else {
 #pragma unroll
-    for (int g = 0; g < GM; ++g)
+    for (int g = 0; g < GM; ++g) {
+      float block[4][GN][4];
 #pragma unroll
-      for (int h = 0; h < GN; ++h) {
-        float block[4][4];
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          block[i][0] = acc[4 * g + i][2 * h].x;
-          block[i][1] = acc[4 * g + i][2 * h].y;
-          block[i][2] = acc[4 * g + i][2 * h + 1].x;
-          block[i][3] = acc[4 * g + i][2 * h + 1].y;
+        for (int h = 0; h < GN; ++h) {
+          block[i][h][0] = acc[4 * g + i][2 * h].x;
+          block[i][h][1] = acc[4 * g + i][2 * h].y;
+          block[i][h][2] = acc[4 * g + i][2 * h + 1].x;
+          block[i][h][3] = acc[4 * g + i][2 * h + 1].y;
         }
-        Epi::tile(ep, M, N, m0 + ty * 4 + 4 * Cfg::TY * g, n0 + tx * 4 + 64 * h,
-                  static_cast<int>((n0 >> 6) + h), tx, block);
-      }
+      Epi::tile(ep, M, N, m0 + r0 + 16 * g, n0 + c0, block);
+    }
   }
 }
 
@@ -225,30 +227,33 @@ struct SimtFwdEpi {
     float* ztok;
     int tok_base;   // token ids are global; W holds vocabulary rows [tok_base, tok_base + N)
   };
+  // a warp has 64 columns, from a multiple of 64 on; the 8 lanes of a row differ in bits 1 to 3 of their number
   static __device__ __forceinline__ void tile(const Params& p, int64_t M, int64_t N, int64_t r0, int64_t c0,
-                                              int ntile, int tx, float (&acc)[4][4]) {
+                                              float (&acc)[4][2][4]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int64_t row = r0 + i;
-      float x[4];
+      float x[8];
       float mx = -INFINITY;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        x[j] = (c0 + j < N) ? acc[i][j] * kLog2e : -INFINITY;
+      for (int j = 0; j < 8; ++j) {
+        x[j] = (c0 + (j >> 2) * 32 + (j & 3) < N) ? acc[i][j >> 2][j & 3] * kLog2e : -INFINITY;
         mx = fmaxf(mx, x[j]);
       }
       const int t = row < M ? __ldg(p.tok + row) - p.tok_base : -1;
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (c0 + j < N && c0 + j == t) p.ztok[row] = acc[i][j];
+      for (int j = 0; j < 8; ++j) {
+        const int64_t c = c0 + (j >> 2) * 32 + (j & 3);
+        if (c < N && c == t) p.ztok[row] = acc[i][j >> 2][j & 3];
+      }
 #pragma unroll
-      for (int o = 8; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      for (int o = 8; o >= 2; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       float s = 0.f;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) s += exp2f(x[j] - mx);
+      for (int j = 0; j < 8; ++j) s += exp2f(x[j] - mx);
 #pragma unroll
-      for (int o = 8; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (tx == 0 && row < M && c0 < N) p.part[static_cast<int64_t>(ntile) * M + row] = make_float2(mx, s);
+      for (int o = 8; o >= 2; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if ((c0 & 63) == 0 && row < M && c0 < N) p.part[(c0 >> 6) * M + row] = make_float2(mx, s);
     }
   }
 };
@@ -262,24 +267,29 @@ struct SimtDzEpi {
     int64_t ldz;
     int tok_base;
   };
-  static __device__ __forceinline__ void tile(const Params& p, int64_t M, int64_t N, int64_t r0, int64_t c0, int,
-                                              int, float (&acc)[4][4]) {
+  template <int GN>
+  static __device__ __forceinline__ void tile(const Params& p, int64_t M, int64_t N, int64_t r0, int64_t c0,
+                                              float (&acc)[4][GN][4]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int64_t row = r0 + i;
       if (row >= M) continue;
       const int t = __ldg(p.tok + row) - p.tok_base;
       const float l = __ldg(p.lse + row), c = __ldg(p.coef + row);
-      float v[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = c * ((c0 + j == t ? 1.f : 0.f) - expf(acc[i][j] - l));
-      float* dst = p.dz + row * p.ldz + c0;
-      if (c0 + 4 <= N) {
-        *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-      } else {
+      for (int h = 0; h < GN; ++h) {
+        const int64_t col = c0 + 32 * h;
+        float v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (c0 + j < N) dst[j] = v[j];
+        for (int j = 0; j < 4; ++j) v[j] = c * ((col + j == t ? 1.f : 0.f) - expf(acc[i][h][j] - l));
+        float* dst = p.dz + row * p.ldz + col;
+        if (col + 4 <= N) {
+          *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (col + j < N) dst[j] = v[j];
+        }
       }
     }
   }
@@ -301,11 +311,14 @@ struct SimtStoreEpi {
     }
     *d = v;
   }
-  static __device__ __forceinline__ void tile(const Params& p, int64_t M, int64_t N, int64_t r0, int64_t c0, int,
-                                              int, float (&acc)[4][4]) {
+  template <int GN>
+  static __device__ __forceinline__ void tile(const Params& p, int64_t M, int64_t N, int64_t r0, int64_t c0,
+                                              float (&acc)[4][GN][4]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-      store4(p, M, N, r0 + i, c0, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
+#pragma unroll
+      for (int h = 0; h < GN; ++h)
+        store4(p, M, N, r0 + i, c0 + 32 * h, make_float4(acc[i][h][0], acc[i][h][1], acc[i][h][2], acc[i][h][3]));
   }
 };
 
@@ -335,8 +348,8 @@ static int launch_simt_cfg(int64_t M, int64_t N, int64_t K, int ranks, Operand A
 // M tiles of 64 rows past the grid's y limit are refused.
 static bool simt_fits(int64_t M) { return (M + kSB - 1) / kSB <= 65535; }
 
-// Z = H W^T: large tiles from three per two SMs on (measured, large / medium: 256 tiles 77 / 87 us, 216
-// tiles 32 / 28 us), medium ones below (small ones were never faster).
+// Z = H W^T: large tiles from three per two SMs on (measured, large / medium: 256 tiles 73 / 78 us, 216
+// tiles 30 / 25 us), medium ones below (small ones were never faster).
 template <class Epi>
 static int launch_z(int64_t M, int64_t N, int64_t K, Operand A, Operand B, const typename Epi::Params& ep,
                     cudaStream_t s, uint32_t* clear) {
@@ -350,12 +363,12 @@ static int launch_z(int64_t M, int64_t N, int64_t K, Operand A, Operand B, const
 // dH = dZ W (its k steps are the vocabulary) and dW = dZ^T H (the rows) may have few tiles: the CTAs of a cluster
 // then share the k steps where that shortens the longest SM's queue. n tiles on an SM take about 2.2, 2.5, 3, 4, 5,
 // ... times the steps of one (three are resident), and the exchange costs about 60 such steps. Measured, 1 / 2 / 4 / 8
-// ranks (us): dH at d = 768, V = 8192, 200 rows 265 / 167 / 113 / 83, 560 rows 271 / 221 / 160 / 184, 1200 rows 419 /
-// 328 / 359 / 347, 2500 rows 855 / 741 / 684 / 697; dW unsplit / by this rule, 8000 rows: d = 128, V = 1024 139 / 57,
-// d = 256, V = 3000 389 / 288, and (282 tiles, not split) d = 128, V = 9000 387 against 402 split.
-// Below 32 tiles, small ones with 8 ranks (dH of 560 rows, d = 128, V = 1024: 10.0 us against 11.8 on medium tiles and
-// 38.1 unsplit), and small ones too where an unsplit product would leave half of the SMs idle (dW there: 12.0 against
-// 17.7 us).
+// ranks (us): dH at d = 768, V = 8192, 200 rows 233 / 160 / 108 / 78, 560 rows 235 / 215 / 154 / 170, 1200 rows 388 /
+// 326 / 335 / 333, 2500 rows 754 / 719 / 652 / 664; dW unsplit / by this rule, 8000 rows: d = 128, V = 1024 208 / 53,
+// d = 256, V = 3000 373 / 276, and (282 tiles, not split) d = 128, V = 9000 371 against 387 split.
+// Below 32 tiles, small ones with 8 ranks (dH of 560 rows, d = 128, V = 1024: 8.2 us against 11.8 on medium tiles and
+// 31 unsplit), and small ones too where an unsplit product would leave half of the SMs idle (dW there: 8.2 against
+// 16.2 us).
 // m_call: the rows of the whole call (dH) or of the whole vocabulary (dW), which decide, so that dH does not depend on
 // how the call is cut into chunks and a vocabulary shard's dW rows are the whole head's.
 template <bool A_K, bool B_K>
