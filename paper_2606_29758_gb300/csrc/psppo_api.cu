@@ -409,66 +409,158 @@ __device__ __forceinline__ float2 merge_parts(const float2* __restrict__ part, i
   return make_float2(m, S);
 }
 
-// A block of the forward's finalize (and of the shard statistics' merge) takes kMergeRows rows, one
-// per lane, and kMergeSlices warps that each merge every kMergeSlices-th of the rows' vocabulary
-// parts. A row of the 152k vocabulary has 1188 parts (9.5 KB), so the kernels are bound by reading
-// them: a warp's 32 rows of one part are 256 contiguous bytes, and 8 parts are in flight per thread.
-// One thread per row instead (two passes over the parts) left a few hundred rows on a handful of
-// SMs with a serial chain of 1188 loads: 254 us for 185 rows and 291 us for 7.8k rows at V = 152064
-// with the loss reduction then launched after it, against 16 and 25 us now; 208 us, 4.9 TB/s, at 106k
-// rows (before: 501 us). The order of the merge depends
-// on the number of parts alone, so a row's result does not depend on the batch around it.
-constexpr int kMergeRows = 32;
-constexpr int kMergeSlices = 16;
-constexpr int kMergeBatch = 8;
+// A block of the forward's finalize (and of the shard statistics' merge) takes 8, 16 or 32 rows. Its threads find the
+// maximum m of each row's parts and copy the parts, chunk by chunk, into a ring in shared memory; all warps but the
+// first turn every x into 2^(x - m), and a lane of warp 0 per row adds the products of the chunk before up in
+// vocabulary order, as merge_parts does, whatever the batch around the row. (Sums over slices of the parts, rescaled and merged,
+// need one reading but left the lse 0.2 to 0.8% further from 64 bits: a mean error of 2.139e-5 instead of 2.134e-5 over
+// 185 rows at V = 152064.) Bound by reading the parts twice, the second time mostly from L2 (a row of the 152k
+// vocabulary has 1188, 9.5 KB; once where the ring holds them all), and for few rows by the 2.5 us that 1188 dependent
+// additions take. Whole kernel at V = 152064: 185 rows 16 us, 8000 rows 32, 106000 rows 329; V = 2000: 7.8, 9.2 and 33.
+// (The same sum by one thread per row that reads its parts twice: 204, 230 and 8.0, 9.2 at 185 and 8000 rows.)
+constexpr int kMergeBatch = 6;                     // parts per thread and chunk
+constexpr int kMergeStages = 4;                    // two in flight, one converted, one added up
+template <int R, int THREADS>
+struct MergeCfg {
+  static constexpr int kRows = R, kThreads = THREADS;
+  static constexpr int kMakers = THREADS - 32;                 // the threads that copy and convert
+  static constexpr int kChunk = kMakers * kMergeBatch;         // elements of a chunk
+  static constexpr int kParts = kChunk / R, kSlices = kMakers / R;   // its parts, and the threads per row
+  static_assert(kMakers % R == 0 && kParts * R == kChunk, "whole parts");
+};
 
-// S 2^(x - m) for parts whose maximum x is at most m; a part without columns (x = -inf, S = 0) adds 0
-// even where no part has any yet (m = -inf).
-__device__ __forceinline__ float scaled_sum(float x, float S, float m) { return x == m ? S : S * exp2f(x - m); }
+__device__ __forceinline__ void cp_async_8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
-// The merged (max, sum) of row `part` (its `count` parts, `stride` apart): valid in warp 0. Every warp
-// of the block calls it; rows past the end (live false) read nothing.
-__device__ __forceinline__ float2 merge_parts_block(const float2* __restrict__ part, int count, int64_t stride,
-                                                    bool live) {
-  __shared__ float2 slice_s[kMergeSlices][kMergeRows];
+// The merged (max, sum) of the block's `rows` <= R rows, row i's in lane i of warp 0. part: the first row's first part,
+// `count` parts `stride` apart. Every thread of the block calls it. Shared memory: min(chunks, kMergeStages) chunks.
+template <class C>
+__device__ __forceinline__ float2 merge_parts_block(const float2* part, int count, int64_t stride, int rows) {
+  extern __shared__ __align__(16) float2 ring[];
+  constexpr int R = C::kRows, kSlices = C::kSlices, kParts = C::kParts, kMakers = C::kMakers;
+  __shared__ float max_s[C::kThreads / 32][R];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float m = -INFINITY, S = 0.f;
-  if (live) {
-    const float2* p = part + static_cast<int64_t>(warp) * stride;
-    const int64_t step = static_cast<int64_t>(kMergeSlices) * stride;
-    int c = warp;
-    for (; c + (kMergeBatch - 1) * kMergeSlices < count; c += kMergeBatch * kMergeSlices, p += kMergeBatch * step) {
-      float2 v[kMergeBatch];
+  const int maker = static_cast<int>(threadIdx.x) - 32, r = threadIdx.x % R;
+  const bool live = r < rows;
+  const int chunks = (count + kParts - 1) / kParts;
+  const bool held = chunks <= kMergeStages;   // every part stays in the ring
+  auto fetch = [&](int k) {   // this thread's parts of chunk k
+    int c = k * kParts + maker / R;
+    const float2* p = part + c * stride + r;
+    float2* to = ring + k % kMergeStages * C::kChunk + maker;
 #pragma unroll
-      for (int j = 0; j < kMergeBatch; ++j) v[j] = p[j * step];
-      float mn = m;
+    for (int j = 0; j < kMergeBatch; ++j, c += kSlices, p += kSlices * stride, to += kMakers)
+      if (live && c < count) cp_async_8(to, p);
+    cp_async_commit();
+  };
+  if (maker >= 0)
+    for (int k = 0; k < (held ? chunks : 2); ++k) fetch(k);
+  float m = -INFINITY;
+  if (held) {
+    cp_async_wait<0>();
+    if (maker >= 0 && live)
+#pragma unroll 6
+      for (int c = maker / R, e = maker; c < count; c += kSlices, e += kMakers) m = fmaxf(m, ring[e].x);
+  } else if (live) {
+    constexpr int kAll = C::kThreads / R, kFly = 12;
+    int c = threadIdx.x / R;
+    const float2* p = part + c * stride + r;
+    for (; c + (kFly - 1) * kAll < count; c += kFly * kAll, p += kFly * kAll * stride) {
+      float x[kFly];
 #pragma unroll
-      for (int j = 0; j < kMergeBatch; ++j) mn = fmaxf(mn, v[j].x);
-      S = scaled_sum(m, S, mn);
-      m = mn;
+      for (int j = 0; j < kFly; ++j) x[j] = p[j * (kAll * stride)].x;
 #pragma unroll
-      for (int j = 0; j < kMergeBatch; ++j) S += scaled_sum(v[j].x, v[j].y, m);
+      for (int j = 0; j < kFly; ++j) m = fmaxf(m, x[j]);
     }
-    for (; c < count; c += kMergeSlices, p += step) {
-      const float2 v = *p;
-      const float mn = fmaxf(m, v.x);
-      S = scaled_sum(m, S, mn) + scaled_sum(v.x, v.y, mn);
-      m = mn;
-    }
+#pragma unroll 4
+    for (; c < count; c += kAll, p += kAll * stride) m = fmaxf(m, p->x);
   }
-  slice_s[warp][lane] = make_float2(m, S);
+#pragma unroll
+  for (int o = 16; o >= R; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane < R) max_s[warp][lane] = m;
   __syncthreads();
-  if (warp == 0) {
 #pragma unroll
-    for (int k = 0; k < kMergeSlices; ++k) m = fmaxf(m, slice_s[k][lane].x);
-    S = 0.f;
+  for (int w = 0; w < C::kThreads / 32; ++w) m = fmaxf(m, max_s[w][r]);
+  float S = 0.f;
+  for (int k = 0; k <= chunks; ++k) {   // chunk k is converted and chunk k - 1 added
+    if (maker >= 0) {
+      if (k < chunks) {
+        if (!held) {
+          fetch(k + 2);   // where chunk k - 2 was, added in the round before
+          cp_async_wait<2>();
+        }
+        const int c = k * kParts + maker / R;
+        float2* v = ring + k % kMergeStages * C::kChunk + maker;
 #pragma unroll
-    for (int k = 0; k < kMergeSlices; ++k) S += scaled_sum(slice_s[k][lane].x, slice_s[k][lane].y, m);
+        for (int j = 0; j < kMergeBatch; ++j)
+          if (live && c + j * kSlices < count) v[j * kMakers].x = exp2f(v[j * kMakers].x - m);
+      }
+    } else if (k > 0 && lane < R) {
+      const float2* b = ring + (k - 1) % kMergeStages * C::kChunk + lane;
+      const int n = min(kParts, count - (k - 1) * kParts);
+      // 10 parts at a time, the next 10 loaded under their additions
+      float2 x[10], y[10];
+      auto take = [&](float2(&to)[10], int c) {
+        if (c + 10 <= n) {
+#pragma unroll
+          for (int j = 0; j < 10; ++j) to[j] = b[(c + j) * R];
+        }
+      };
+      auto add = [&](const float2(&of)[10]) {
+#pragma unroll
+        for (int j = 0; j < 10; ++j) S = fmaf(of[j].y, of[j].x, S);
+      };
+      int c = 0;
+      take(x, 0);
+      for (; c + 10 <= n; c += 10) {
+        take(y, c + 10);
+        add(x);
+        c += 10;
+        if (c + 10 > n) break;
+        take(x, c + 10);
+        add(y);
+      }
+      for (; c < n; ++c) S = fmaf(b[c * R].y, b[c * R].x, S);
+    }
+    __syncthreads();
   }
   return make_float2(m, S);
 }
 
-static unsigned merge_blocks(int64_t N) { return static_cast<unsigned>((N + kMergeRows - 1) / kMergeRows); }
+template <class C, class Kernel, class... Args>
+static int launch_merge_cfg(Kernel kern, int64_t N, int count, cudaStream_t s, Args... args) {
+  const int chunks = (count + C::kParts - 1) / C::kParts;
+  const size_t smem = sizeof(float2) * C::kChunk * (chunks < kMergeStages ? chunks : kMergeStages);
+  // more than the 48 KB that a launch may have without asking (the kernel's own arrays included)
+  if (smem > 45 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               static_cast<int>(smem)) != cudaSuccess)
+    return PS_ERR_CUDA;
+  return launch_after(kern, dim3(static_cast<unsigned>((N + C::kRows - 1) / C::kRows)), C::kThreads, smem, s, 1, 1, true,
+                      N, args...) == cudaSuccess
+             ? PS_OK
+             : PS_ERR_CUDA;
+}
+// Launches the kernel that `pick` gives for a MergeCfg. Few rows are spread over the SMs, 8 to a block; then a warp
+// finalises more of them (its double arithmetic costs the same for 32 rows as for 8). Small blocks leave an SM 8 rings
+// and 8 adding warps, which pays once there are enough of them: 60000 rows at V = 152064 take 195 us with 128 threads
+// and 203 with 512, at V = 32000 51 and 81, at V = 2000 23 and 46. A row of one chunk wants no more threads either
+// (600 rows, V = 2000: 7.7 and 8.3 us; 250 parts: 10.1 and 9.7).
+template <class Pick, class... Args>
+static int launch_merge(Pick pick, int64_t N, int count, cudaStream_t s, Args... args) {
+  const int64_t sms = num_sms_current();
+  auto go = [&](auto cfg) { return launch_merge_cfg<decltype(cfg)>(pick(cfg), N, count, s, args...); };
+  const bool one_chunk = count <= MergeCfg<8, 128>::kParts;
+  if (N <= 8 * 2 * sms) return one_chunk ? go(MergeCfg<8, 128>()) : go(MergeCfg<8, 512>());
+  if (N <= 16 * 2 * sms && !one_chunk) return go(MergeCfg<16, 512>());
+  if (N <= 32 * 2 * sms && !one_chunk) return go(MergeCfg<32, 512>());
+  return go(MergeCfg<32, 128>());
+}
 
 // Sum of v over the block in a fixed order (warp shuffles, then warp 0 over the warps' sums), in thread 0.
 __device__ __forceinline__ double block_sum(double v) {
@@ -488,7 +580,8 @@ __device__ __forceinline__ double block_sum(double v) {
 // The block's sum of row losses goes where its rows' first parts were (nobody else reads them), and
 // the last block to finish (`ticket`, zeroed at the call's start, counts them) adds the sums up: one
 // launch less than a separate reduction, and the same order of addition whichever block is last.
-__global__ void __launch_bounds__(kMergeRows* kMergeSlices)
+template <class C>
+__global__ void __launch_bounds__(C::kThreads, 1024 / C::kThreads)
     fwd_finalize_kernel(int64_t N, int V, int splits, float2* __restrict__ part, const float* __restrict__ ztok,
                         const int32_t* __restrict__ tok, const float* __restrict__ oldlogp,
                         const float* __restrict__ adv, const float* __restrict__ w, double eps, double loss_scale,
@@ -497,17 +590,19 @@ __global__ void __launch_bounds__(kMergeRows* kMergeSlices)
                         uint32_t* ticket, uint32_t* status) {
   __shared__ bool last;
   wait_for_previous_kernel();
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * kMergeRows + (threadIdx.x & 31);
-  const float2 ms = merge_parts_block(part + i, splits, N, i < N);
+  constexpr int R = C::kRows;
+  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * R, i = i0 + threadIdx.x;
+  const int rows = static_cast<int>(N - i0 < R ? N - i0 : R);
+  const float2 ms = merge_parts_block<C>(part + i0, splits, N, rows);
   if (threadIdx.x < 32) {
     double rl = 0.0;
-    if (i < N)
+    if (threadIdx.x < rows)
       rl = finalize_row(i, ms.x, ms.y, ztok[i], tok[i], V, oldlogp, adv, w, eps, loss_scale, lse, logp, ratio, coef,
                         row_loss, status);
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) rl += __shfl_down_sync(0xffffffffu, rl, o);
+    for (int o = R / 2; o >= 1; o >>= 1) rl += __shfl_down_sync(0xffffffffu, rl, o);
     if (threadIdx.x == 0) {
-      *reinterpret_cast<double*>(part + i) = rl;
+      *reinterpret_cast<double*>(part + i0) = rl;
       __threadfence();
       last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
@@ -517,21 +612,24 @@ __global__ void __launch_bounds__(kMergeRows* kMergeSlices)
   __threadfence();
   double v = 0.0;
   for (int64_t b = threadIdx.x; b < gridDim.x; b += blockDim.x)
-    v += __ldcg(reinterpret_cast<const double*>(part + b * kMergeRows));
+    v += __ldcg(reinterpret_cast<const double*>(part + b * R));
   v = block_sum(v);
   if (threadIdx.x == 0) *loss = v;
 }
 
 // A vocabulary shard's statistics: its vocabulary tiles' (max, sum) pairs merged per row, and the
 // chosen logit where the row's token lies in the shard ([tok_base, tok_base + Vs)), -inf elsewhere.
-__global__ void __launch_bounds__(kMergeRows* kMergeSlices)
+template <class C>
+__global__ void __launch_bounds__(C::kThreads, 1024 / C::kThreads)
     stats_merge_kernel(int64_t N, int splits, const float2* __restrict__ part, const float* __restrict__ ztok_ws,
                        const int32_t* __restrict__ tok, int64_t tok_base, int Vs, float2* __restrict__ stats,
                        float* __restrict__ ztok) {
   wait_for_previous_kernel();
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * kMergeRows + (threadIdx.x & 31);
-  const float2 ms = merge_parts_block(part + i, splits, N, i < N);
-  if (threadIdx.x >= 32 || i >= N) return;
+  constexpr int R = C::kRows;
+  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * R, i = i0 + threadIdx.x;
+  const int rows = static_cast<int>(N - i0 < R ? N - i0 : R);
+  const float2 ms = merge_parts_block<C>(part + i0, splits, N, rows);
+  if (threadIdx.x >= rows) return;
   stats[i] = ms;
   const int64_t t = static_cast<int64_t>(tok[i]) - tok_base;
   ztok[i] = (t >= 0 && t < Vs) ? ztok_ws[i] : -INFINITY;
@@ -792,11 +890,9 @@ static int lmhead_fwd_impl(int64_t N, int d, int V, int dtype, const void* Hpk, 
                       status_word(ws), s);
   }
   if (rc != PS_OK) return rc;
-  return launch_after(fwd_finalize_kernel, dim3(merge_blocks(N)), kMergeRows * kMergeSlices, 0, s, 1, 1, true, N, V, splits,
-                      f.part, f.ztok, tok, oldlogp, adv, w, eps, loss_scale, loss, lse, logp, ratio, coef, row_loss,
-                      ticket_word(ws), status_word(ws)) == cudaSuccess
-             ? PS_OK
-             : PS_ERR_CUDA;
+  return launch_merge([](auto cfg) { return fwd_finalize_kernel<decltype(cfg)>; }, N, splits, s, V, splits, f.part,
+                      f.ztok, tok, oldlogp, adv, w, eps, loss_scale, loss, lse, logp, ratio, coef, row_loss, ticket_word(ws),
+                      status_word(ws));
 }
 
 // The backward from a logit store of V vocabulary columns whose first is global token id tok_base.
@@ -927,10 +1023,8 @@ static int logit_stats_impl(int64_t N, int d, int Vs, int64_t v0, int dtype, con
                       f.ztok, status_word(ws), s, static_cast<int>(v0));
   }
   if (rc != PS_OK) return rc;
-  return launch_after(stats_merge_kernel, dim3(merge_blocks(N)), kMergeRows * kMergeSlices, 0, s, 1, 1, true, N, splits,
-                      f.part, f.ztok, tok, v0, Vs, reinterpret_cast<float2*>(stats), ztok) == cudaSuccess
-             ? PS_OK
-             : PS_ERR_CUDA;
+  return launch_merge([](auto cfg) { return stats_merge_kernel<decltype(cfg)>; }, N, splits, s, splits, f.part, f.ztok,
+                      tok, v0, Vs, reinterpret_cast<float2*>(stats), ztok);
 }
 
 extern "C" {
