@@ -278,30 +278,23 @@ __global__ void group_offsets_kernel(int B, const int32_t* __restrict__ L, int64
 constexpr int kDesignThreads = 256;
 constexpr int kDesignWarps = kDesignThreads / 32;
 
-// Arrays of 2 T_max entries that the capped design takes from each of bW, bs and bn per prompt (the workspace
-// has room for 16 of each).
-constexpr int kDesignArrays = 16;
+// Prefixes that the capped design tries side by side, a lane of a warp each, on a stack of T_max blocks each: the
+// workspace has these of bW, bs and bn per prompt. The arrays of one prefix tried by the whole CTA (2 T_max entries
+// each, a few of each kind) lie in the same place.
+constexpr int kCapLanes = 32;
 struct DesignWs {
   double* w;       // [P][T_max] weights
   double* xi;      // [P][T_max]
-  double* bW;      // [P][kDesignArrays][2 T_max]
-  double* bs;      // [P][kDesignArrays][2 T_max]
-  int32_t* bn;     // [P][kDesignArrays][2 T_max]
+  double* bW;      // [P][T_max][kCapLanes] block weights, one stack per lane (interleaved)
+  double* bs;      // [P][T_max][kCapLanes] block scores sqrt(W / n)
+  int32_t* bn;     // [P][T_max][kCapLanes] block lengths
 };
 
 // True when the block (Wc, nc) violates the order against the block (Wp, np) below it, i.e. when
 // sqrt(Wp / np) < sqrt(Wc / nc) with both quotients and roots rounded to double, exactly as the
 // sequential definition decides it. The cross products Wp nc and Wc np settle every case whose
-// quotients differ by more than 2^-40 relative (then the rounded roots are ordered the same way), and
-// in float (each within 2^-22) those that differ by more than 2^-19: an SM of GB300 does two FP64 operations a clock,
-// so double operations, let alone the near-ties' divisions and square roots, are slow (the design
-// of 8 prompts of 15350 steps: 1.71 ms, without the float test 1.86).
-__device__ __forceinline__ bool pav_violates(double Wp, int np, double Wc, int nc) {
-  const float fa = static_cast<float>(Wp) * static_cast<float>(nc), fb = static_cast<float>(Wc) * static_cast<float>(np);
-  if (fa > 1e-30f && fb > 1e-30f && fa < 1e30f && fb < 1e30f) {
-    if (fb > fa * (1.0f + 0x1p-19f)) return true;
-    if (fb < fa * (1.0f - 0x1p-19f)) return false;
-  }
+// quotients differ by more than 2^-40 relative (then the rounded roots are ordered the same way).
+__device__ __forceinline__ bool pav_violates_double(double Wp, int np, double Wc, int nc) {
   const double a = __dmul_rn(Wp, static_cast<double>(nc));
   const double b = __dmul_rn(Wc, static_cast<double>(np));
   if (a > 0x1p-900 && b > 0x1p-900 && a < 0x1p900 && b < 0x1p900) {
@@ -309,6 +302,17 @@ __device__ __forceinline__ bool pav_violates(double Wp, int np, double Wc, int n
     if (b < __dmul_rn(a, 1.0 - 0x1p-40)) return false;
   }
   return __dsqrt_rn(__ddiv_rn(Wp, static_cast<double>(np))) < __dsqrt_rn(__ddiv_rn(Wc, static_cast<double>(nc)));
+}
+// The same, with the products taken in float first (each within 2^-22), which settles quotients that differ by more
+// than 2^-19: an SM of GB300 does two FP64 operations a clock, so double operations, let alone the near-ties'
+// divisions and square roots, are slow (the design of 8 prompts of 15350 steps: 1.71 ms, without the float test 1.86).
+__device__ __forceinline__ bool pav_violates(double Wp, int np, double Wc, int nc) {
+  const float fa = static_cast<float>(Wp) * static_cast<float>(nc), fb = static_cast<float>(Wc) * static_cast<float>(np);
+  if (fa > 1e-30f && fb > 1e-30f && fa < 1e30f && fb < 1e30f) {
+    if (fb > fa * (1.0f + 0x1p-19f)) return true;
+    if (fb < fa * (1.0f - 0x1p-19f)) return false;
+  }
+  return pav_violates_double(Wp, np, Wc, nc);
 }
 
 // Float-float numbers (an unevaluated sum hi + lo of two floats, about 44 significant bits). Knuth's TwoSum
@@ -471,13 +475,12 @@ __device__ void hull_links(const float2* S, int n, int32_t* link, float2* hull_S
 // instead the links of the weights taken from the right give the first block [t, T - link) of every suffix
 // design at once. With D(t) = sum over a suffix's blocks of n_m s_m = sqrt(n_m W_m), which is its first block's
 // term plus D at that block's end, the suffix design starts at g(t) = (B - t) s_front / D(t). status[t] records
-// whether g(t) is clearly above 1 (0), clearly below (2) or within kCapBand of 1 (1); only the last kind, and
-// the first clear one, are then decided by the exact rounded sequence of the definition.
+// whether g(t) is clearly above 1 (0), clearly below (2) or within kCapBand of 1 (1); all but the first kind are then
+// decided by the exact rounded sequence of the definition, in increasing order, until one passes.
 // The first block's mean is the largest slope from t, hence at least Q_t / (T - t) with Q_t the sum of the
 // suffix, of which the float-float sums are off by 2^-45: its weight is off by 2^-45 (T - t) / n relative, 2^-21 at
 // the largest T. Roots, products and the comparison add a few 2^-24: far inside kCapBand.
 constexpr double kCapBand = 0x1p-16;
-constexpr int kMaxNearCap = 64;        // prefixes within the band decided exactly (beyond: the full scan)
 
 // S, link: of the weights from the right, u = T - t, S negated. D [T + 1] scratch.
 __device__ void cap_status(const float2* S, const int32_t* link, int T, double B, float2* D, float* status) {
@@ -679,6 +682,42 @@ struct Pooled {
   }
 };
 
+// Pools w[0..T) one weight after another into one lane's stack (element m of the stack at index m * kCapLanes), each
+// block sum added as the definition adds it. The last block stays in registers, and memory is read only when a merge
+// uncovers the block below. (Traces that get here are nearly flat: the float test would only add to the double one. 4000
+// weights within 1e-7 of each other, budget 4000: 0.70 s without it, 0.81 with it.) Returns the number of blocks.
+__device__ __noinline__ int pav_stack(const double* w, int T, double* bW, int32_t* bn) {
+  int nb = 0, nt = 0;
+  double Wt = 0.0, wnext = T > 0 ? w[0] : 0.0;
+  for (int t = 0; t < T; ++t) {
+    if (t + 16 < T) asm volatile("prefetch.global.L1 [%0];" ::"l"(w + t + 16));
+    double Wc = wnext;
+    if (t + 1 < T) wnext = w[t + 1];
+    int nc = 1;
+    while (nb > 0 && pav_violates_double(Wt, nt, Wc, nc)) {
+      Wc = __dadd_rn(Wt, Wc);
+      nc += nt;
+      --nb;
+      if (nb > 0) {
+        Wt = bW[static_cast<int64_t>(nb - 1) * kCapLanes];
+        nt = bn[static_cast<int64_t>(nb - 1) * kCapLanes];
+      }
+    }
+    if (nb > 0) {
+      bW[static_cast<int64_t>(nb - 1) * kCapLanes] = Wt;
+      bn[static_cast<int64_t>(nb - 1) * kCapLanes] = nt;
+    }
+    Wt = Wc;
+    nt = nc;
+    ++nb;
+  }
+  if (nb > 0) {
+    bW[static_cast<int64_t>(nb - 1) * kCapLanes] = Wt;
+    bn[static_cast<int64_t>(nb - 1) * kCapLanes] = nt;
+  }
+  return nb;
+}
+
 // Timestep weights of the OPTIMIZED and HEURISTIC designs, before the floor: w_t = gamma_bar_t * u_t with
 // gamma_bar_t = (1/K) sum over the completions that reach t, and the largest of each kWeightSteps steps. A
 // division costs tens of FP64 operations, of which an SM of GB300 does two a clock, so the steps are spread over
@@ -733,7 +772,7 @@ __global__ void __launch_bounds__(kDesignThreads)
   __syncthreads();
   if (tid == 0) {
     for (int i = 1; i < kDesignWarps; ++i) wmax = fmax(wmax, red_d[i]);
-    ws.bW[static_cast<int64_t>(p) * 2 * T_max * kDesignArrays + blockIdx.y] = wmax;   // free until the pooling
+    ws.bW[static_cast<int64_t>(p) * T_max * kCapLanes + blockIdx.y] = wmax;   // free until the pooling
   }
 }
 
@@ -750,8 +789,8 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
   __shared__ unsigned long long red_b[kDesignThreads / 32];
   __shared__ int red_i[kDesignThreads / 32];
   __shared__ double lam_s;
-  __shared__ int ncand_s, nnear_s, tdef_s, decided_s;
-  __shared__ int cand_s[kMaxNearCap + 1];
+  __shared__ int decided_s, found_s;
+  __shared__ int cand_s[kCapLanes], nb_s[kCapLanes];
   __shared__ double den_s;
   extern __shared__ __align__(16) float2 dyn_smem[];    // the hull's vertices (kDesignDynSmem bytes)
   const int lane = tid & 31, wid = tid >> 5;
@@ -778,7 +817,7 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
     // the floor under the weights: the largest of them from the weights kernel's parts
     double wmax = 0.0;
     {
-      const double* parts = ws.bW + static_cast<int64_t>(p) * 2 * T_max * kDesignArrays;
+      const double* parts = ws.bW + static_cast<int64_t>(p) * T_max * kCapLanes;
       for (int c = tid; c * kWeightSteps < Tp; c += kDesignThreads) wmax = fmax(wmax, parts[c]);
     }
 #pragma unroll
@@ -794,13 +833,16 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
       // The smallest saturated prefix s whose suffix design (budget B - s) starts at or below 1, decided by
       // the definition's exact rounded sequence: for a candidate s, w[s..T) is pooled, the blocks' scores are
       // s_m = sqrt(W_m / n_m), den = sum_m n_m s_m in block order, and it passes if (B - s) s_1 / den <= 1.
-      // Candidates: the prefixes whose status is within the band of 1, then the first clearly below it, in
-      // increasing order; the first that passes is the answer. (If the band holds too many, or none
-      // passes, every prefix is tried in order.)
+      // Candidates, in increasing order: the prefixes whose status is not clearly above 1. As a rule the first or
+      // second passes. The whole CTA tries them one by one until that has taken the steps of two whole traces; the
+      // rest go 32 at a time, a lane each: a budget at or above the horizon puts every suffix that is flat to 2^-16
+      // into the band, hundreds of them, and where the weights fall slowly none passes before the last. (4000
+      // steps that fall by 3e-6 in all, budget 4000: 0.5 s so, 15.8 s one by one.)
+      const int64_t stacks = static_cast<int64_t>(p) * T_max * kCapLanes;
       const int64_t pitch = 2 * static_cast<int64_t>(T_max);   // at least T + 1
-      double* fW = ws.bW + p * pitch * kDesignArrays;
-      double* fs = ws.bs + p * pitch * kDesignArrays;
-      int32_t* fn = ws.bn + p * pitch * kDesignArrays;
+      double* fW = ws.bW + stacks;
+      double* fs = ws.bs + stacks;
+      int32_t* fn = ws.bn + stacks;
       float2* S = reinterpret_cast<float2*>(fW);
       float2* D = reinterpret_cast<float2*>(fW + pitch);
       double* blockW = fW + 2 * pitch;      // Pooled::W
@@ -822,45 +864,26 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
       ff_prefix_sums([&](int i) { return scaled(Tp - 1 - i); }, Tp, -1.f, S);
       hull_links(S, Tp, link, hull_S, hull, hull_deep);
       cap_status(S, link, Tp, Bp, D, status);
-      int td = Tp;
-      for (int t = tid; t < Tp; t += kDesignThreads)
-        if (status[t] == 2.f) {
-          td = t;
-          break;
-        }
-#pragma unroll
-      for (int o = 16; o >= 1; o >>= 1) td = min(td, __shfl_xor_sync(0xffffffffu, td, o));
-      if (lane == 0) red_i[wid] = td;
-      if (tid == 0) nnear_s = 0;
-      __syncthreads();
-      if (tid == 0) {
-        int m = Tp;
-        for (int i = 0; i < kDesignThreads / 32; ++i) m = min(m, red_i[i]);
-        tdef_s = m;
-      }
-      __syncthreads();
-      const int tdef = tdef_s;
-      for (int t = tid; t < tdef; t += kDesignThreads)
-        if (status[t] == 1.f) {
-          const int i = atomicAdd(&nnear_s, 1);
-          if (i < kMaxNearCap) cand_s[i] = t;
-        }
-      __syncthreads();
-      if (tid == 0) {
-        const int n = min(nnear_s, kMaxNearCap);
-        for (int i = 1; i < n; ++i) {          // the few near-band prefixes, in increasing order
-          const int v = cand_s[i];
-          int j = i - 1;
-          while (j >= 0 && cand_s[j] > v) {
-            cand_s[j + 1] = cand_s[j];
-            --j;
+      // The next prefixes from `from` on that are to be tried, at most `most` of them, into cand_s in increasing
+      // order; returns their number (the whole CTA). above: those whose status is clearly above 1 instead.
+      auto candidates = [&](int from, int most, bool above) {
+        int count = 0;
+        for (int t0 = from; t0 < Tp && count < most; t0 += kDesignThreads) {
+          const int t = t0 + tid;
+          const bool take = t < Tp && (status[t] == 0.f) == above;
+          const unsigned mask = __ballot_sync(0xffffffffu, take);
+          if (lane == 0) red_i[wid] = __popc(mask);
+          __syncthreads();
+          int at = count + __popc(mask & ((1u << lane) - 1u));
+          for (int k = 0; k < kDesignWarps; ++k) {
+            if (k < wid) at += red_i[k];
+            count += red_i[k];
           }
-          cand_s[j + 1] = v;
+          if (take && at < most) cand_s[at] = t;
+          __syncthreads();
         }
-        ncand_s = nnear_s > kMaxNearCap ? 0 : n + (tdef < Tp ? 1 : 0);
-        if (tdef < Tp && nnear_s <= kMaxNearCap) cand_s[n] = tdef;
-      }
-      __syncthreads();
+        return min(count, most);
+      };
       int nb = 0;
       // Pools w[s..T) and tests the prefix; block m's end is ends[nb - 1 - m].
       auto passes = [&](int s) {
@@ -893,13 +916,47 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
         __syncthreads();
         return __ddiv_rn(__dmul_rn(__dsub_rn(Bp, static_cast<double>(s)), score[0]), den_s) <= 1.0;
       };
-      int found = -1;
-      for (int c = 0; c < ncand_s && found < 0; ++c)
-        if (passes(cand_s[c])) found = cand_s[c];
-      // every prefix in order: only when the band held too many prefixes or no candidate passed, which the
-      // accuracy of the statuses rules out in practice (an infinite weight has no design: PS_DEV_NONFINITE)
-      for (int t = 0; found < 0 && t < Tp && isfinite(wm); ++t)
-        if (passes(t)) found = t;
+      // The first of cand_s[0..n) that passes, -1 if none does; lane l of warp 0 pools for cand_s[l].
+      auto first_passing = [&](int n) {
+        if (wid == 0) nb_s[lane] = lane < n ? pav_stack(w + cand_s[lane], Tp - cand_s[lane], fW + lane, fn + lane) : 0;
+        __syncthreads();
+        for (int l = 0; l < n; ++l)
+          for (int m = tid; m < nb_s[l]; m += kDesignThreads) {
+            const int64_t at = static_cast<int64_t>(m) * kCapLanes + l;
+            fs[at] = __dsqrt_rn(__ddiv_rn(fW[at], static_cast<double>(fn[at])));
+          }
+        __syncthreads();
+        if (wid == 0) {
+          bool ok = false;
+          if (lane < n) {
+            double den = 0.0;
+            for (int64_t m = 0, at = lane; m < nb_s[lane]; ++m, at += kCapLanes)
+              den = __dadd_rn(den, __dmul_rn(static_cast<double>(fn[at]), fs[at]));
+            ok = __ddiv_rn(__dmul_rn(__dsub_rn(Bp, static_cast<double>(cand_s[lane])), fs[lane]), den) <= 1.0;
+          }
+          const unsigned m = __ballot_sync(0xffffffffu, ok);
+          if (lane == 0) found_s = m != 0u ? cand_s[__ffs(m) - 1] : -1;
+        }
+        __syncthreads();
+        return found_s;
+      };
+      int found = -1, from = 0;
+      if (isfinite(wm)) {   // (an infinite weight has no design: PS_DEV_NONFINITE)
+        for (int64_t steps = 0; found < 0 && candidates(from, 1, false) == 1;) {
+          const int t = cand_s[0];
+          steps += Tp - t;
+          if (steps > 2 * static_cast<int64_t>(Tp)) break;
+          if (passes(t)) found = t;
+          from = t + 1;
+        }
+        // (the last prefix always passes, so those clearly above 1 are tried only if the statuses were wrong)
+        for (int above = 0; above < 2 && found < 0; ++above, from = 0)
+          for (int n; found < 0 && (n = candidates(from, kCapLanes, above != 0)) > 0;) {
+            from = cand_s[n - 1] + 1;
+            found = first_passing(n);
+            if (found >= 0) passes(found);   // its blocks
+          }
+      }
       __syncthreads();
       if (found < 0) {
         for (int t = tid; t < Tp; t += kDesignThreads) xi[t] = 1.0;
@@ -1213,9 +1270,9 @@ static DesignWs design_ws(void* ws, int P, int T_max) {
   d.xi = reinterpret_cast<double*>(b);
   b += al256(sizeof(double) * pt);
   d.bW = reinterpret_cast<double*>(b);
-  b += al256(sizeof(double) * pt * 2 * kDesignArrays);
+  b += al256(sizeof(double) * pt * kCapLanes);
   d.bs = reinterpret_cast<double*>(b);
-  b += al256(sizeof(double) * pt * 2 * kDesignArrays);
+  b += al256(sizeof(double) * pt * kCapLanes);
   d.bn = reinterpret_cast<int32_t*>(b);
   return d;
 }
@@ -1223,8 +1280,8 @@ static DesignWs design_ws(void* ws, int P, int T_max) {
 size_t ps_design_cutoffs_workspace_size(int P, int K, int T_max) {
   if (P < 1 || K < 1 || T_max < 1) return 0;
   const size_t pt = static_cast<size_t>(P) * T_max;
-  return kWsHeader + al256(sizeof(double) * pt) * 2 + al256(sizeof(double) * pt * 2 * kDesignArrays) * 2 +
-         al256(sizeof(int32_t) * pt * 2 * kDesignArrays) + al256(sizeof(int64_t) * static_cast<size_t>(P) * K);
+  return kWsHeader + al256(sizeof(double) * pt) * 2 + al256(sizeof(double) * pt * kCapLanes) * 2 +
+         al256(sizeof(int32_t) * pt * kCapLanes) + al256(sizeof(int64_t) * static_cast<size_t>(P) * K);
 }
 
 int ps_design_cutoffs(int P, int K, int T_max, const int32_t* L, const float* gamma_full, const float* u,

@@ -1,0 +1,64 @@
+"""The capped design's search for the saturated prefix, where many prefixes lie on the cap, against the oracle bit for
+bit, and its time beside that of an ordinary trace of the same length (which takes one or two poolings)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import design
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(w, budget, reps=3):
+    """(q, xi, milliseconds) of one prompt of one completion whose scores, and so its weights, are w."""
+    from paper_2606_29758_gb300 import PS_DESIGN_OPTIMIZED, CutoffDesign, DesignShape
+    T = len(w)
+    cd = CutoffDesign(DesignShape(1, 1, T, 8, 32, T, 0))
+    cd.gamma.copy_(torch.from_numpy(w))
+    cd.u.fill_(1.0)
+    L = torch.tensor([T], dtype=torch.int32, device="cuda")
+    ms = []
+    for _ in range(reps):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        cd.design(L, budget, PS_DESIGN_OPTIMIZED)
+        b.record()
+        torch.cuda.synchronize()
+        ms.append(a.elapsed_time(b))
+    cd.check_status()
+    return cd.q.cpu().numpy().view(np.uint64), cd.xi.cpu().numpy(), min(ms)
+
+
+def _ordinary(T):
+    rng = np.random.default_rng(1)
+    return np.exp(0.7 * rng.standard_normal(T) - np.arange(T) / T).astype(np.float32)
+
+
+# (trace, the most poolings' worth of time: an ordinary trace's is 1) at a budget of the whole trace, where every
+# suffix that pools to one block starts at exactly 1
+def _flat_tail(T):            # the first prefix on the cap passes
+    w = _ordinary(T)
+    w[-100:] = 1e-3
+    return w
+
+
+def _rising(T):               # hundreds on the cap, the first of them passes
+    w = _ordinary(T)
+    w[T // 2:] *= np.linspace(3.0, 30.0, T - T // 2, dtype=np.float32)
+    return w
+
+
+def _slow_fall(T):            # every prefix within the band, none passes but the last few
+    return np.linspace(1.0, 1.0 - 3e-6, T).astype(np.float32)
+
+
+@pytest.mark.parametrize("trace,most", [(_flat_tail, 20.0), (_rising, 20.0), (_slow_fall, 1500.0)])
+def test_many_prefixes_on_the_cap(trace, most):
+    T = 1500
+    w = trace(T)
+    q, xi, ms = _run(w, float(T))
+    q_ref, xi_ref = design.design_cutoff_masses(np.array([T], dtype=np.int32), 1, w, np.ones((1, T), np.float32),
+                                                float(T), "optimized")
+    assert np.array_equal(xi, xi_ref)
+    assert np.array_equal(q, q_ref)
+    assert ms < most * _run(_ordinary(T), 100.0)[2], ms
