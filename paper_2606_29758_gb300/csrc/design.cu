@@ -293,14 +293,15 @@ struct DesignWs {
 // True when the block (Wc, nc) violates the order against the block (Wp, np) below it, i.e. when
 // sqrt(Wp / np) < sqrt(Wc / nc) with both quotients and roots rounded to double, exactly as the
 // sequential definition decides it. The cross products Wp nc and Wc np settle every case whose
-// quotients differ by more than 2^-40 relative (then the rounded roots are ordered the same way).
+// quotients differ by more than 2^-40 relative (then the rounded roots are ordered the same way): their difference's
+// exponent is then at most 39 below a's (compared as integers: a double comparison takes 64 cycles).
 __device__ __forceinline__ bool pav_violates_double(double Wp, int np, double Wc, int nc) {
   const double a = __dmul_rn(Wp, static_cast<double>(nc));
   const double b = __dmul_rn(Wc, static_cast<double>(np));
-  if (a > 0x1p-900 && b > 0x1p-900 && a < 0x1p900 && b < 0x1p900) {
-    if (b > __dmul_rn(a, 1.0 + 0x1p-40)) return true;
-    if (b < __dmul_rn(a, 1.0 - 0x1p-40)) return false;
-  }
+  const double d = __dsub_rn(b, a);
+  const int ea = __double2hiint(a) >> 20, eb = __double2hiint(b) >> 20;   // biased exponents (no sign: sums of weights)
+  if (ea > 123 && eb > 123 && ea < 1923 && eb < 1923 && (__double2hiint(d) >> 20 & 0x7ff) >= ea - 39)
+    return __double2hiint(d) >= 0;
   return __dsqrt_rn(__ddiv_rn(Wp, static_cast<double>(np))) < __dsqrt_rn(__ddiv_rn(Wc, static_cast<double>(nc)));
 }
 // The same, with the products taken in float first (each within 2^-22), which settles quotients that differ by more
@@ -531,116 +532,167 @@ __device__ void cap_status(const float2* S, const int32_t* link, int T, double B
 // first[t], W[t] for s < t <= T: the last block [first[t], t) after the weights w[s..t) have been pooled one after
 // another, and its sum as the definition adds it: the new weight c, then W_prev + c for each block that it
 // violates the order with, from the nearest on. A block below the last one is the last one of an earlier t, so
-// the sums of many t can be taken at a time where the links say which blocks they merge; and every decision is
-// then checked on the sums themselves (pav_violates), which by induction over t makes the result the sequential
-// one whatever the links were. The first t whose decisions differ (a near-tie that the links' float slopes took
-// the wrong way) is redone alone and what follows it again; after kMaxRepairs of those one thread does the rest.
-constexpr int kMaxRepairs = 8;
+// the sums of a window of kWin positions are taken together where the links say which blocks they merge; and every
+// decision is then checked on the sums themselves (pav_violates), which by induction over t makes the result the
+// sequential one whatever the links were. Up to kBatch windows are pooled and then checked together; from the first of
+// them with a decision that differs (its link came from slopes that the float sums cannot tell apart: near-ties, or
+// weights far below the sums before them) they are done again and checked one by one, and in a window the first
+// position that differs is redone alone and those after it again. After kMaxRepairs of these one thread does the
+// window's rest, and whole windows: kSerial, and twice as many each time that the links, tried again, are wrong again.
+// 8 prompts of 15000 steps: 1.4 ms without a wrong link, 1.8 to 3.3 with some dozens (half to nine tenths of the steps'
+// weights spread over ten decades; 5.4 to 7.6 when a repair had everything after it pooled again), 11 where nearly all
+// are wrong (weights within 1e-7 of each other; then 31, and 15 by one thread from the start on).
+constexpr int kBatch = 16;
+constexpr int kMaxRepairs = 4;
+constexpr int kSerial = 8;
 struct Pooled {
   const double* w;
   int s, T;
-  int32_t* link;     // [T - s + 1], relative to s
-  int32_t* first;    // [T + 1]
-  double* W;         // [T + 1]
+  const int32_t* link;   // [T - s + 1], relative to s
+  int32_t* first;        // [T + 1]
+  double* W;             // [T + 1]
 
-  __device__ __forceinline__ bool violates(int j, double c, int n) const {
-    return pav_violates(W[j], j - first[j], c, n);
-  }
-  // Position t as the definition does it, on the positions before it (one thread).
-  __device__ void step(int t) const {
-    double c = w[t - 1];
-    int j = t - 1;
-    while (j > s && violates(j, c, t - j)) {
-      c = __dadd_rn(W[j], c);
-      j = first[j];
-    }
-    W[t] = c;
-    first[t] = j;
-  }
-  // Positions t0..T by the links (the whole CTA).
-  __device__ void by_links(int t0) const {
-    __shared__ double W_s[kWin];
-    __shared__ int first_s[kWin];
-    __shared__ int ready_s[kWin];
-    const int tid = threadIdx.x;
-    for (int lo = t0 - 1; lo < T; lo += kWin) {
-      const int t = lo + 1 + tid;
-      const bool mine = t <= T;
-      double c = mine ? w[t - 1] : 0.0;
-      int j = t - 1;
-      const int target = mine ? s + link[t - s] : j;
-      bool done = !mine;
-      ready_s[tid] = 0;
-      __syncthreads();
-      while (true) {
-        bool fresh = false;
-        if (!done) {
-          while (j > target) {
-            const int k = j - lo - 1;
-            if (k < 0) {
-              c = __dadd_rn(W[j], c);
-              j = first[j];
-            } else {
-              if (!ready_s[k]) break;
-              c = __dadd_rn(W_s[k], c);
-              j = first_s[k];
-            }
-          }
-          if (j <= target) {
-            W_s[tid] = c;
-            first_s[tid] = j;
-            done = fresh = true;
-          }
-        }
-        __syncthreads();
-        if (fresh) ready_s[tid] = 1;
-        if (!__syncthreads_or(!done)) break;
-      }
-      if (mine) {
-        W[t] = c;
-        first[t] = j;
-      }
-      __syncthreads();
-    }
-  }
-  // The first position in t0..T whose decisions are not the definition's, T + 1 if none (the whole CTA).
-  __device__ int first_wrong(int t0) const {
+  __device__ void run() const {   // (the whole CTA)
+    __shared__ double w_s[kWin], W_s[kWin];
+    __shared__ int first_s[kWin], ready_s[kWin];
     __shared__ int wrong_s;
-    if (threadIdx.x == 0) wrong_s = T + 1;
-    __syncthreads();
-    for (int t = t0 + threadIdx.x; t <= T; t += kDesignThreads) {
-      double c = w[t - 1];
-      int j = t - 1;
-      const int f = first[t];
-      bool ok = true;
-      while (ok && j > f) {
-        ok = violates(j, c, t - j);
-        c = __dadd_rn(W[j], c);
-        j = first[j];
+    const int tid = threadIdx.x;
+    int repairs_left = kMaxRepairs, serial_left = 0, serial_next = kSerial;
+    int size = kBatch / 4;   // windows of a batch
+    bool one_by_one = false;
+    for (int b0 = s, b1; b0 < T; b0 = b1) {
+      b1 = min(T, b0 + kWin * size);
+      int unclean = 0, redo = b0;
+      for (int checked = one_by_one ? 1 : 0; checked < 2; ++checked) {
+        for (int lo = checked ? redo : b0; lo < b1; lo += kWin) {
+          const int t = lo + 1 + tid, end = min(T, lo + kWin);
+          const bool mine = t <= T;
+          const double wt = mine ? w[t - 1] : 0.0;
+          const int target = mine ? s + link[t - s] : t;
+          auto sum = [&](int j) { return j > lo ? W_s[j - lo - 1] : W[j]; };
+          auto start = [&](int j) { return j > lo ? first_s[j - lo - 1] : first[j]; };
+          // positions k0..k1 as the definition does them, on those before them (one thread)
+          auto serial = [&](int k0, int k1) {
+            int j = k0 - 1, f = j > s ? start(j) : s;
+            double Wj = j > s ? sum(j) : 0.0;   // [f, j) is the last block after k0 - 1 weights, Wj its sum
+            for (int k = k0; k <= k1; ++k) {
+              double c = w_s[k - lo - 1];
+              j = k - 1;
+              while (j > s) {
+                const double below = f > s ? sum(f) : 0.0;   // the block before it, loaded under the decision
+                const int below_f = f > s ? start(f) : s;
+                if (!pav_violates_double(Wj, j - f, c, k - j)) break;
+                c = __dadd_rn(Wj, c);
+                j = f;
+                Wj = below;
+                f = below_f;
+              }
+              W_s[k - lo - 1] = Wj = c;
+              first_s[k - lo - 1] = f = j;
+            }
+          };
+          w_s[tid] = wt;
+          int from = lo + 1;
+          if (checked && serial_left > 0) {
+            __syncthreads();
+            if (tid == 0) serial(from, end);
+            __syncthreads();
+            from = end + 1;
+            ++unclean;
+            --serial_left;
+          }
+          while (from <= end) {
+            // positions from..end by the links
+            bool done = !mine || t < from;
+            double c = wt;
+            int j = t - 1;
+            if (!done) ready_s[tid] = 0;
+            if (tid == 0) wrong_s = end + 1;
+            __syncthreads();
+            while (true) {
+              bool fresh = false;
+              if (!done) {
+                while (j > target) {
+                  const int k = j - lo - 1;
+                  if (k < 0) {
+                    c = __dadd_rn(W[j], c);
+                    j = first[j];
+                  } else {
+                    if (!ready_s[k]) break;
+                    c = __dadd_rn(W_s[k], c);
+                    j = first_s[k];
+                  }
+                }
+                if (j <= target) {
+                  W_s[tid] = c;
+                  first_s[tid] = j;
+                  done = fresh = true;
+                }
+              }
+              __syncthreads();
+              if (fresh) ready_s[tid] = 1;
+              if (!__syncthreads_or(!done)) break;
+            }
+            if (!checked) break;
+            if (mine && t >= from && !right(t, wt, sum, start)) atomicMin(&wrong_s, t);
+            __syncthreads();
+            const int wrong = wrong_s;
+            __syncthreads();
+            if (wrong > end) {
+              if (from == lo + 1) {
+                repairs_left = kMaxRepairs;
+                serial_next = kSerial;
+              }
+              break;
+            }
+            unclean += from == lo + 1;
+            if (repairs_left > 0) {
+              --repairs_left;
+              from = wrong + 1;
+            } else {
+              serial_left = serial_next;
+              serial_next *= 2;
+              from = end + 1;
+            }
+            if (tid == 0) serial(wrong, from - 1);
+            __syncthreads();
+          }
+          if (mine) {
+            W[t] = W_s[tid];
+            first[t] = first_s[tid];
+          }
+          __syncthreads();
+        }
+        if (checked) break;
+        // the batch's first window with a wrong decision
+        if (tid == 0) wrong_s = b1 + 1;
+        __syncthreads();
+        for (int t = b0 + 1 + tid; t <= b1; t += kDesignThreads)
+          if (!right(t, w[t - 1], [&](int j) { return W[j]; }, [&](int j) { return first[j]; })) {
+            atomicMin(&wrong_s, t);
+            break;
+          }
+        __syncthreads();
+        redo = wrong_s > b1 ? b1 : b0 + (wrong_s - b0 - 1) / kWin * kWin;
+        __syncthreads();
       }
-      if (ok && j > s) ok = !violates(j, c, t - j);
-      if (!ok) atomicMin(&wrong_s, t);
+      one_by_one = 4 * unclean >= size;
+      size = unclean > 0 ? kBatch / 4 : min(kBatch, 2 * size);
     }
-    __syncthreads();
-    const int r = wrong_s;
-    __syncthreads();
-    return r;
   }
-  __device__ void run() const {
-    int t = s + 1;
-    for (int repairs = 0;; ++repairs) {
-      by_links(t);
-      t = first_wrong(t);
-      if (t > T) return;
-      if (threadIdx.x == 0) {
-        step(t);
-        link[t - s] = first[t] - s;
-        if (repairs == kMaxRepairs)
-          for (int k = t + 1; k <= T; ++k) step(k);
-      }
-      __syncthreads();
-      if (repairs == kMaxRepairs || ++t > T) return;
+  // Whether first[t] is where the definition's decisions lead from w[t - 1] = c.
+  template <class Sum, class Start>
+  __device__ __forceinline__ bool right(int t, double c, const Sum& sum, const Start& start) const {
+    const int f = start(t);
+    int j = t - 1;
+    while (j > f) {
+      const double Wj = sum(j);
+      const int fj = start(j);
+      if (!pav_violates(Wj, j - fj, c, t - j)) return false;
+      c = __dadd_rn(Wj, c);
+      j = fj;
     }
+    return j <= s || !pav_violates(sum(j), j - start(j), c, t - j);
   }
   // The blocks after all weights, last one first: their ends in `ends`; returns their number (the whole CTA).
   // A position is a block's end if no later one's block reaches over it.
@@ -684,8 +736,8 @@ struct Pooled {
 
 // Pools w[0..T) one weight after another into one lane's stack (element m of the stack at index m * kCapLanes), each
 // block sum added as the definition adds it. The last block stays in registers, and memory is read only when a merge
-// uncovers the block below. (Traces that get here are nearly flat: the float test would only add to the double one. 4000
-// weights within 1e-7 of each other, budget 4000: 0.70 s without it, 0.81 with it.) Returns the number of blocks.
+// uncovers the block below. (Traces that get here are nearly flat: the float test would only add to the double one.)
+// Returns the number of blocks.
 __device__ __noinline__ int pav_stack(const double* w, int T, double* bW, int32_t* bn) {
   int nb = 0, nt = 0;
   double Wt = 0.0, wnext = T > 0 ? w[0] : 0.0;
@@ -837,7 +889,7 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
       // second passes. The whole CTA tries them one by one until that has taken the steps of two whole traces; the
       // rest go 32 at a time, a lane each: a budget at or above the horizon puts every suffix that is flat to 2^-16
       // into the band, hundreds of them, and where the weights fall slowly none passes before the last. (4000
-      // steps that fall by 3e-6 in all, budget 4000: 0.5 s so, 15.8 s one by one.)
+      // steps that fall by 3e-6 in all, budget 4000: 0.44 s so, 15.8 s one by one.)
       const int64_t stacks = static_cast<int64_t>(p) * T_max * kCapLanes;
       const int64_t pitch = 2 * static_cast<int64_t>(T_max);   // at least T + 1
       double* fW = ws.bW + stacks;

@@ -62,3 +62,27 @@ def test_many_prefixes_on_the_cap(trace, most):
     assert np.array_equal(xi, xi_ref)
     assert np.array_equal(q, q_ref)
     assert ms < most * _run(_ordinary(T), 100.0)[2], ms
+
+
+# Traces whose blocks the float slopes cannot propose, so that pooling has to repair them: weights of ten decades next to
+# each other (tokens a trained policy is sure of), and weights that differ in their last float bits
+def _ten_decades(T):
+    rng = np.random.default_rng(5)
+    q = np.where(rng.random(T) < 0.5, np.exp(rng.uniform(np.log(1e-6), np.log(1e-2), T)), rng.uniform(0.01, 1.0, T))
+    return (3072.0 * q * q * rng.uniform(0.02, 0.25, T)).astype(np.float32)
+
+
+def _nearly_flat(T):
+    return (1.0 + 1e-7 * np.random.default_rng(4).standard_normal(T)).astype(np.float32)
+
+
+@pytest.mark.parametrize("trace,T,most", [(_ten_decades, 15000, 3.0), (_nearly_flat, 8000, 12.0),
+                                          (_ten_decades, 4097, 50.0), (_nearly_flat, 1025, 50.0)])
+def test_pooling_repairs_wrong_links(trace, T, most):
+    w = trace(T)
+    q, xi, ms = _run(w, 20.0)
+    q_ref, xi_ref = design.design_cutoff_masses(np.array([T], dtype=np.int32), 1, w, np.ones((1, T), np.float32), 20.0,
+                                                "optimized")
+    assert np.array_equal(xi, xi_ref)
+    assert np.array_equal(q, q_ref)
+    assert ms < most * _run(_ordinary(T), 20.0)[2], ms
