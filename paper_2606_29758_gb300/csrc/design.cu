@@ -321,13 +321,17 @@ __device__ __forceinline__ bool pav_violates(double Wp, int np, double Wc, int n
 struct FF {
   float hi, lo;
 };
+__device__ __forceinline__ FF two_sum(float a, float b) {
+  const float s = a + b;
+  const float bb = s - a;
+  return FF{s, (a - (s - bb)) + (b - bb)};
+}
 __device__ __forceinline__ FF ff_add(FF a, FF b) {
   const float lo = a.lo + b.lo;
-  const float s = a.hi + b.hi;
-  const float bb = s - a.hi;
-  const float e = ((a.hi - (s - bb)) + (b.hi - bb)) + lo;
-  const float h = s + e;
-  return FF{h, e - (h - s)};
+  const FF s = two_sum(a.hi, b.hi);
+  const float e = s.lo + lo;
+  const float h = s.hi + e;
+  return FF{h, e - (h - s.hi)};
 }
 __device__ __forceinline__ FF ff_select(bool c, FF a, FF b) { return FF{c ? a.hi : b.hi, c ? a.lo : b.lo}; }
 
@@ -358,12 +362,15 @@ constexpr int kWin = kDesignThreads;
 constexpr int kHullSmem = 14336;       // hull vertices in shared memory (deeper ones in the workspace)
 constexpr size_t kDesignDynSmem = kHullSmem * (sizeof(float2) + sizeof(int32_t));
 
-// S[u], u = 0..n: the sums of the first u values (float-float), times sign. value(i) is the i-th one.
+// S[u], u = 0..n: the sums of the first u values (float-float), times sign. value(i) is the i-th one. The sums before a
+// window are carried in three floats, so that what a sum is off by does not grow with the windows before it: 2^-47
+// relative, measured up to 2^22 values of one size or of eleven decades (in two floats, warp after warp: 2^-45 at 2^14
+// values and 2^-41 at 2^22). At most it is the 14 float-float additions behind it, 2^-46 each.
 template <class F>
 __device__ void ff_prefix_sums(F value, int n, float sign, float2* S) {
   __shared__ float2 warp_s[kDesignWarps];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  FF carry{0.f, 0.f};
+  float c0 = 0.f, c1 = 0.f, c2 = 0.f;
   if (tid == 0) S[0] = make_float2(0.f, 0.f);
   for (int i0 = 0; i0 < n; i0 += kDesignThreads) {
     const int i = i0 + tid;
@@ -376,14 +383,20 @@ __device__ void ff_prefix_sums(F value, int n, float sign, float2* S) {
     }
     if (lane == 31) warp_s[wid] = make_float2(v.hi, v.lo);
     __syncthreads();
-    FF before = carry;
+    FF before{0.f, 0.f}, all{0.f, 0.f};   // the window's sums before this warp, and the whole window's
     for (int k = 0; k < kDesignWarps; ++k) {
-      const FF x{warp_s[k].x, warp_s[k].y};
-      if (k < wid) before = ff_add(before, x);
-      carry = ff_add(carry, x);
+      if (k == wid) before = all;
+      all = ff_add(all, FF{warp_s[k].x, warp_s[k].y});
     }
-    v = ff_add(before, v);
+    v = ff_add(FF{c0, c1}, ff_add(before, v));
     if (i < n) S[i + 1] = make_float2(sign * v.hi, sign * v.lo);
+    // (c0, c1, c2) += all: TwoSums down the three floats, then renormalised
+    const FF s0 = two_sum(c0, all.hi), s1 = two_sum(c1, all.lo), s2 = two_sum(s1.hi, s0.lo);
+    c2 += s1.lo + s2.lo;
+    c0 = s0.hi + s2.hi;
+    const float r = s2.hi - (c0 - s0.hi);
+    c1 = r + c2;
+    c2 -= c1 - r;
     __syncthreads();
   }
 }
@@ -479,8 +492,10 @@ __device__ void hull_links(const float2* S, int n, int32_t* link, float2* hull_S
 // whether g(t) is clearly above 1 (0), clearly below (2) or within kCapBand of 1 (1); all but the first kind are then
 // decided by the exact rounded sequence of the definition, in increasing order, until one passes.
 // The first block's mean is the largest slope from t, hence at least Q_t / (T - t) with Q_t the sum of the
-// suffix, of which the float-float sums are off by 2^-45: its weight is off by 2^-45 (T - t) / n relative, 2^-21 at
-// the largest T. Roots, products and the comparison add a few 2^-24: far inside kCapBand.
+// suffix. A float-float sum is off by 2^-42 of itself at most (ff_prefix_sums), so the block's weight, the difference of
+// two, by 2^-41 (T - t) / n relative: 2^-17 at the largest T of 2^24 (2^-22 with the 2^-47 that is measured), 2^-27 at
+// 2^14. Its root halves that; D, an addition per window, is off by 2^-30, and roots, products and the comparison add a
+// few 2^-24: inside kCapBand at every T.
 constexpr double kCapBand = 0x1p-16;
 
 // S, link: of the weights from the right, u = T - t, S negated. D [T + 1] scratch.

@@ -86,3 +86,15 @@ def test_pooling_repairs_wrong_links(trace, T, most):
     assert np.array_equal(xi, xi_ref)
     assert np.array_equal(q, q_ref)
     assert ms < most * _run(_ordinary(T), 20.0)[2], ms
+
+
+@pytest.mark.parametrize("trace", [_ordinary, _ten_decades])
+@pytest.mark.parametrize("T", [(1 << 18) + 3, 1 << 20])
+def test_long_traces(trace, T):
+    # sums over a thousand windows and more; a small budget, so that the oracle pools once
+    w = trace(T)
+    q, xi, _ = _run(w, 5.0, reps=1)
+    q_ref, xi_ref = design.design_cutoff_masses(np.array([T], dtype=np.int32), 1, w, np.ones((1, T), np.float32), 5.0,
+                                                "optimized")
+    assert np.array_equal(xi, xi_ref)
+    assert np.array_equal(q, q_ref)
