@@ -554,12 +554,13 @@ __device__ void cap_status(const float2* S, const int32_t* link, int T, double B
 // weights far below the sums before them) they are done again and checked one by one, and in a window the first
 // position that differs is redone alone and those after it again. After kMaxRepairs of these one thread does the
 // window's rest, and whole windows: kSerial, and twice as many each time that the links, tried again, are wrong again.
-// 8 prompts of 15000 steps: 1.4 ms without a wrong link, 1.8 to 3.3 with some dozens (half to nine tenths of the steps'
-// weights spread over ten decades; 5.4 to 7.6 when a repair had everything after it pooled again), 11 where nearly all
-// are wrong (weights within 1e-7 of each other; then 31, and 15 by one thread from the start on).
+// 8 prompts of 15000 steps: 1.4 ms without a wrong link, 1.6 to 2.0 with some dozens (half to nine tenths of the steps'
+// weights spread over ten decades; 5.4 to 7.6 when a repair had everything after it pooled again, and with 4 repairs
+// and 8 windows 1.7 to 6.0), 11 where nearly all are wrong (weights within 1e-7 of each other; then 31, and 15 by one
+// thread from the start on).
 constexpr int kBatch = 16;
-constexpr int kMaxRepairs = 4;
-constexpr int kSerial = 8;
+constexpr int kMaxRepairs = 12;
+constexpr int kSerial = 2;
 struct Pooled {
   const double* w;
   int s, T;
