@@ -1,8 +1,8 @@
 /*
  * psppo_diag.h -- diagnostic entry points of libpsppo.
  *
- * The paper has no counterpart for these: they expose, for tests, the two pieces
- * of machinery that the update pass is built on. Conventions (device pointers,
+ * The paper has no counterpart for these: they expose, for tests, pieces of
+ * machinery that the update pass is built on. Conventions (device pointers,
  * workspace status word, stream ordering, ps_status returns) are those of psppo.h.
  */
 #ifndef PSPPO_DIAG_H_
@@ -29,6 +29,14 @@ extern "C" {
 int ps_diag_gemm_bf16(int M, int N, int K, int a_mn_major, int b_mn_major, const void* A, int64_t lda,
                       const void* B, int64_t ldb, float* C, int64_t ldc, int accumulate, int variant,
                       void* ws, size_t ws_bytes, ps_stream_t stream);
+
+/*
+ * How the backward cuts the K loop of an M x N product of num_kb blocks of 64 over the CTAs of a cluster, on a device
+ * of `sms` SMs that runs `pairs`, `fours` and `eights` clusters of 2, 4 and 8 CTAs at once (0: none fits). *ranks: CTAs
+ * per output tile, 1 if the loop is not cut; *halves: the tile's height in 128 rows. Host only.
+ */
+int ps_diag_choose_splitk(int64_t M, int64_t N, int num_kb, int narrow_too, int sms, int pairs, int fours, int eights,
+                          int* ranks, int* halves);
 
 /*
  * Launch one CTA that waits on a shared-memory barrier that nothing ever completes,

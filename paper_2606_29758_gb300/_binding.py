@@ -34,7 +34,7 @@ EXPORTS = [
     "ps_lmhead_ppo_fwd_from_stats_workspace_size", "ps_lmhead_ppo_fwd_from_stats", "ps_lmhead_ppo_bwd_vocab_shard",
     "ps_lmhead_logit_store_size", "ps_lmhead_ppo_fwd_store", "ps_lmhead_ppo_bwd_from_store_workspace_size",
     "ps_lmhead_ppo_bwd_from_store", "ps_lmhead_logit_stats_store", "ps_lmhead_ppo_bwd_vocab_shard_from_store",
-    "ps_diag_gemm_bf16", "ps_diag_wait_timeout", "ps_lmhead_ppo_fwd_noalloc",
+    "ps_diag_gemm_bf16", "ps_diag_choose_splitk", "ps_diag_wait_timeout", "ps_lmhead_ppo_fwd_noalloc",
     "ps_lmhead_score_proxy_workspace_size", "ps_lmhead_score_proxy",
     "ps_design_cutoffs_workspace_size", "ps_design_cutoffs",
     "ps_reward_uncertainty_workspace_size", "ps_reward_uncertainty", "ps_binarize_rewards",
@@ -98,6 +98,7 @@ _SIGS = {
                                                         _vp, _vp, _sz, _vp, _vp, _i32, _vp, _sz, _vp]),
     "ps_diag_gemm_bf16": (_i32, [_i32, _i32, _i32, _i32, _i32, _vp, _i64, _vp, _i64, _vp, _i64, _i32, _i32, _vp, _sz,
                                  _vp]),
+    "ps_diag_choose_splitk": (_i32, [_i64, _i64, _i32, _i32, _i32, _i32, _i32, _i32, _vp, _vp]),
     "ps_diag_wait_timeout": (_i32, [_u64, _vp, _sz, _vp]),
     "ps_lmhead_score_proxy_workspace_size": (_sz, [_i64, _i32, _i32, _i32, _i32]),
     "ps_lmhead_score_proxy": (_i32, [_i64, _i32, _i32, _i32, _vp, _vp, _vp, _vp, _vp, _i32, _vp, _vp, _vp, _sz,
@@ -367,6 +368,15 @@ def ps_diag_gemm_bf16(M, N, K, a_mn_major, b_mn_major, A, lda, B, ldb, C, ldc, a
     rc = lib().ps_diag_gemm_bf16(M, N, K, int(a_mn_major), int(b_mn_major), _ptr(A), lda, _ptr(B), ldb, _ptr(C), ldc,
                                  int(accumulate), int(variant), _ptr(ws), _nbytes(ws), _stream(stream))
     _check(rc, "ps_diag_gemm_bf16")
+
+
+def ps_diag_choose_splitk(M, N, num_kb, narrow_too, sms, at_once):
+    """(ranks, halves) for clusters of 2, 4 and 8 CTAs of which at_once run at a time."""
+    ranks, halves = ctypes.c_int(0), ctypes.c_int(0)
+    rc = lib().ps_diag_choose_splitk(M, N, num_kb, int(narrow_too), sms, *at_once, ctypes.byref(ranks),
+                                     ctypes.byref(halves))
+    _check(rc, "ps_diag_choose_splitk")
+    return ranks.value, halves.value
 
 
 def ps_diag_wait_timeout(timeout_ns, ws, stream=None):

@@ -66,6 +66,12 @@ int bwd_chunk_f32(int64_t rc, int d, int V, const float* Hpk, const float* W, co
                   const float* lse, const float* coef, float* dH, float* dW, int dw_accumulate, float* dz,
                   int64_t ldz, uint32_t* status, cudaStream_t s, int tok_base, int dh_accumulate, int64_t n_call, int64_t v_call, bool clear);
 
+// CTAs of a cluster per output tile of the split-K product (1: not split) and the tile's height in 128-row halves.
+struct SplitK {
+  int ranks, halves;
+};
+SplitK choose_splitk(int64_t M, int64_t N, int num_kb, bool narrow_too, int sms, const int (&at_once)[3]);
+
 // Plain tensor-core GEMM (test hook): C[M][N] (+)= sum_k A(m,k) B(k,n), f32 out. variant: 0 one
 // CTA per 128 x 256 tile, 1 a CTA pair per 256 x 256 tile, 2 one CTA per 256 x 256 tile.
 int gemm_bf16(int M, int N, int K, int a_mn, int b_mn, const void* A, int64_t lda, const void* B, int64_t ldb,

@@ -537,17 +537,17 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+// The driver's function of this name, nullptr if it has none.
+static void* driver_fn(const char* name) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  return cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+                 q == cudaDriverEntryPointSuccess
+             ? p
+             : nullptr;
+}
 static EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  });
+  static const EncodeTiledFn fn = reinterpret_cast<EncodeTiledFn>(driver_fn("cuTensorMapEncodeTiled"));
   return fn;
 }
 
@@ -655,16 +655,19 @@ static int launch_gemm_pair(const CUtensorMap& ta, const CUtensorMap& tb, int64_
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }
 
-// Clusters of `ranks` CTAs of the split-K kernel that run at once (one CTA per SM; a cluster stays inside
-// a GPC, so 152 SMs hold 76 pairs but 36 clusters of four and 16 of eight). Asked once per device.
-static int splitk_clusters_at_once(int ranks) {
-  constexpr int kDevices = 64;
-  static std::atomic<int> known[kDevices][4];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return num_sms_current() / (ranks + 1);
-  std::atomic<int>& slot = known[dev][ranks == 2 ? 1 : ranks == 4 ? 2 : 3];
-  int n = slot.load(std::memory_order_relaxed);
-  if (n > 0) return n;
+// Clusters of 2 << i CTAs of the split-K kernel that run at once in the current context (one CTA per SM; a cluster
+// stays inside a GPC, so 152 SMs hold 76 pairs but 36 clusters of four and 16 of eight), 0 where none fits. Asked once
+// per context, which has its own set of SMs; a slot holds (context id, answer + 1) in one word.
+static int splitk_clusters_at_once(int i) {
+  constexpr int kSlots = 64;
+  static std::atomic<uint64_t> known[kSlots][3];
+  static const auto ctx_id = reinterpret_cast<CUresult (*)(CUcontext, unsigned long long*)>(driver_fn("cuCtxGetId"));
+  unsigned long long id = 0;
+  const bool have_id = ctx_id != nullptr && ctx_id(nullptr, &id) == CUDA_SUCCESS;
+  std::atomic<uint64_t>& slot = known[id % kSlots][i];
+  const uint64_t word = slot.load(std::memory_order_relaxed);
+  if (have_id && (word & 0xffff) != 0 && word >> 16 == id) return static_cast<int>(word & 0xffff) - 1;
+  const int ranks = 2 << i;
   auto kern = umma_gemm_splitk_kernel<false, true, 2>;
   constexpr size_t smem = sizeof(GemmSplitSmem<2>) + 1024;
   cudaLaunchConfig_t cfg = {};
@@ -678,12 +681,13 @@ static int splitk_clusters_at_once(int ranks) {
   cfg.dynamicSmemBytes = smem;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  int n = 0;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(kern), &cfg) != cudaSuccess || n <= 0) {
+      cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(kern), &cfg) != cudaSuccess || n < 0) {
     cudaGetLastError();
-    n = num_sms_current() / (ranks + 1);
+    n = 0;
   }
-  slot.store(n, std::memory_order_relaxed);
+  if (have_id) slot.store(static_cast<uint64_t>(id) << 16 | static_cast<uint64_t>(n + 1), std::memory_order_relaxed);
   return n;
 }
 
@@ -699,12 +703,9 @@ static int splitk_clusters_at_once(int ranks) {
 // rows, d = 3584, V = 32000: 172 us with 8 ranks, 158 with 2). From two wide tiles per SM on the persistent kernel's
 // last round costs less than a third, and the split is off, so that whole batches and their shards (hundreds of
 // tiles each) add dH up in the same order.
-struct SplitK {
-  int ranks, halves;
-};
-// narrow_too: the unsplit product may run on 128-row tiles (54 hundredths a k-block).
-static SplitK choose_splitk(int64_t M, int64_t N, int num_kb, bool narrow_too) {
-  const int sms = num_sms_current();
+// narrow_too: the unsplit product may run on 128-row tiles (54 hundredths a k-block). at_once: clusters of 2, 4 and 8 CTAs
+// that run at once, 0 where that size is not to be had.
+SplitK choose_splitk(int64_t M, int64_t N, int num_kb, bool narrow_too, int sms, const int (&at_once)[3]) {
   const int64_t nb = (N + kBN - 1) / kBN;
   const int64_t tiles[3] = {0, (M + kBM - 1) / kBM * nb, (M + 2 * kBM - 1) / (2 * kBM) * nb};
   SplitK best{1, 2};
@@ -712,9 +713,10 @@ static SplitK choose_splitk(int64_t M, int64_t N, int num_kb, bool narrow_too) {
   int64_t best_cost = (tiles[2] + sms - 1) / sms * num_kb * 100;
   if (narrow_too) best_cost = std::min(best_cost, (tiles[1] + sms - 1) / sms * num_kb * 54);
   for (int halves = 2; halves >= 1; --halves)
-    for (int S = 2; S <= 8 && S <= num_kb; S *= 2) {
-      const int64_t at_once = splitk_clusters_at_once(S);
-      const int64_t c = (tiles[halves] + at_once - 1) / at_once *
+    for (int i = 0; i < 3 && 2 << i <= num_kb; ++i) {
+      if (at_once[i] < 1) continue;
+      const int S = 2 << i;
+      const int64_t c = (tiles[halves] + at_once[i] - 1) / at_once[i] *
                         ((num_kb + S - 1) / S * (halves == 2 ? 100 : 54) + (halves == 2 ? 1200 : 700));
       if (c * 100 < best_cost * 97) {
         best = SplitK{S, halves};
@@ -722,6 +724,12 @@ static SplitK choose_splitk(int64_t M, int64_t N, int num_kb, bool narrow_too) {
       }
     }
   return best;
+}
+static SplitK choose_splitk_here(int64_t M, int64_t N, int num_kb, bool narrow_too) {
+  const int sms = num_sms_current();
+  int at_once[3];
+  for (int i = 0; i < 3; ++i) at_once[i] = splitk_clusters_at_once(i);
+  return choose_splitk(M, N, num_kb, narrow_too, sms, at_once);
 }
 
 template <bool A_MN, bool B_MN, int HALVES>
@@ -733,11 +741,12 @@ static int launch_gemm_splitk(const CUtensorMap& ta, const CUtensorMap& tb, int6
   constexpr size_t smem = sizeof(GemmSplitSmem<HALVES>) + 1024;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
     return PS_ERR_CUDA;
-  return launch_after(kern, dim3(static_cast<unsigned>(m_blocks * n_blocks * ranks)), kSplitThreads, smem, s,
-                      static_cast<unsigned>(ranks), 1, true, ta, tb, n_blocks, static_cast<int>((K + kBK - 1) / kBK), o,
-                      status, kDefaultTimeoutNs) == cudaSuccess
-             ? PS_OK
-             : PS_ERR_CUDA;
+  if (launch_after(kern, dim3(static_cast<unsigned>(m_blocks * n_blocks * ranks)), kSplitThreads, smem, s,
+                   static_cast<unsigned>(ranks), 1, true, ta, tb, n_blocks, static_cast<int>((K + kBK - 1) / kBK), o,
+                   status, kDefaultTimeoutNs) == cudaSuccess)
+    return PS_OK;
+  cudaGetLastError();
+  return PS_ERR_CUDA;
 }
 
 int fwd_tile_splits_bf16(int V) { return (V + kBN - 1) / kBN; }
@@ -952,16 +961,19 @@ int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, flo
     if (!map_kmajor(&ta, dz, rc, V, ldz, 2 * kBM) || !map_mnmajor(&tb, W, V, d, d) || !map_out_f32(&tc, dH, rc, d, d))
       return PS_ERR_INVALID_ARG;
     StoreF32Epi::Params ep{d, dh_accumulate};
-    const SplitK split = choose_splitk(n_call, d, (V + kBK - 1) / kBK, false);
+    const SplitK split = choose_splitk_here(n_call, d, (V + kBK - 1) / kBK, false);
+    rcode = PS_ERR_CUDA;
     if (split.ranks > 1) {
       const SplitOut o{dH, d, static_cast<int>(rc), d, dh_accumulate};
       if (split.halves == 2) {
         rcode = launch_gemm_splitk<false, true, 2>(ta, tb, rc, d, V, split.ranks, o, status, s);
       } else {
-        if (!map_kmajor(&ta, dz, rc, V, ldz, kBM)) return PS_ERR_INVALID_ARG;
-        rcode = launch_gemm_splitk<false, true, 1>(ta, tb, rc, d, V, split.ranks, o, status, s);
+        CUtensorMap half;
+        if (!map_kmajor(&half, dz, rc, V, ldz, kBM)) return PS_ERR_INVALID_ARG;
+        rcode = launch_gemm_splitk<false, true, 1>(half, tb, rc, d, V, split.ranks, o, status, s);
       }
-    } else
+    }
+    if (rcode != PS_OK)   // not split, or the stream's SMs do not take such a cluster
       rcode = launch_gemm_single<false, true, StoreF32Epi, 2>(ta, tb, tc, rc, d, V, 0, kBandGrad, ep, status, s);
     if (rcode != PS_OK) return rcode;
   }
@@ -971,13 +983,14 @@ int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, flo
       return PS_ERR_INVALID_ARG;
     StoreF32Epi::Params ep{d, dw_accumulate};
     const int kb = static_cast<int>((rc + kBK - 1) / kBK);
-    const SplitK split = choose_splitk(v_call, d, kb, true);
+    const SplitK split = choose_splitk_here(v_call, d, kb, true);
     if (split.ranks > 1) {
       // a small vocabulary has few tiles, and many rows as their K loop: 8000 rows, d = 128, V = 1024 47 us unsplit, 14
       // split; d = 392, V = 2000 65 / 27; 100000 rows 737 / 256; d = 128, V = 9000 53 / 37
       const SplitOut o{dW, d, V, d, dw_accumulate};
-      return split.halves == 2 ? launch_gemm_splitk<true, true, 2>(ta, tb, V, d, rc, split.ranks, o, status, s)
-                               : launch_gemm_splitk<true, true, 1>(ta, tb, V, d, rc, split.ranks, o, status, s);
+      rcode = split.halves == 2 ? launch_gemm_splitk<true, true, 2>(ta, tb, V, d, rc, split.ranks, o, status, s)
+                                : launch_gemm_splitk<true, true, 1>(ta, tb, V, d, rc, split.ranks, o, status, s);
+      if (rcode == PS_OK) return PS_OK;   // (else as above)
     }
     // dW of 65 to 256 rows (2 to 4 k-blocks) is bound by its stores, which the narrow tile's epilogue overlaps whole
     // with the next tile (200 rows, V = 152064: d = 3584 407 us narrow / 443 wide, d = 1536 183 / 200; 571 rows

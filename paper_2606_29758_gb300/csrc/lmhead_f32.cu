@@ -330,14 +330,16 @@ static int64_t simt_tiles(int64_t M, int64_t N) {
 template <class Cfg, bool A_K, bool B_K, class Epi>
 static int launch_simt_cfg(int64_t M, int64_t N, int64_t K, int ranks, Operand A, Operand B,
                            const typename Epi::Params& ep, cudaStream_t s, uint32_t* clear = nullptr) {
-  const dim3 grid(static_cast<unsigned>((N + Cfg::TN - 1) / Cfg::TN), static_cast<unsigned>((M + Cfg::TM - 1) / Cfg::TM),
-                  static_cast<unsigned>(ranks));
+  dim3 grid(static_cast<unsigned>((N + Cfg::TN - 1) / Cfg::TN), static_cast<unsigned>((M + Cfg::TM - 1) / Cfg::TM),
+            static_cast<unsigned>(ranks));
   if constexpr (std::is_same<Epi, SimtStoreEpi>::value) {
-    if (ranks > 1)
-      return launch_after(simt_gemm_kernel<Cfg, A_K, B_K, Epi, true>, grid, Cfg::kThreads, 0, s, 1,
-                          static_cast<unsigned>(ranks), true, M, N, K, A, B, ep, nullptr) == cudaSuccess
-                 ? PS_OK
-                 : PS_ERR_CUDA;
+    if (ranks > 1) {
+      if (launch_after(simt_gemm_kernel<Cfg, A_K, B_K, Epi, true>, grid, Cfg::kThreads, 0, s, 1,
+                       static_cast<unsigned>(ranks), true, M, N, K, A, B, ep, nullptr) == cudaSuccess)
+        return PS_OK;
+      cudaGetLastError();   // the stream's SMs do not take such a cluster: not split
+      grid.z = 1;
+    }
   }
   return launch_after(simt_gemm_kernel<Cfg, A_K, B_K, Epi, false>, grid, Cfg::kThreads, 0, s, 1, 1, clear == nullptr, M, N,
                       K, A, B, ep, clear) == cudaSuccess

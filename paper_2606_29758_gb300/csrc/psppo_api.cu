@@ -1169,6 +1169,16 @@ int ps_diag_gemm_bf16(int M, int N, int K, int a_mn_major, int b_mn_major, const
   return gemm_bf16(M, N, K, a_mn_major, b_mn_major, A, lda, B, ldb, C, ldc, accumulate, variant, status_word(ws), s);
 }
 
+int ps_diag_choose_splitk(int64_t M, int64_t N, int num_kb, int narrow_too, int sms, int pairs, int fours, int eights,
+                          int* ranks, int* halves) {
+  if (M < 1 || N < 1 || num_kb < 1 || sms < 1 || !ranks || !halves) return PS_ERR_INVALID_ARG;
+  const int at_once[3] = {pairs, fours, eights};
+  const SplitK k = choose_splitk(M, N, num_kb, narrow_too != 0, sms, at_once);
+  *ranks = k.ranks;
+  *halves = k.halves;
+  return PS_OK;
+}
+
 int ps_diag_wait_timeout(uint64_t timeout_ns, void* ws, size_t ws_bytes, ps_stream_t stream) {
   if (timeout_ns > 10000000000ull) return PS_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
