@@ -1270,7 +1270,7 @@ int ps_lmhead_score_proxy(int64_t N, int d, int V, int dtype, const void* Hrows,
   float2* tpart = reinterpret_cast<float2*>(base + fixed + sizeof(float4) * static_cast<size_t>(S) * N);
   uint32_t* status = static_cast<uint32_t*>(ws);
   row_sqnorm_kernel<<<num_sms_current() * 8, 256, 0, s>>>(N, d, 1, Hrows, hn, status);
-  if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
+  if (cudaGetLastError() != cudaSuccess) return refused(PS_ERR_CUDA, ws, s);
   // With the top-k lists, as many vocabulary ranges as the workspace holds (up to 16): shorter
   // ranges keep the CTAs of a band closer together along W (16 ranges measured 4% faster than
   // the 11 the forward's chooser picks at 7B). Without them, the forward's per-tile schedule.
@@ -1317,7 +1317,7 @@ int ps_reward_uncertainty(int P, int K, int T_max, const int32_t* L, const float
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   int64_t* off = reinterpret_cast<int64_t*>(static_cast<uint8_t*>(ws) + kWsHeader);
   group_offsets_kernel<<<1, 32, 0, s>>>(P * K, L, off, static_cast<uint32_t*>(ws));
-  if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
+  if (cudaGetLastError() != cudaSuccess) return refused(PS_ERR_CUDA, ws, s);
   const size_t smem = (sizeof(int32_t) + sizeof(double)) * kUncWarps * unc_entries(K, topk);
   if (cudaFuncSetAttribute(uncertainty_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(smem)) != cudaSuccess)

@@ -8,6 +8,7 @@ namespace psk {
 
 int num_sms_current();
 int device_is_sm103();
+int refused(int rc, void* ws, cudaStream_t s);   // rc, the workspace's status zeroed: an error before a call's first kernel
 
 // Forward GEMM with the online-logsumexp epilogue. part: [splits * fwd_partials_per_split_bf16()][N]
 // (max2, sum) pairs (max in log2 units); ztok: [N] chosen-token logit, written only for rows whose token id minus

@@ -45,6 +45,12 @@ static int begin_call(void* ws, size_t ws_bytes, size_t need, cudaStream_t s) {
   return PS_OK;
 }
 
+// An error before such a first kernel was launched: the status is zeroed here instead.
+int refused(int rc, void* ws, cudaStream_t s) {
+  cudaMemsetAsync(ws, 0, kWsHeader, s);
+  return rc;
+}
+
 static uint32_t* status_word(void* ws) { return static_cast<uint32_t*>(ws); }
 // A second word of the header, zeroed with the status at the call's start: a count of finished blocks.
 static uint32_t* ticket_word(void* ws) { return static_cast<uint32_t*>(ws) + 1; }
@@ -809,7 +815,7 @@ int ps_pack_prefixes(int P, int K, int T_max, int d, int dtype, const int32_t* L
   const int adv_ctas = P < kAdvWarps * sms ? (P + kAdvWarps - 1) / kAdvWarps : sms;
   pack_meta_kernel<<<1 + adv_ctas, kMetaThreads, 0, s>>>(P, K, T_max, L, n, R, adv_mode, capacity, cu_seqlens, pw,
                                                          status_word(ws));
-  if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
+  if (cudaGetLastError() != cudaSuccess) return refused(PS_ERR_CUDA, ws, s);
   const int64_t row_vec = hid_full ? static_cast<int64_t>(d) * elem_size(dtype) / 16 : 0;
   const int grid = sms * 8;
   if (launch_after(pack_rows_kernel, dim3(static_cast<unsigned>(grid)), kPackThreads, 0, s, 1, 1, true, B, K, T_max,
@@ -889,7 +895,7 @@ static int lmhead_fwd_impl(int64_t N, int d, int V, int dtype, const void* Hpk, 
     rc = fwd_gemm_f32(N, d, V, static_cast<const float*>(Hpk), static_cast<const float*>(W), tok, f.part, f.ztok,
                       status_word(ws), s);
   }
-  if (rc != PS_OK) return rc;
+  if (rc != PS_OK) return refused(rc, ws, s);
   return launch_merge([](auto cfg) { return fwd_finalize_kernel<decltype(cfg)>; }, N, splits, s, V, splits, f.part,
                       f.ztok, tok, oldlogp, adv, w, eps, loss_scale, loss, lse, logp, ratio, coef, row_loss, ticket_word(ws),
                       status_word(ws));
@@ -926,7 +932,7 @@ static int bwd_from_store_impl(int64_t N, int d, int V, int64_t tok_base, int64_
   const float* scale = reinterpret_cast<const float*>(static_cast<const uint8_t*>(store) + L.scale_off);
   rc = dz_from_store_bf16(N, V, store, L.ldz, scale, N, tok, lse, logp, coef, status_word(ws), s,
                           static_cast<int>(tok_base));
-  if (rc != PS_OK) return rc;
+  if (rc != PS_OK) return refused(rc, ws, s);
   return bwd_grads_bf16(N, d, V, Hpk, W, dH, dW, (flags & PS_DW_ACCUMULATE) ? 1 : 0, store, L.ldz, status_word(ws),
                         s, (flags & PS_DH_ACCUMULATE) ? 1 : 0, N, v_call);
 }
@@ -1022,7 +1028,7 @@ static int logit_stats_impl(int64_t N, int d, int Vs, int64_t v0, int dtype, con
     rc = fwd_gemm_f32(N, d, Vs, static_cast<const float*>(Hpk), static_cast<const float*>(W_shard), tok, f.part,
                       f.ztok, status_word(ws), s, static_cast<int>(v0));
   }
-  if (rc != PS_OK) return rc;
+  if (rc != PS_OK) return refused(rc, ws, s);
   return launch_merge([](auto cfg) { return stats_merge_kernel<decltype(cfg)>; }, N, splits, s, splits, f.part, f.ztok,
                       tok, v0, Vs, reinterpret_cast<float2*>(stats), ztok);
 }
@@ -1132,7 +1138,7 @@ static int lmhead_bwd_impl(int64_t N, int d, int V, int64_t tok_base, int64_t v_
                          dH ? dH + r0 * d : nullptr, dW, acc, static_cast<float*>(dz), ldz, status_word(ws), s,
                          static_cast<int>(tok_base), hacc, N, v_call, r0 == 0);
     }
-    if (rc != PS_OK) return rc;
+    if (rc != PS_OK) return r0 == 0 ? refused(rc, ws, s) : rc;
   }
   return PS_OK;
 }

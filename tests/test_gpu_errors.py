@@ -137,3 +137,32 @@ def test_non_finite_design_weight_sets_its_bit():
     B.ps_design_cutoffs(cfg.P, cfg.K, T, torch.from_numpy(L).cuda(), torch.from_numpy(gamma).cuda(),
                         torch.from_numpy(u).cuda(), 40.0, B.PS_DESIGN_OPTIMIZED, 0.0, q, None, ws)
     assert B.ps_workspace_status(ws)[0] == B.PS_OK
+
+
+def test_a_refused_call_leaves_a_cleared_status():
+    # The f32 head refuses more row tiles than a grid holds, after the workspace has been accepted: the status word of
+    # whatever call used the workspace before is zero then, not that call's.
+    B = _B()
+    N, d, V = 65535 * 64 + 1, 8, 8
+    H = torch.zeros(N, d, device="cuda")
+    W = torch.zeros(V, d, device="cuda")
+    tok = torch.zeros(N, dtype=torch.int32, device="cuda")
+    col = torch.zeros(N, device="cuda")
+    out = [torch.empty(N, device="cuda") for _ in range(5)]
+    loss = torch.empty(1, dtype=torch.float64, device="cuda")
+    dH = torch.empty(N, d, device="cuda")
+
+    def stale(nbytes):
+        return torch.full((nbytes,), 255, dtype=torch.uint8, device="cuda")
+    ws = stale(B.ps_lmhead_ppo_fwd_workspace_size(N, d, V, B.PS_DTYPE_F32))
+    with pytest.raises(B.PsppoError, match="supported"):
+        B.ps_lmhead_ppo_fwd(N, d, V, B.PS_DTYPE_F32, H, W, tok, col, col, col, 0.2, 1.0, loss, *out, ws)
+    assert B.ps_workspace_status(ws) == (B.PS_OK, 0)
+    ws = stale(B.ps_lmhead_ppo_bwd_workspace_size(N, d, V, B.PS_DTYPE_F32, N))
+    with pytest.raises(B.PsppoError, match="supported"):
+        B.ps_lmhead_ppo_bwd(N, d, V, B.PS_DTYPE_F32, H, W, tok, col, col, dH, None, 0, ws)
+    assert B.ps_workspace_status(ws) == (B.PS_OK, 0)
+    ws = stale(B.ps_lmhead_logit_stats_workspace_size(N, d, V, B.PS_DTYPE_F32))
+    with pytest.raises(B.PsppoError, match="supported"):
+        B.ps_lmhead_logit_stats(N, d, V, 0, B.PS_DTYPE_F32, H, W, tok, torch.empty(N, 2, device="cuda"), col, ws)
+    assert B.ps_workspace_status(ws) == (B.PS_OK, 0)
