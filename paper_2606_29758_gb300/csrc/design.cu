@@ -1349,7 +1349,7 @@ size_t ps_design_cutoffs_workspace_size(int P, int K, int T_max) {
   if (P < 1 || K < 1 || T_max < 1) return 0;
   const size_t pt = static_cast<size_t>(P) * T_max;
   return kWsHeader + al256(sizeof(double) * pt) * 2 + al256(sizeof(double) * pt * kCapLanes) * 2 +
-         al256(sizeof(int32_t) * pt * kCapLanes) + al256(sizeof(int64_t) * static_cast<size_t>(P) * K);
+         al256(sizeof(int32_t) * pt * kCapLanes);
 }
 
 int ps_design_cutoffs(int P, int K, int T_max, const int32_t* L, const float* gamma_full, const float* u,

@@ -1,8 +1,10 @@
 // f32 LM-head forward/backward on the CUDA cores.
 //
 // The tensor cores have no full-f32 mode (tf32 keeps a 10-bit mantissa), so f32
-// inputs run here with exact f32 products and f32 accumulation, every output element over
-// its k in increasing order. One tiled kernel computes C(m, n) = sum_k A(m, k) B(k, n) for
+// inputs run here with exact f32 products and f32 accumulation, every element of Z, and of a dH or dW
+// that is not split, over its k in increasing order. Split gradients (few tiles: launch_grad) add up 2, 4
+// or 8 shares of k that way and then the shares in that order; whether they are split follows from the
+// sizes of the whole call and the number of SMs. One tiled kernel computes C(m, n) = sum_k A(m, k) B(k, n) for
 // operands whose k or whose m (n) is contiguous (Z = H W^T, dH = dZ W and dW = dZ^T H) and
 // hands blocks of its tile to an epilogue: the forward's per-row (max, sum of exp) over 64
 // columns (rows reduced across the 8 lanes that share them with warp shuffles), the

@@ -335,35 +335,35 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
             }
           } else {
 #pragma unroll 1
-          for (int c = grp * CPG; c < grp * CPG + CPG; ++c) {
-            uint32_t r[32];
-            tmem_ld32(t_row + c * 32, r);
-            tmem_ld_wait();
-            if (c == grp * CPG + CPG - 1) {
-              // this half of the accumulator has been read: hand it back to the MMA warp (a wide
-              // tile returns its two halves one after the other, tempty[0] and tempty[1])
-              tc_fence_before();
-              mbar_arrive(&sm.tempty[HALVES == 2 ? h : acc]);
-            }
-            const int col0 = nb * kBN + c * 32;
-            if constexpr (Epi::kTmaStore) {
-              // the slice goes to a staging buffer, then one lane stores the warp's 32 x 32 box
-              if (col0 < Epi::cols(ep)) {
-                uint8_t* buf = sm.stage[ew];
-                if (lane == 0) bulk_wait_group_read<0>();   // the store that last used it has read it
-                __syncwarp();
-                Epi::chunk_to_smem(ep, st[h], row, col0, r, buf, lane);
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) {
-                  Epi::store(ep, &tmC, buf, col0, m_blk * Cfg::kRows + h * kBM + quad * 32);
-                  bulk_commit_group();
-                }
+            for (int c = grp * CPG; c < grp * CPG + CPG; ++c) {
+              uint32_t r[32];
+              tmem_ld32(t_row + c * 32, r);
+              tmem_ld_wait();
+              if (c == grp * CPG + CPG - 1) {
+                // this half of the accumulator has been read: hand it back to the MMA warp (a wide
+                // tile returns its two halves one after the other, tempty[0] and tempty[1])
+                tc_fence_before();
+                mbar_arrive(&sm.tempty[HALVES == 2 ? h : acc]);
               }
-            } else {
-              Epi::chunk(ep, st[h], row, col0, r);
+              const int col0 = nb * kBN + c * 32;
+              if constexpr (Epi::kTmaStore) {
+                // the slice goes to a staging buffer, then one lane stores the warp's 32 x 32 box
+                if (col0 < Epi::cols(ep)) {
+                  uint8_t* buf = sm.stage[ew];
+                  if (lane == 0) bulk_wait_group_read<0>();   // the store that last used it has read it
+                  __syncwarp();
+                  Epi::chunk_to_smem(ep, st[h], row, col0, r, buf, lane);
+                  fence_proxy_async_smem();
+                  __syncwarp();
+                  if (lane == 0) {
+                    Epi::store(ep, &tmC, buf, col0, m_blk * Cfg::kRows + h * kBM + quad * 32);
+                    bulk_commit_group();
+                  }
+                }
+              } else {
+                Epi::chunk(ep, st[h], row, col0, r);
+              }
             }
-          }
           }
         }
       }
