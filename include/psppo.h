@@ -19,7 +19,8 @@
  *  - Data that can only be checked on the device (masses that do not sum to 2^62,
  *    a length out of range, a token id outside [0, V), more rows than capacity, a
  *    barrier wait that ran out of time) set bits in a status word at the start of
- *    the call's workspace. Each call clears that word when it starts;
+ *    the call's workspace. Each call that accepts its arguments and workspace clears
+ *    that word when it starts, also if it then fails on the host;
  *    ps_workspace_status() synchronises the stream and reports it.
  *  - Row-major layouts. "bf16" is IEEE bfloat16, "f32" IEEE binary32.
  *  - No global state: calls on different streams with different workspaces may
