@@ -789,38 +789,46 @@ __device__ __noinline__ int pav_stack(const double* w, int T, double* bW, int32_
 // Timestep weights of the OPTIMIZED and HEURISTIC designs, before the floor: w_t = gamma_bar_t * u_t with
 // gamma_bar_t = (1/K) sum over the completions that reach t, and the largest of each kWeightSteps steps. A
 // division costs tens of FP64 operations, of which an SM of GB300 does two a clock, so the steps are spread over
-// the chip: 17 us for 8 prompts of 16 completions and 15350 steps.
+// the chip: 17 us for 8 prompts of 16 completions and 15350 steps. Traces of one such part are weighed by the design
+// kernel itself, a launch less (heuristic design of 20 steps: 11.6 us, 15 with the launch).
 constexpr int kWeightSteps = 512;
-__global__ void __launch_bounds__(kDesignThreads)
-    design_weights_kernel(int K, int T_max, const int32_t* __restrict__ L, const float* __restrict__ gamma,
-                          const float* __restrict__ u, DesignWs ws, uint32_t* status) {
+// A prompt's rows before its first completion (with_rows) and its horizon, the longest completion (the whole CTA).
+struct Group {
+  long long base;
+  int horizon;
+};
+__device__ __forceinline__ Group group_of(int p, int K, const int32_t* __restrict__ L, bool with_rows) {
   __shared__ long long red_l[kDesignWarps];
   __shared__ int red_i[kDesignWarps];
-  __shared__ double red_d[kDesignWarps];
-  const int p = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  long long base = 0;   // rows before the group's first completion
-  for (int k = tid; k < p * K; k += kDesignThreads) base += L[k];
-  int Tp = 0;           // the group's horizon
-  for (int j = tid; j < K; j += kDesignThreads) Tp = max(Tp, L[p * K + j]);
+  const int tid = threadIdx.x;
+  Group g{0, 0};
+  if (with_rows)
+    for (int k = tid; k < p * K; k += kDesignThreads) g.base += L[k];
+  for (int j = tid; j < K; j += kDesignThreads) g.horizon = max(g.horizon, L[p * K + j]);
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) {
-    base += __shfl_xor_sync(0xffffffffu, base, o);
-    Tp = max(Tp, __shfl_xor_sync(0xffffffffu, Tp, o));
+    g.base += __shfl_xor_sync(0xffffffffu, g.base, o);
+    g.horizon = max(g.horizon, __shfl_xor_sync(0xffffffffu, g.horizon, o));
   }
-  if (lane == 0) {
-    red_l[wid] = base;
-    red_i[wid] = Tp;
+  if ((tid & 31) == 0) {
+    red_l[tid >> 5] = g.base;
+    red_i[tid >> 5] = g.horizon;
   }
   __syncthreads();
-  base = 0;
+  g.base = 0;
   for (int i = 0; i < kDesignWarps; ++i) {
-    base += red_l[i];
-    Tp = max(Tp, red_i[i]);
+    g.base += red_l[i];
+    g.horizon = max(g.horizon, red_i[i]);
   }
-  Tp = min(max(Tp, 1), T_max);
+  return g;
+}
+// The weights of the steps [t0, t1) into w; returns the largest of this thread's.
+__device__ __forceinline__ double design_weights(int p, int K, int T_max, const int32_t* __restrict__ L,
+                                                 const float* __restrict__ gamma, const float* __restrict__ u,
+                                                 long long base, int t0, int t1, double* __restrict__ w,
+                                                 uint32_t* status) {
   double wmax = 0.0;
-  const int t1 = min(Tp, static_cast<int>(blockIdx.y + 1) * kWeightSteps);
-  for (int t = blockIdx.y * kWeightSteps + tid; t < t1; t += kDesignThreads) {
+  for (int t = t0 + static_cast<int>(threadIdx.x); t < t1; t += kDesignThreads) {
     double acc = 0.0;
     long long off = base;
     for (int j = 0; j < K; ++j) {
@@ -831,12 +839,24 @@ __global__ void __launch_bounds__(kDesignThreads)
     double v = __ddiv_rn(acc, static_cast<double>(K));
     if (u) v = __dmul_rn(v, static_cast<double>(u[static_cast<int64_t>(p) * T_max + t]));
     if (!isfinite(v)) raise_status(status, PS_DEV_NONFINITE);
-    ws.w[static_cast<int64_t>(p) * T_max + t] = v;
+    w[t] = v;
     wmax = fmax(wmax, v);
   }
+  return wmax;
+}
+__global__ void __launch_bounds__(kDesignThreads)
+    design_weights_kernel(int K, int T_max, const int32_t* __restrict__ L, const float* __restrict__ gamma,
+                          const float* __restrict__ u, DesignWs ws, uint32_t* status) {
+  __shared__ double red_d[kDesignWarps];
+  const int p = blockIdx.x, tid = threadIdx.x;
+  const Group g = group_of(p, K, L, true);
+  const int Tp = min(max(g.horizon, 1), T_max);
+  double wmax = design_weights(p, K, T_max, L, gamma, u, g.base, blockIdx.y * kWeightSteps,
+                               min(Tp, static_cast<int>(blockIdx.y + 1) * kWeightSteps),
+                               ws.w + static_cast<int64_t>(p) * T_max, status);
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) wmax = fmax(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
-  if (lane == 0) red_d[wid] = wmax;
+  if ((tid & 31) == 0) red_d[tid >> 5] = wmax;
   __syncthreads();
   if (tid == 0) {
     for (int i = 1; i < kDesignWarps; ++i) wmax = fmax(wmax, red_d[i]);
@@ -844,14 +864,15 @@ __global__ void __launch_bounds__(kDesignThreads)
   }
 }
 
-// One CTA per prompt (and, OPTIMIZED, 172 KB of shared memory each): registers are not what limits residency.
+// One CTA per prompt (and, OPTIMIZED, 172 KB of shared memory each): registers are not what limits residency. gamma, u:
+// the weights are taken here; nullptr: design_weights_kernel has taken them, or the strategy has none.
 template <bool OPTIMIZED>
 __global__ void __launch_bounds__(kDesignThreads, 1)
-    design_kernel(int K, int T_max, const int32_t* __restrict__ L, double budget, int strategy, double param,
-                  uint64_t* __restrict__ q, double* __restrict__ xi_out, DesignWs ws, uint32_t* status) {
+    design_kernel(int K, int T_max, const int32_t* __restrict__ L, const float* __restrict__ gamma,
+                  const float* __restrict__ u, double budget, int strategy, double param, uint64_t* __restrict__ q,
+                  double* __restrict__ xi_out, DesignWs ws, uint32_t* status) {
   const int p = blockIdx.x;
   const int tid = threadIdx.x;
-  __shared__ int Tp_s;
   __shared__ double red_d[kDesignThreads / 32];
   __shared__ unsigned long long red_u[kDesignThreads / 32];
   __shared__ unsigned long long red_b[kDesignThreads / 32];
@@ -865,26 +886,17 @@ __global__ void __launch_bounds__(kDesignThreads, 1)
   double* w = ws.w + static_cast<int64_t>(p) * T_max;
   double* xi = ws.xi + static_cast<int64_t>(p) * T_max;
 
-  // horizon of the group
-  int Tmax = 0;
-  for (int j = tid; j < K; j += kDesignThreads) Tmax = max(Tmax, L[p * K + j]);
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) Tmax = max(Tmax, __shfl_xor_sync(0xffffffffu, Tmax, o));
-  if (lane == 0) red_i[wid] = Tmax;
-  __syncthreads();
-  if (tid == 0) {
-    for (int i = 1; i < kDesignWarps; ++i) Tmax = max(Tmax, red_i[i]);
-    if (Tmax < 1 || Tmax > T_max) raise_status(status, PS_DEV_BAD_LENGTH);
-    Tp_s = Tmax < 1 ? 1 : (Tmax > T_max ? T_max : Tmax);
-  }
-  __syncthreads();
-  const int Tp = Tp_s;
+  const Group group = group_of(p, K, L, gamma != nullptr);
+  if (tid == 0 && (group.horizon < 1 || group.horizon > T_max)) raise_status(status, PS_DEV_BAD_LENGTH);
+  const int Tp = min(max(group.horizon, 1), T_max);
   const double Bp = fmin(budget, static_cast<double>(Tp));
 
   if (OPTIMIZED || strategy == PS_DESIGN_HEURISTIC) {
-    // the floor under the weights: the largest of them from the weights kernel's parts
+    // the floor under the weights: the largest of them, taken here or from the weights kernel's parts
     double wmax = 0.0;
-    {
+    if (gamma != nullptr) {
+      wmax = design_weights(p, K, T_max, L, gamma, u, group.base, 0, Tp, w, status);
+    } else {
       const double* parts = ws.bW + static_cast<int64_t>(p) * T_max * kCapLanes;
       for (int c = tid; c * kWeightSteps < Tp; c += kDesignThreads) wmax = fmax(wmax, parts[c]);
     }
@@ -1369,20 +1381,22 @@ int ps_design_cutoffs(int P, int K, int T_max, const int32_t* L, const float* ga
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (cudaMemsetAsync(ws, 0, kWsHeader, s) != cudaSuccess) return PS_ERR_CUDA;
   const DesignWs d = design_ws(ws, P, T_max);
-  if (uses_gamma) {
+  uint32_t* status = static_cast<uint32_t*>(ws);
+  const float* gamma = uses_gamma ? gamma_full : nullptr;
+  if (uses_gamma && T_max > kWeightSteps) {
     const dim3 grid(static_cast<unsigned>(P), static_cast<unsigned>((T_max + kWeightSteps - 1) / kWeightSteps));
-    design_weights_kernel<<<grid, kDesignThreads, 0, s>>>(K, T_max, L, gamma_full, u, d, static_cast<uint32_t*>(ws));
+    design_weights_kernel<<<grid, kDesignThreads, 0, s>>>(K, T_max, L, gamma, u, d, status);
     if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
+    gamma = nullptr;
   }
   if (strategy == PS_DESIGN_OPTIMIZED) {
     if (cudaFuncSetAttribute(design_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(kDesignDynSmem)) != cudaSuccess)
       return PS_ERR_CUDA;
-    design_kernel<true><<<P, kDesignThreads, kDesignDynSmem, s>>>(K, T_max, L, budget, strategy, param, q, xi, d,
-                                                                  static_cast<uint32_t*>(ws));
+    design_kernel<true><<<P, kDesignThreads, kDesignDynSmem, s>>>(K, T_max, L, gamma, u, budget, strategy, param, q, xi, d,
+                                                                  status);
   } else {
-    design_kernel<false><<<P, kDesignThreads, 0, s>>>(K, T_max, L, budget, strategy, param, q, xi, d,
-                                                      static_cast<uint32_t*>(ws));
+    design_kernel<false><<<P, kDesignThreads, 0, s>>>(K, T_max, L, gamma, u, budget, strategy, param, q, xi, d, status);
   }
   return cudaGetLastError() == cudaSuccess ? PS_OK : PS_ERR_CUDA;
 }

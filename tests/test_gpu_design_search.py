@@ -98,3 +98,56 @@ def test_long_traces(trace, T):
                                                 "optimized")
     assert np.array_equal(xi, xi_ref)
     assert np.array_equal(q, q_ref)
+
+
+@pytest.mark.parametrize("T", [1, 2, 20, 511, 512, 513, 1025])
+@pytest.mark.parametrize("strategy", ["optimized", "heuristic"])
+def test_weights_of_one_part_and_of_several(T, strategy):
+    # traces of up to 512 steps are weighed by the design kernel, longer ones by a launch of their own; several
+    # prompts of unequal completions, so that every prompt's first row counts
+    from paper_2606_29758_gb300 import PS_DESIGN_HEURISTIC, PS_DESIGN_OPTIMIZED, CutoffDesign, DesignShape
+    rng = np.random.default_rng(T)
+    P, K = 5, 3
+    L = rng.integers(1, T + 1, size=P * K).astype(np.int32)
+    L[rng.integers(P * K)] = T
+    gamma = rng.lognormal(0.0, 1.0, int(L.sum())).astype(np.float32)
+    u = rng.uniform(0.01, 0.5, (P, T)).astype(np.float32)
+    cd = CutoffDesign(DesignShape(P, K, T, 8, 32, int(L.sum()), 16))
+    cd.gamma.copy_(torch.from_numpy(gamma))
+    cd.u.copy_(torch.from_numpy(u))
+    for budget in (1.0, 0.4 * T + 0.7):
+        cd.design(torch.from_numpy(L).cuda(), budget,
+                  PS_DESIGN_OPTIMIZED if strategy == "optimized" else PS_DESIGN_HEURISTIC)
+        cd.check_status()
+        q_ref, xi_ref = design.design_cutoff_masses(L, K, gamma, u, budget, strategy)
+        assert np.array_equal(cd.xi.cpu().numpy().reshape(P, T), xi_ref)
+        assert np.array_equal(cd.q.cpu().numpy().view(np.uint64).reshape(P, T), q_ref)
+
+
+def test_a_short_trace_is_weighed_without_a_launch_of_its_own():
+    # graph replays, so that the host's calls do not count
+    from paper_2606_29758_gb300 import PS_DESIGN_HEURISTIC, PS_DESIGN_UNIFORM, CutoffDesign, DesignShape
+    P, K, T = 5, 3, 20
+    cd = CutoffDesign(DesignShape(P, K, T, 8, 32, P * K * T, 0))
+    cd.gamma.uniform_(0.5, 1.5)
+    cd.u.fill_(0.1)
+    L = torch.full((P * K,), T, dtype=torch.int32, device="cuda")
+
+    def us(strategy, calls=100):
+        cd.design(L, 8.0, strategy)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            for _ in range(calls):
+                cd.design(L, 8.0, strategy)
+        best = 1e9
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            g.replay()
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) / calls * 1e3)
+        return best
+    heuristic, uniform = us(PS_DESIGN_HEURISTIC), us(PS_DESIGN_UNIFORM)
+    assert heuristic < 2.0 * uniform, (heuristic, uniform)
