@@ -187,6 +187,7 @@ __global__ void __launch_bounds__(kSampThreads)
     for (int j = kSampThreads - 1 - tid; j < K; j += kSampThreads) {   // from the last thread on: a short trace leaves it free
       const uint64_t x = xs[j];
       if (x < tile_from || x >= carry) continue;
+      const int k = p * K + j, Lk = L[k];
       int lo = 0, hi = kSampThreads - 1;   // the first step with x < u_s; the last one is carry
       while (lo < hi) {
         const int mid = (lo + hi) >> 1;
@@ -194,9 +195,9 @@ __global__ void __launch_bounds__(kSampThreads)
         else lo = mid + 1;
       }
       const bool valid = u_s[lo] <= kOne62;   // a bucket past 2^62 (an invalid row) decides nothing
-      const int k = p * K + j, h = base + lo + 1;
+      const int h = base + lo + 1;
       H[k] = valid ? h : 0;
-      n[k] = valid ? min(h, L[k]) : 0;
+      n[k] = valid ? min(h, Lk) : 0;
     }
   }
 }
