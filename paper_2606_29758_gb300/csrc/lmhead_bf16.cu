@@ -391,7 +391,7 @@ struct BwdDzEpi {
 // The output is all this epilogue moves: a tile of a short K loop (dW over a few hundred rows) is
 // bound by writing it. dW of 185 rows (3 k-blocks per tile) at d = 3584, V = 152064 takes 336 us, 6.5 TB/s
 // of its 2.2 GB, against 860 us with 4 warps that stored 16 bytes per row and instruction from their
-// registers; a step of 7.8k rows gained 2%.
+// registers.
 struct StoreF32Epi {
   static constexpr int kEpiWarps = 8;
   static constexpr bool kTmaStore = true, kReadAhead = true;
@@ -994,7 +994,7 @@ int bwd_grads_bf16(int64_t rc, int d, int V, const void* Hpk, const void* W, flo
     }
     // dW of 65 to 256 rows (2 to 4 k-blocks) is bound by its stores, which the narrow tile's epilogue overlaps whole
     // with the next tile (200 rows, V = 152064: d = 3584 407 us narrow / 443 wide, d = 1536 183 / 200; 571 rows
-    // 610 / 592).
+    // 610 / 592). One k-block goes by the rounds, like the long loops.
     if ((kb >= 2 && kb <= 4) || tile_halves(V, d, 17) == 1)
       rcode = launch_gemm_single<true, true, StoreF32Epi, 1>(ta, tb, tc, V, d, rc, 0, 2 * kBandGrad, ep, status, s);
     else
